@@ -41,7 +41,7 @@ METRIC = "GGArray insert Gelem/s & % HBM roofline; mem/needed; served p99 latenc
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # Kernels per phase: a write batch of 2^20 or more goes through bins (count,
 # scan, scatter into bins, apply), a smaller one is one kernel.
-LAUNCHES_PER_STEP = {"clear": 2, "insert": 4, "read": 1, "write": 4, "rw_b": 1, "rw_g": 1, "flatten": 1}
+LAUNCHES_PER_STEP = {"clear": 1, "insert": 4, "read": 1, "write": 4, "rw_b": 1, "rw_g": 1, "flatten": 1}
 BINNED_WRITE_MIN = 1 << 20
 
 
@@ -817,7 +817,7 @@ def run_batched(args, world, rank, local):
            "dtype": "u32/u64/record", "data": "synthetic",
            "config": {"workload": f"batched_{len(sizes)}_lognormal_median64K_sigma1.5_cap16M", "arrays": len(sizes),
                       "elements": total, "bytes": bytes_written, "rule": rule.to_json() if hasattr(rule, "to_json") else rule.__dict__,
-                      "step": "captured graph: clear every array + one persistent grow launch + fix-up + finalize"},
+                      "step": "captured graph: clear every array + one persistent grow launch + finalize"},
            "roofline": {"bound": "hbm", "achieved": round(gbs, 1), "peak": peak, "unit": "GB/s",
                         "frac": round(gbs / peak, 3), "traffic": None, "kernel": "batch_grow_kernel",
                         "algorithmic_bytes_per_launch": bytes_written},
@@ -825,7 +825,7 @@ def run_batched(args, world, rank, local):
            "plain_one_launch_per_array": {"ms": round(plain_ms, 3),
                                           "gelem_s": round(total / (plain_ms / 1e3) / 1e9, 3),
                                           "speedup_of_batched": round(plain_ms / ms, 2)},
-           "gpu_launches": K * 5, "clocks": clocks}
+           "gpu_launches": K * 4, "clocks": clocks}
     batching.teardown(pool, arrays, batch)
     return res
 

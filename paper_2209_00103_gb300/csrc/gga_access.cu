@@ -706,29 +706,28 @@ __global__ void __launch_bounds__(kFlThreads) flatten_kernel(ArrayView v, uint8_
 // ---------------------------------------------------------------------------
 // Clear, capacities, accounting.
 
-// Every bucket (live or spare) goes back to the queue of its index.
+// Every bucket (live or spare) goes back to the queue of its index, and the
+// sizes and their prefix sums become zero.  Thread (l, b) takes bucket b of
+// LFVector l; l runs to L inclusive, the prefix sums' last entry.
 __global__ void clear_kernel(ArrayView v) {
   const uint64_t gt = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const uint64_t l = gt / kMaxBuckets;
   const uint32_t b = static_cast<uint32_t>(gt % kMaxBuckets);
-  if (l >= v.L) return;
+  if (l > v.L) return;
+  if (b == 0) {
+    v.offsets[l] = 0;
+    v.fl_prefix[l] = 0;
+  }
+  if (l == v.L) return;
+  if (b == 0) {
+    v.nbuckets[l] = 0;
+    v.sizes[l] = 0;
+  }
   uint64_t* slot = v.buckets + l * kMaxBuckets + b;
   const uint64_t a = *slot;
   if (a) {
     if (!ring_push(v.pool, class_of(bucket_len(b, v.log2B) * v.E), a)) latch_error(v.status, GGA_ERR_INVALID);
     *slot = 0;
-  }
-}
-
-__global__ void clear_sizes_kernel(ArrayView v) {
-  const uint64_t l = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (l < v.L) {
-    v.nbuckets[l] = 0;
-    v.sizes[l] = 0;
-  }
-  if (l <= v.L) {
-    v.offsets[l] = 0;
-    v.fl_prefix[l] = 0;
   }
 }
 
@@ -877,9 +876,8 @@ int launch_flatten(const ArrayView& v, void* dst, uint64_t cap_elems, int num_sm
 }
 
 int launch_clear(const ArrayView& v, cudaStream_t st) {
-  const uint64_t n = static_cast<uint64_t>(v.L) * kMaxBuckets;
+  const uint64_t n = (static_cast<uint64_t>(v.L) + 1) * kMaxBuckets;
   clear_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(v);
-  clear_sizes_kernel<<<static_cast<unsigned>((v.L + 1 + 255) / 256), 256, 0, st>>>(v);
   return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 

@@ -134,17 +134,19 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchMinBlocks) batch_grow_ker
   }
 }
 
-// Fold the pops of the grow kernel into every pool's queue heads; reset
-// the ticket for the next run.
-__global__ void batch_fixup_kernel(PoolState* const* pools, uint32_t n_pools, uint32_t* ticket) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_pools) ring_fixup(pools[i]);
-  if (i == 0) *ticket = 0;
-}
-
-__global__ void __launch_bounds__(256) batch_finalize_kernel(const BatchJob* __restrict__ jobs) {
-  __shared__ uint64_t s_warp[33];
-  finalize_block(jobs[blockIdx.x].v, nullptr, nullptr, nullptr, 1, s_warp);
+// The prefix sums of every job's array, one block each.  After a growth
+// (pools given) the blocks also fold the grow kernel's pops into the pools'
+// queue heads -- a batch has no more pools than jobs -- and reset the ticket
+// for the next run.
+__global__ void __launch_bounds__(256) batch_finalize_kernel(const BatchJob* __restrict__ jobs,
+                                                             PoolState* const* pools, uint32_t n_pools,
+                                                             uint32_t* ticket) {
+  __shared__ FinalizeShared sh;
+  if (pools) {
+    if (blockIdx.x < n_pools) ring_fixup_class(pools[blockIdx.x], threadIdx.x);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
+  }
+  finalize_block(jobs[blockIdx.x].v, nullptr, nullptr, nullptr, 1, sh);
 }
 
 // Every bucket of every item back to its pool's queue; sizes to zero.
@@ -184,18 +186,16 @@ struct gga_batch_t {
 namespace {
 
 int batch_grow(gga_batch_t* b, cudaStream_t st) {
-  if (b->n_items) {
+  if (b->n_items)
     gga::batch_grow_kernel<<<b->grid, gga::kBatchThreads, gga::kBatchStageBytes, st>>>(b->jobs, b->items,
                                                                                          b->n_items, b->ticket);
-    gga::batch_fixup_kernel<<<(b->n_pools + 63) / 64 + 1, 64, 0, st>>>(b->pools, b->n_pools, b->ticket);
-  }
-  if (b->n_jobs) gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs);
+  if (b->n_jobs) gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs, b->pools, b->n_pools, b->ticket);
   return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 
 int batch_clear(gga_batch_t* b, cudaStream_t st) {
   if (b->n_items) gga::batch_clear_kernel<<<b->n_items, 64, 0, st>>>(b->jobs, b->items);
-  if (b->n_jobs) gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs);
+  if (b->n_jobs) gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs, nullptr, 0, nullptr);
   return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 

@@ -53,28 +53,38 @@ __device__ __forceinline__ bool ring_push(PoolState* p, uint32_t c, uint64_t add
   return true;
 }
 
-// After an insertion kernel: fold its pops into the queue heads (one thread).
-__device__ __forceinline__ void ring_fixup(PoolState* p) {
-  for (int c = 0; c < kPoolClasses; ++c) {
-    if (p->ring_cap[c] == 0) continue;
-    const unsigned long long h = p->ring_head[c] + p->ring_taken[c];
-    p->ring_head[c] = h < p->ring_tail[c] ? h : p->ring_tail[c];
-    p->ring_taken[c] = 0;
-  }
+// After an insertion kernel: fold its pops into the queue heads.  Called
+// by the first kPoolClasses threads of a block (t < kPoolClasses), one class
+// each, so the step is one round trip to memory: by one thread over all
+// classes it was 7 of finalize_kernel's 12 us on GB300.
+__device__ __forceinline__ void ring_fixup_class(PoolState* p, uint32_t t) {
+  if (t >= static_cast<uint32_t>(kPoolClasses)) return;
+  const unsigned long long cap = p->ring_cap[t], head = p->ring_head[t], tail = p->ring_tail[t];
+  const unsigned long long taken = p->ring_taken[t];
+  if (cap == 0 || taken == 0) return;
+  p->ring_head[t] = head + taken < tail ? head + taken : tail;
+  p->ring_taken[t] = 0;
 }
 
 // Chunks of kChunkBytes covering the live part of LFVector of `size`
-// elements, bucket by bucket (flatten / rw_b work units).
+// elements, bucket by bucket (flatten / rw_b work units).  Full bucket b
+// has 2^(e + b) bytes, e = log2(B * E): one chunk while that is at most a
+// chunk, 2^(e + b - 14) chunks from there on, so the full buckets before
+// the last one sum in closed form.
+__host__ __device__ __forceinline__ uint64_t full_bucket_chunks(uint32_t nfull, uint32_t e) {
+  constexpr uint32_t kLog2Chunk = 14;
+  const uint32_t c0 = e >= kLog2Chunk ? 0 : kLog2Chunk - e;   // first bucket of at least a whole chunk
+  if (nfull <= c0) return nfull;
+  return c0 + (((1ull << (nfull - c0)) - 1ull) << (e >= kLog2Chunk ? e - kLog2Chunk : 0));
+}
+
 __device__ __forceinline__ uint64_t bucket_chunks(uint64_t size, uint32_t log2B, uint32_t E) {
-  uint64_t n = 0;
-  for (uint32_t b = 0; b < static_cast<uint32_t>(kMaxBuckets); ++b) {
-    const uint64_t first = bucket_first(b, log2B);
-    if (first >= size) break;
-    uint64_t len = bucket_len(b, log2B);
-    if (size - first < len) len = size - first;
-    n += (len * E + kChunkBytes - 1) / kChunkBytes;
-  }
-  return n;
+  static_assert(kChunkBytes == 1u << 14, "full_bucket_chunks holds log2 of the chunk");
+  uint32_t nfull;     // the bucket of position `size`: every bucket before it is full
+  uint64_t part;      // and what lies in it
+  bucket_of(size, log2B, nfull, part);
+  return full_bucket_chunks(nfull, log2B + (31u - static_cast<uint32_t>(__clz(static_cast<int>(E))))) +
+         (part * E + kChunkBytes - 1) / kChunkBytes;
 }
 
 // ---------------------------------------------------------------------------

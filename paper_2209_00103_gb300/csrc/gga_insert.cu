@@ -38,13 +38,13 @@ constexpr int kCopyU = kCopyChunkBytes / 16 / 32;             // 16-byte groups 
 constexpr int kCountThreads = 256;
 
 // ---------------------------------------------------------------------------
-// Finalize: prefix sum of sizes, flatten/rw_b chunk prefix, copy chunk prefix.
-// Run by one block (any multiple of 32 threads, <= 1024).
+// Finalize, after a kernel that pushed: the pool's queue heads and the
+// prefix sums over the LFVector sizes.
 
 __global__ void __launch_bounds__(1024) finalize_kernel(ArrayView v) {
-  __shared__ uint64_t s_warp[33];
-  if (threadIdx.x == 0) ring_fixup(v.pool);
-  finalize_block(v, nullptr, nullptr, nullptr, 1, s_warp);
+  __shared__ FinalizeShared sh;
+  ring_fixup_class(v.pool, threadIdx.x);
+  finalize_block(v, nullptr, nullptr, nullptr, 1, sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(uint64_t* tile, uint64_
 
 __global__ void __launch_bounds__(256) reserve_kernel(ArrayView v, InsertScratch s, uint32_t R, uint64_t n_values,
                                                       uint64_t n_tiles, uint32_t copy_chunk_elems) {
-  __shared__ uint64_t s_warp[33];
+  __shared__ FinalizeShared s_fin;
   __shared__ int s_last;
   const uint64_t gt = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const bool ok = s.tile_pre[n_tiles] == n_values;
@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(256) reserve_kernel(ArrayView v, InsertScratch
       }
 #pragma unroll
       for (int k = 0; k < kResK; ++k) {
+        if (r0 + k * 32 >= R) break;   // warp-uniform
         const uint32_t r = r0 + k * 32 + lane;
         const uint64_t inc = warp_incl_scan(t[k]);
         if (r < R) pre_l[r] = S + inc - t[k];
@@ -251,8 +252,8 @@ __global__ void __launch_bounds__(256) reserve_kernel(ArrayView v, InsertScratch
   __syncthreads();
   if (s_last) {
     __threadfence();
-    if (threadIdx.x == 0) ring_fixup(v.pool);
-    finalize_block(v, s.ins_base, s.ins_len, s.cp_prefix, copy_chunk_elems, s_warp);
+    ring_fixup_class(v.pool, threadIdx.x);
+    finalize_block(v, s.ins_base, s.ins_len, s.cp_prefix, copy_chunk_elems, s_fin);
     if (threadIdx.x == 0) s.counters[1] = 0;
   }
 }

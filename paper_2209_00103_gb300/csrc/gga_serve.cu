@@ -29,6 +29,7 @@ constexpr uint64_t kAppendChunk = 16384;   // elements one block of the write ke
 struct AppendParams {
   uint32_t n_req;
   uint32_t pad;
+  PoolState* pool;                  // the pool of every request's array
   uint64_t* res_base;               // per (request, LFVector): first reserved index
   uint64_t* res_len;                // and the number of elements it got (0 if the pool was short)
   const ArrayView* view[kServeMax];
@@ -85,7 +86,7 @@ __device__ void append_run(const ArrayView& v, uint32_t l, uint64_t start, uint6
 // update, Algorithm 2 for the buckets it reaches) by its own thread, then
 // the block recomputes the array's offsets from the new sizes.
 __global__ void __launch_bounds__(kServeThreads) append_reserve_kernel(const __grid_constant__ AppendParams P) {
-  __shared__ uint64_t s_warp[33];
+  __shared__ FinalizeShared sh;
   const uint32_t r = blockIdx.x;
   const ArrayView& v = *P.view[r];
   for (uint32_t l = threadIdx.x; l < v.L; l += blockDim.x) {
@@ -109,11 +110,14 @@ __global__ void __launch_bounds__(kServeThreads) append_reserve_kernel(const __g
     P.res_len[P.slot0[r] + l] = len;
   }
   __syncthreads();
-  finalize_block(v, nullptr, nullptr, nullptr, 1, s_warp);
+  finalize_block(v, nullptr, nullptr, nullptr, 1, sh);
 }
 
-// Write blocks: kAppendChunk elements of one (request, LFVector) each.
+// Write blocks: kAppendChunk elements of one (request, LFVector) each.  The
+// first one also folds the reservations' pops into the pool's queue heads
+// (nothing here touches the pool).
 __global__ void __launch_bounds__(kServeThreads) append_write_kernel(const __grid_constant__ AppendParams P) {
+  if (blockIdx.x == 0) ring_fixup_class(P.pool, threadIdx.x);
   uint32_t lo = 0, hi = P.n_req;
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;
@@ -135,8 +139,6 @@ __global__ void __launch_bounds__(kServeThreads) append_write_kernel(const __gri
     default: append_run<16>(v, l, base + k0, cnt, vfirst); break;
   }
 }
-
-__global__ void serve_fixup_kernel(PoolState* pool) { ring_fixup(pool); }
 
 template <int E>
 __device__ void read_run(const ArrayView& v, uint64_t n, uint64_t seed, void* out) {
@@ -198,6 +200,7 @@ int gga_append_batch(const gga_append_req* reqs, uint32_t n, void* stream) {
   while (i0 < n) {
     gga::AppendParams P;
     P.pad = 0;
+    P.pool = pool;
     P.res_base = res;
     P.res_len = res + gga::kServeSlots;
     uint32_t m = 0, slots = 0, chunks = 0;
@@ -222,7 +225,6 @@ int gga_append_batch(const gga_append_req* reqs, uint32_t n, void* stream) {
     P.slot0[m] = slots;
     P.chunk0[m] = chunks;
     gga::append_reserve_kernel<<<m, gga::kServeThreads, 0, st>>>(P);
-    gga::serve_fixup_kernel<<<1, 1, 0, st>>>(pool);
     gga::append_write_kernel<<<chunks, gga::kServeThreads, 0, st>>>(P);
     i0 += m;
   }
