@@ -244,11 +244,12 @@ int gga_insert_generated(gga_handle h, const gga_gen_spec* spec, uint32_t rounds
  *  in the handle's status word and returned by gga_last_error / gga_size.
  *
  * gga_push_generated -- gga_insert_generated written as a user kernel of
- *  the device API: one block of T threads per LFVector, one push per round
- *  through a gga::BlockPusher, then gga_device_commit.  Same draws, same
- *  result, same errors as gga_insert_generated; it is the per-round form of
- *  Algorithm 1, which gga_insert_generated batches over rounds.  Each push
- *  is assembled in shared memory and written with 128-bit stores.
+ *  the device API: one block per LFVector, each thread playing four of its T
+ *  threads, one push per round through a gga::BlockPusher, then
+ *  gga_device_commit.  Same draws, same result, same errors as
+ *  gga_insert_generated; it is the per-round form of Algorithm 1, which
+ *  gga_insert_generated batches over rounds.  Each push is assembled in
+ *  shared memory and written with 128-bit stores.
  *
  * gga_push_expand -- pushes of values read from device memory, written as a
  *  user kernel of the device API (one block per LFVector of T <= 512 slots,

@@ -213,6 +213,8 @@ template <class T>
 struct BlockPusher {
   const ArrayView* view;
   PushShared* sh;
+  uint64_t* tab;         // LFVector l's bucket table
+  uint64_t* size_at;     // and its size in the array
   uint4* stage;          // shared memory for staged writes (two halves), or nullptr
   uint32_t half_elems;   // capacity of one half in elements (a multiple of 16 bytes)
   uint64_t size, cap;
@@ -220,6 +222,7 @@ struct BlockPusher {
   uint32_t pend_n;       //   its length (0: none)
   uint32_t pend_half;    //   and its half of the stage
   uint32_t l, nb, par;
+  uint32_t log2B;
   bool valid;
 
   // stage / stage_bytes (optional): a 16-byte aligned shared-memory buffer
@@ -231,18 +234,21 @@ struct BlockPusher {
   // or for a larger push, every thread stores its own elements.
   __device__ BlockPusher(const ArrayView* v, uint32_t lfv, PushShared& s, void* stage_smem = nullptr,
                          uint32_t stage_bytes = 0)
-      : view(v), sh(&s), stage(static_cast<uint4*>(stage_smem)),
+      : view(v), sh(&s), tab(nullptr), size_at(nullptr), stage(static_cast<uint4*>(stage_smem)),
         half_elems(stage_smem ? (stage_bytes / 32u) * 16u / static_cast<uint32_t>(sizeof(T)) : 0u),
-        size(0), cap(0), pend_base(0), pend_n(0), pend_half(0), l(lfv), nb(0), par(0) {
+        size(0), cap(0), pend_base(0), pend_n(0), pend_half(0), l(lfv), nb(0), par(0), log2B(v->log2B) {
     __syncthreads();   // this block's earlier writes to the LFVector are visible
     valid = lfv < v->L && sizeof(T) == v->E;
+    if (v->B < 16 / sizeof(T)) half_elems = 0;   // a 16-byte group could straddle buckets: not staged
     if (!valid) {
       if (block_rank() == 0) latch_error(v->status, GGA_ERR_INVALID);
       return;
     }
-    size = v->sizes[lfv];
+    tab = v->buckets + static_cast<uint64_t>(lfv) * kMaxBuckets;
+    size_at = v->sizes + lfv;
+    size = *size_at;
     nb = v->nbuckets[lfv];
-    cap = prefix_capacity(nb, v->log2B);
+    cap = prefix_capacity(nb, log2B);
   }
 
   // Append count elements value_of_k(0..count-1) of this thread after those
@@ -250,8 +256,19 @@ struct BlockPusher {
   // (in every thread) when the block's elements were appended.
   template <class F>
   __device__ bool push(uint32_t count, F value_of_k, uint64_t* first = nullptr) {
+    return push_run(count, [&](auto put) {
+      for (uint32_t k = 0; k < count; ++k) put(k, value_of_k(k));
+    }, first);
+  }
+
+  // push with the thread's elements in any order: write(put) is called once
+  // and calls put(k, element k) for every k < count.  A thread that stands
+  // for several consecutive threads of the LFVector (its elements are the
+  // first one's, then the next one's) then writes each one's elements at
+  // their known places, without a search per element.
+  template <class W>
+  __device__ bool push_run(uint32_t count, W write, uint64_t* first = nullptr) {
     if (!valid) return false;
-    const ArrayView& v = *view;
     const uint32_t nt = block_threads(), t = block_rank();
     const uint32_t lane = t & 31, w = t >> 5, nw = (nt + 31) >> 5;
     const uint32_t in_warp = nt - (w << 5) < 32 ? nt - (w << 5) : 32;
@@ -281,9 +298,17 @@ struct BlockPusher {
     __syncthreads();
     write_pending();   // the previous push's stage is complete (barrier above)
 
-    // 2. Every warp: the block total and its own offset from the warp totals.
+    // 2. Every warp: the block total and its own offset from the warp
+    //    totals: summed as they are for up to four warps, by a warp scan for
+    //    more.
     uint64_t total = 0, woff = 0;
-    if (in_warp == 32) {
+    if (nw <= 4 || in_warp < 32) {
+      for (uint32_t i = 0; i < nw; ++i) {
+        const uint64_t y = sh->warp[pb][i];
+        total += y;
+        if (i < w) woff += y;
+      }
+    } else {
       const uint64_t y = lane < nw ? sh->warp[pb][lane] : 0;
       if (__all_sync(0xffffffffu, y < (1ull << 26))) {   // 32 of them cannot wrap 32 bits
         const uint32_t y32 = static_cast<uint32_t>(y);
@@ -305,12 +330,6 @@ struct BlockPusher {
         total = __shfl_sync(0xffffffffu, yi, 31);
         woff = __shfl_sync(0xffffffffu, yi - y, w);
       }
-    } else {
-      for (uint32_t i = 0; i < nw; ++i) {
-        const uint64_t y = sh->warp[pb][i];
-        total += y;
-        if (i < w) woff += y;
-      }
     }
 
     // 3. Reservation.  All threads hold the same size and capacity, so they
@@ -320,10 +339,11 @@ struct BlockPusher {
     bool ok = true;
     if (end <= cap && end >= base) {
       size = end;
-      if (t == 0 && total > 0) v.sizes[l] = end;
+      if (t == 0 && total > 0) *size_at = end;
     } else {
       if (w == 0) {
-        const uint32_t need = end < base ? kMaxBuckets + 1u : buckets_for(end, v.log2B);
+        const ArrayView& v = *view;
+        const uint32_t need = end < base ? kMaxBuckets + 1u : buckets_for(end, log2B);
         uint32_t got;
         if (mask == 0xffffffffu && (blockDim.x & 31) == 0) {
           got = grow_buckets_warp(v, l, nb, need);
@@ -335,7 +355,7 @@ struct BlockPusher {
         if (lane == 0) {
           const bool fits = got >= need;
           v.nbuckets[l] = got;
-          if (fits) v.sizes[l] = end;
+          if (fits) *size_at = end;
           else latch_error(v.status, GGA_ERR_POOL_EXHAUSTED);
           sh->nb[pb] = got;
           sh->ok[pb] = fits ? 1u : 0u;
@@ -343,7 +363,7 @@ struct BlockPusher {
       }
       __syncthreads();   // the buckets exist before any write
       nb = sh->nb[pb];
-      cap = prefix_capacity(nb, v.log2B);
+      cap = prefix_capacity(nb, log2B);
       ok = sh->ok[pb] != 0;
       if (ok) size = end;
     }
@@ -358,31 +378,33 @@ struct BlockPusher {
     if (!ok) return false;
     constexpr uint32_t VEC = 16 / sizeof(T);
     const uint32_t shv = static_cast<uint32_t>(base & (VEC - 1));
-    if (stage && total > 0 && total + shv <= half_elems && v.B >= VEC) {   // block-uniform
-      T* st = reinterpret_cast<T*>(stage) + static_cast<uint64_t>(pb) * half_elems;
-      const uint32_t q0 = static_cast<uint32_t>(j0 - base) + shv;
-      for (uint32_t k = 0; k < count; ++k) st[q0 + k] = static_cast<T>(value_of_k(k));
+    if (total > 0 && total + shv <= half_elems) {   // block-uniform
+      T* st = reinterpret_cast<T*>(stage) + static_cast<uint64_t>(pb) * half_elems +
+              (static_cast<uint32_t>(j0 - base) + shv);
+      write([&](uint32_t k, T e) { st[k] = e; });
       pend_base = base;
       pend_n = static_cast<uint32_t>(total);
       pend_half = pb;
       return true;
     }
     if (count > 0) {
-      const uint64_t* tab = v.buckets + static_cast<uint64_t>(l) * kMaxBuckets;
+      // The bucket of the run's first element; elements past its end look
+      // theirs up.
       uint32_t b;
       uint64_t off;
-      bucket_of(j0, v.log2B, b, off);
+      bucket_of(j0, log2B, b, off);
       T* p = reinterpret_cast<T*>(tab[b]) + off;
-      uint64_t left = bucket_len(b, v.log2B) - off;
-      for (uint32_t k = 0; k < count; ++k) {
-        if (left == 0) {
-          ++b;
-          p = reinterpret_cast<T*>(tab[b]);
-          left = bucket_len(b, v.log2B);
+      const uint64_t left = bucket_len(b, log2B) - off;
+      write([&](uint32_t k, T e) {
+        if (k < left) {
+          p[k] = e;
+        } else {
+          uint32_t bk;
+          uint64_t ok_;
+          bucket_of(j0 + k, log2B, bk, ok_);
+          reinterpret_cast<T*>(tab[bk])[ok_] = e;
         }
-        *p++ = static_cast<T>(value_of_k(k));
-        --left;
-      }
+      });
     }
     return true;
   }
@@ -399,10 +421,9 @@ struct BlockPusher {
   // barrier that follows its stage writes).
   __device__ void write_pending() {
     if (pend_n == 0) return;
-    const ArrayView& v = *view;
     constexpr uint32_t VEC = 16 / sizeof(T);
     const uint32_t shv = static_cast<uint32_t>(pend_base & (VEC - 1));
-    stage_to_buckets<T>(v.buckets + static_cast<uint64_t>(l) * kMaxBuckets, v.log2B, v.B, pend_base, pend_n, shv,
+    stage_to_buckets<T>(tab, log2B, 1ull << log2B, pend_base, pend_n, shv,
                         stage + static_cast<uint64_t>(pend_half) * (half_elems * sizeof(T) / 16u),
                         block_rank(), block_threads());
     pend_n = 0;

@@ -285,6 +285,42 @@ __host__ __device__ constexpr uint32_t max_count() {
   return DIST == GGA_DIST_BERNOULLI ? 1u : (DIST == GGA_DIST_UNIFORM3 ? 2u : 0u);
 }
 
+// Threshold counts (ascending thresholds) per interval of 2^24 draws, in
+// shared memory: ptab[i] holds c_i = #{k : thr[k] <= i * 2^24} in its top 7
+// bits and, in its low 25, the offset of the next threshold thr[c_i] from
+// i * 2^24 when that threshold lies inside the interval, else 2^24 (no draw
+// of the interval reaches it).  A draw u of interval i counts c_i when its
+// low 24 bits stay below that offset -- one table load -- and otherwise
+// steps over the thresholds from c_i + 1.
+struct ThresholdTable {
+  uint32_t thr[GGA_MAX_THRESHOLDS];
+  uint32_t ptab[256];
+
+  // Fill from ascending g.thr[0 .. nthr) (every thread of the block; a
+  // barrier must follow).
+  __device__ __forceinline__ void fill(const GenParams& g, uint32_t t, uint32_t nt) {
+    for (uint32_t i = t; i < GGA_MAX_THRESHOLDS; i += nt) thr[i] = g.thr[i];
+    for (uint32_t i = t; i < 256; i += nt) {
+      uint32_t c = 0;
+      for (uint32_t k = 0; k < g.nthr; ++k) c += g.thr[k] <= (i << 24) ? 1u : 0u;
+      const uint64_t lo = static_cast<uint64_t>(i) << 24;
+      const uint32_t rel = c < g.nthr && g.thr[c] < lo + (1u << 24) ? static_cast<uint32_t>(g.thr[c] - lo) : (1u << 24);
+      ptab[i] = (c << 25) | rel;
+    }
+  }
+
+  // #{k < nthr : u >= thr[k]} for the high word u of a draw.
+  __device__ __forceinline__ uint32_t count(uint32_t nthr, uint32_t u) const {
+    const uint32_t e = ptab[u >> 24];
+    uint32_t c = e >> 25;
+    if ((u & 0xFFFFFFu) >= (e & 0x1FFFFFFu)) {
+      ++c;
+      while (c < nthr && u >= thr[c]) ++c;
+    }
+    return c;
+  }
+};
+
 struct GenShared {
   uint32_t wt[4][32];         // packed warp prefixes (K / 2 <= 4 words)
   uint32_t rb[9];             // pass-relative start of every round (K <= 8)
@@ -292,29 +328,8 @@ struct GenShared {
   uint32_t commit, nb;
   int stop;                   // 1: pool exhausted, 2: target reached
   uint64_t tab[kMaxBuckets];  // the LFVector's bucket table (copy)
-  // Threshold counts (ascending thresholds) per interval of 2^24 draws:
-  // ptab[i] holds c_i = #{k : thr[k] <= i * 2^24} in its top 7 bits and, in
-  // its low 25, the offset of the next threshold thr[c_i] from i * 2^24 when
-  // that threshold lies inside the interval, else 2^24 (no draw of the
-  // interval reaches it).  A draw u of interval i counts c_i when its low 24
-  // bits stay below that offset -- one table load -- and otherwise steps
-  // over the thresholds from c_i + 1.
-  uint32_t thr[GGA_MAX_THRESHOLDS];
-  uint32_t ptab[256];
+  ThresholdTable thr;
 };
-
-// Count of draw u (the high word) against ascending thresholds through the
-// table: start from the thresholds below u's interval of 2^24, then step
-// over those inside it.  Equal to #{k < nthr : u >= thr[k]}.
-__device__ __forceinline__ uint32_t table_count(const GenShared& sh, uint32_t nthr, uint32_t u) {
-  const uint32_t e = sh.ptab[u >> 24];
-  uint32_t c = e >> 25;
-  if ((u & 0xFFFFFFu) >= (e & 0x1FFFFFFu)) {
-    ++c;
-    while (c < nthr && u >= sh.thr[c]) ++c;
-  }
-  return c;
-}
 
 // Returns the number of rounds it drew; *done is set when the LFVector
 // reached `target` or the pool ran out.  Every thread of the block calls
@@ -347,16 +362,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
     for (uint32_t i = t0; i < nb0; i += NT) sh.tab[i] = bk[i];
   }
   const bool tabled = DIST == GGA_DIST_POISSON && g.thr_sorted;   // uniform
-  if (tabled) {
-    for (uint32_t i = t0; i < GGA_MAX_THRESHOLDS; i += NT) sh.thr[i] = g.thr[i];
-    for (uint32_t i = t0; i < 256; i += NT) {
-      uint32_t c = 0;
-      for (uint32_t k = 0; k < g.nthr; ++k) c += g.thr[k] <= (i << 24) ? 1u : 0u;
-      const uint64_t lo = static_cast<uint64_t>(i) << 24;
-      const uint32_t rel = c < g.nthr && g.thr[c] < lo + (1u << 24) ? static_cast<uint32_t>(g.thr[c] - lo) : (1u << 24);
-      sh.ptab[i] = (c << 25) | rel;
-    }
-  }
+  if (tabled) sh.thr.fill(g, t0, NT);
   __syncthreads();
   uint32_t r0 = 0;
   while (r0 < R && sh.stop == 0) {
@@ -382,7 +388,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
         for (int i = 0; i < KV; ++i) {
           uint32_t ci = 0;
           if (k < kk && (KV == 1 || static_cast<uint32_t>(i) < kv) && tfirst + i < v.T) {
-            if (DIST == GGA_DIST_POISSON && tabled) ci = table_count(sh, g.nthr, splitmix_mix_hi(dv[i].state(r)));
+            if (DIST == GGA_DIST_POISSON && tabled) ci = sh.thr.count(g.nthr, splitmix_mix_hi(dv[i].state(r)));
             else ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r));
           }
           if (KV > 1 && i < KV - 1) {
