@@ -302,7 +302,14 @@ struct BlockPusher {
     //    totals: summed as they are for up to four warps, by a warp scan for
     //    more.
     uint64_t total = 0, woff = 0;
-    if (nw <= 4 || in_warp < 32) {
+    if (nw <= 4) {
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) {
+        const uint64_t y = i < nw ? sh->warp[pb][i] : 0;
+        total += y;
+        if (i < w) woff += y;
+      }
+    } else if (in_warp < 32) {
       for (uint32_t i = 0; i < nw; ++i) {
         const uint64_t y = sh->warp[pb][i];
         total += y;

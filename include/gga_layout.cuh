@@ -148,11 +148,13 @@ __device__ __forceinline__ V warp_incl_scan(V v) {
 // Every 16-byte group of positions inside the run goes out as one aligned
 // 128-bit store (a group never straddles buckets when B is a multiple of
 // 16 / sizeof(T), and buckets start on 256-byte boundaries); the partial
-// groups at the run's ends go element by element.  The buckets are those
-// of `tab` (the LFVector's bucket table), already allocated.  Each thread
-// keeps the bucket its last group fell in (first position, end, address)
-// and looks the table up again only when its positions pass that bucket's
-// end.
+// groups at the run's ends go element by element, one thread each.  The
+// buckets are those of `tab` (the LFVector's bucket table), already
+// allocated.  A run lies in one bucket or a few, so the bucket math is done
+// once per bucket by every thread and a group costs a shared-memory load, a
+// store and a few additions.  With the bucket math done per group it was a
+// fifth of the generated insertion's instructions (0.71 -> 0.55 ms on GB300
+// for 2^28 int32, together with branch-free draws).
 
 template <class T>
 __device__ __forceinline__ void stage_to_buckets(const uint64_t* tab, uint32_t log2B, uint64_t B, uint64_t base,
@@ -160,34 +162,38 @@ __device__ __forceinline__ void stage_to_buckets(const uint64_t* tab, uint32_t l
                                                  uint32_t nt) {
   constexpr uint32_t VEC = 16 / sizeof(T);
   const T* stage = reinterpret_cast<const T*>(stage4);
-  const bool group_ok = B >= VEC;
-  const uint64_t gbeg = base - shv;
-  const uint32_t nvec = (n + shv + VEC - 1) / VEC;
-  uint64_t cfirst = 0, cend = 0, caddr = 0;   // the bucket of this thread's last group
-  for (uint32_t vi = t; vi < nvec; vi += nt) {
-    const uint64_t p = gbeg + static_cast<uint64_t>(vi) * VEC;
-    const uint32_t lo = vi * VEC;   // stage index of position p
-    if (group_ok && lo >= shv && lo + VEC <= n + shv) {
-      if (p < cfirst || p >= cend) {
-        uint32_t bb;
-        uint64_t off;
-        bucket_of(p, log2B, bb, off);
-        cfirst = p - off;
-        cend = cfirst + bucket_len(bb, log2B);
-        caddr = tab[bb];
-      }
-      __stcs(reinterpret_cast<uint4*>(caddr + (p - cfirst) * sizeof(T)), stage4[vi]);
-    } else {
-#pragma unroll
-      for (uint32_t e = 0; e < VEC; ++e) {
-        const uint32_t si = lo + e;
-        if (si < shv || si >= n + shv) continue;
-        uint32_t bb;
-        uint64_t off;
-        bucket_of(p + e, log2B, bb, off);
-        *reinterpret_cast<T*>(tab[bb] + off * sizeof(T)) = stage[si];
-      }
+  const uint64_t gbeg = base - shv;      // the position of stage element 0: a multiple of VEC
+  const uint32_t end = n + shv;          // stage elements shv .. end - 1 are the run
+  auto put = [&](uint32_t si) {
+    uint32_t bb;
+    uint64_t off;
+    bucket_of(gbeg + si, log2B, bb, off);
+    *reinterpret_cast<T*>(tab[bb] + off * sizeof(T)) = stage[si];
+  };
+  if (B < VEC) {   // block-uniform: buckets smaller than a group
+    for (uint32_t si = shv + t; si < end; si += nt) put(si);
+    return;
+  }
+  const uint32_t g0 = shv ? 1u : 0u;     // whole groups: g0 .. g1 - 1
+  const uint32_t g1 = end / VEC;
+  if (VEC > 1) {
+    // Before and after the whole groups: at most VEC - 1 elements each.
+    const uint32_t head = g0 * VEC < end ? g0 * VEC : end;
+    const uint32_t tail = (g1 > g0 ? g1 : g0) * VEC;
+    for (uint32_t i = t; i < 2 * VEC; i += nt) {
+      const uint32_t si = i < VEC ? shv + i : tail + (i - VEC);
+      if (si < (i < VEC ? head : end)) put(si);
     }
+  }
+  for (uint32_t g = g0; g < g1;) {       // block-uniform: the run's part in one bucket
+    uint32_t bb;
+    uint64_t off;
+    bucket_of(gbeg + static_cast<uint64_t>(g) * VEC, log2B, bb, off);
+    const uint64_t room = (bucket_len(bb, log2B) - off) / VEC;
+    const uint32_t m = room < g1 - g ? static_cast<uint32_t>(room) : g1 - g;
+    uint4* dst = reinterpret_cast<uint4*>(tab[bb] + off * sizeof(T));
+    for (uint32_t vi = t; vi < m; vi += nt) __stcs(dst + vi, stage4[g + vi]);
+    g += m;
   }
 }
 

@@ -347,6 +347,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
   const int lane = t0 & 31, warp = t0 >> 5, nwarps = NT >> 5;
   const uint32_t kv = KV == 1 ? 1u : (v.T + NT - 1) / NT;
   const uint64_t tfirst = static_cast<uint64_t>(t0) * kv;        // first virtual thread
+  const uint32_t nvt = tfirst < v.T ? min(kv, v.T - static_cast<uint32_t>(tfirst)) : 0u;   // virtual threads played
   const uint64_t gfirst = static_cast<uint64_t>(l) * v.T + tfirst;
   const uint64_t* bk = v.buckets + static_cast<uint64_t>(l) * kMaxBuckets;
   RoundDraws dv[KV];   // virtual threads gfirst, ..., gfirst + KV - 1
@@ -386,11 +387,12 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
         uint32_t sum = 0;
 #pragma unroll
         for (int i = 0; i < KV; ++i) {
-          uint32_t ci = 0;
-          if (k < kk && (KV == 1 || static_cast<uint32_t>(i) < kv) && tfirst + i < v.T) {
-            if (DIST == GGA_DIST_POISSON && tabled) ci = sh.thr.count(g.nthr, splitmix_mix_hi(dv[i].state(r)));
-            else ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r));
-          }
+          // Drawn unconditionally and masked: a branch around every draw
+          // costs more than the draws of the threads and rounds past the end.
+          uint32_t ci;
+          if (DIST == GGA_DIST_POISSON && tabled) ci = sh.thr.count(g.nthr, splitmix_mix_hi(dv[i].state(r)));
+          else ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r));
+          if (!(k < kk && static_cast<uint32_t>(i) < nvt)) ci = 0;
           if (KV > 1 && i < KV - 1) {
             const int q = static_cast<int>(k) * (KV - 1) + i;
             cw[KV > 1 ? q / 4 : 0] |= ci << (8 * (q % 4));
@@ -468,60 +470,85 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
     // one store loop over the run of both.  (With four the switch points
     // cost registers the kernels do not have.)
     constexpr bool kMergedRun = KV == 2 && !(DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2);
+    if (whole) {
+      T* const st0 = stage + shv;
 #pragma unroll
-    for (int j = 0; j < KP; ++j) {
-      const uint32_t ex = sh.wt[j][warp] + inc[j] - pk[j];
+      for (int j = 0; j < KP; ++j) {
+        const uint32_t ex = sh.wt[j][warp] + inc[j] - pk[j];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t k = 2 * j + h;
-        uint32_t st = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
-        const uint32_t csum = (pk[j] >> (16 * h)) & 0xFFFFu;
-        if (kMergedRun && whole) {
-          // The thread's virtual threads own consecutive positions of the
-          // round, so their elements form one run of csum positions from
-          // st: one loop over the run, moving to the next virtual thread's
-          // values at its first position (an empty virtual thread's switch
-          // point equals the next one's, and the later switch wins).  One
-          // shared-memory store per warp iteration over the run, against one
-          // per iteration of each virtual thread's own loop.
-          uint32_t sw[KV > 1 ? KV - 1 : 1];
-          uint32_t acc = 0;
-#pragma unroll
-          for (int i = 0; i < KV - 1; ++i) {
-            const int q = static_cast<int>(k) * (KV - 1) + i;
-            acc += (cw[q / 4] >> (8 * (q % 4))) & 0xFFu;
-            sw[i] = acc;
-          }
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t k = 2 * j + h;
+          T* st = st0 + sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
+          const uint32_t csum = (pk[j] >> (16 * h)) & 0xFFFFu;
           const V v0 = vr + vb * static_cast<V>(k);
-          V val = v0;
-          for (uint32_t m = 0; m < csum; ++m, val += vc) {
+          if (kMergedRun) {
+            // The thread's virtual threads own consecutive positions of the
+            // round, so their elements form one run of csum positions: one
+            // loop over the run, moving to the next virtual thread's values
+            // at its first position (an empty virtual thread's switch point
+            // equals the next one's, and the later switch wins).  One
+            // shared-memory store per warp iteration over the run, against
+            // one per iteration of each virtual thread's own loop.
+            uint32_t sw[KV > 1 ? KV - 1 : 1];
+            uint32_t acc = 0;
 #pragma unroll
-            for (int i = 0; i < KV - 1; ++i)
-              if (m == sw[i]) val = v0 + va * static_cast<V>(i + 1);
-            stage[st + m + shv] = gen_value<E>(val);
+            for (int i = 0; i < KV - 1; ++i) {
+              const int q = static_cast<int>(k) * (KV - 1) + i;
+              acc += (cw[q / 4] >> (8 * (q % 4))) & 0xFFu;
+              sw[i] = acc;
+            }
+            V val = v0;
+            for (uint32_t m = 0; m < csum; ++m, val += vc) {
+#pragma unroll
+              for (int i = 0; i < KV - 1; ++i)
+                if (m == sw[i]) val = v0 + va * static_cast<V>(i + 1);
+              st[m] = gen_value<E>(val);
+            }
+            continue;
           }
-          continue;
+          uint32_t before = 0;   // elements of the earlier virtual threads of this round
+#pragma unroll
+          for (int i = 0; i < KV; ++i) {
+            uint32_t c = csum - before;
+            if (KV > 1 && i < KV - 1) {
+              const int q = static_cast<int>(k) * (KV - 1) + i;
+              c = (cw[KV > 1 ? q / 4 : 0] >> (8 * (q % 4))) & 0xFFu;
+            }
+            before += c;
+            V val = v0 + va * static_cast<V>(i);
+            if (DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2) {
+              // At most two elements: predicated stores, no loop.
+              if (c > 0) st[0] = gen_value<E>(val);
+              if (max_count<DIST>() > 1 && c > 1) st[1] = gen_value<E>(val + vc);
+            } else {
+              for (uint32_t m = 0; m < c; ++m, val += vc) st[m] = gen_value<E>(val);
+            }
+            st += c;
+          }
         }
-        uint32_t before = 0;   // elements of the earlier virtual threads of this round
+      }
+    } else {
+      // A clipped or unstaged pass: element by element.
 #pragma unroll
-        for (int i = 0; i < KV; ++i) {
-          uint32_t c = csum - before;
-          if (KV > 1 && i < KV - 1) {
-            const int q = static_cast<int>(k) * (KV - 1) + i;
-            c = (cw[KV > 1 ? q / 4 : 0] >> (8 * (q % 4))) & 0xFFu;
-          }
-          before += c;
-          V val = vr + va * static_cast<V>(i) + vb * static_cast<V>(k);
-          if (whole && DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2) {
-            // At most two elements: predicated stores, no loop.
-            if (c > 0) stage[st + shv] = gen_value<E>(val);
-            if (max_count<DIST>() > 1 && c > 1) stage[st + 1 + shv] = gen_value<E>(val + vc);
-          } else if (whole) {
-            for (uint32_t m = 0; m < c; ++m, val += vc) stage[st + m + shv] = gen_value<E>(val);
-          } else {
-            for (uint32_t m = 0; m < c; ++m, val += vc) {
-              const uint32_t q = st + m;
-              if (q >= commit) break;
+      for (int j = 0; j < KP; ++j) {
+        const uint32_t ex = sh.wt[j][warp] + inc[j] - pk[j];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t k = 2 * j + h;
+          uint32_t q = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
+          const uint32_t csum = (pk[j] >> (16 * h)) & 0xFFFFu;
+          uint32_t before = 0;
+#pragma unroll
+          for (int i = 0; i < KV; ++i) {
+            uint32_t c = csum - before;
+            if (KV > 1 && i < KV - 1) {
+              const int qq = static_cast<int>(k) * (KV - 1) + i;
+              c = (cw[KV > 1 ? qq / 4 : 0] >> (8 * (qq % 4))) & 0xFFu;
+            }
+            before += c;
+            V val = vr + va * static_cast<V>(i) + vb * static_cast<V>(k);
+            for (uint32_t m = 0; m < c; ++m, ++q, val += vc) {
+              if (q >= commit) continue;
               if (staged) {
                 stage[q + shv] = gen_value<E>(val);
               } else {
@@ -532,7 +559,6 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
               }
             }
           }
-          st += c;
         }
       }
     }

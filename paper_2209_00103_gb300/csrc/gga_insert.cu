@@ -804,7 +804,8 @@ int launch_finalize(const ArrayView& v, cudaStream_t st) {
 // and one share of every barrier serve them), GGA_GEN_MINB_VT resident per
 // SM with a GGA_GEN_STAGE_VT-byte stage: measured on GB300 for the
 // paper-shaped workload (1024 LFVectors x 512 threads x 512 rounds, int32),
-// 128 threads x 4, 8 per SM: 0.737 ms; 256 x 2, 4 per SM: 0.753 ms; 512 x 1,
+// 128 threads x 4, 8 per SM: 0.737 ms (0.545 ms since the draws are branch-free
+// and the write-out does its bucket math per bucket); 256 x 2, 4 per SM: 0.753 ms; 512 x 1,
 // 3 per SM (40 registers, 48 KB stage): 0.816 ms.  Other T use one virtual
 // thread per thread, blocks of up to 512 threads 3 per SM (up to 1024: 1).
 #ifndef GGA_GEN_VT
