@@ -440,6 +440,40 @@ struct BlockPusher {
   __device__ uint64_t lfv_size() const { return size; }
 };
 
+// What RoundsPusher::push_run hands to its writer for one round: put(m, x)
+// stores the thread's element m of the round.  kOneStore: it is a single
+// shared-memory store (the usual case: the whole push is staged), so a
+// writer may unroll around it; otherwise it tests and looks buckets up.
+template <class T>
+struct StagePut {
+  static constexpr bool kOneStore = true;
+  T* at;
+  __device__ __forceinline__ void operator()(uint32_t m, T x) const { at[m] = x; }
+};
+
+template <class T>
+struct CheckedPut {
+  static constexpr bool kOneStore = false;
+  T* stage;              // the stage (position base at its start), or nullptr: to the buckets
+  const uint64_t* tab;   // the LFVector's bucket table
+  uint64_t base;         // position of the push's first element
+  uint32_t log2B;
+  uint32_t q;            // the thread's first element of the round, from base
+  uint32_t n;            // elements kept
+  __device__ __forceinline__ void operator()(uint32_t m, T x) const {
+    const uint32_t p = q + m;
+    if (p >= n) return;
+    if (stage) {
+      stage[p] = x;
+    } else {
+      uint32_t b;
+      uint64_t off;
+      bucket_of(base + p, log2B, b, off);
+      reinterpret_cast<T*>(tab[b])[off] = x;
+    }
+  }
+};
+
 // Shared memory of one RoundsPusher<T, K> (declare it __shared__, one per
 // pusher).
 template <int K>
@@ -519,6 +553,26 @@ struct RoundsPusher {
   template <uint32_t CMAX = 0, class F>
   __device__ uint32_t push(const uint32_t (&count)[K], F value_of, uint32_t* kept = nullptr,
                            uint64_t* first = nullptr) {
+    return push_run(count, [&](uint32_t kr, auto put) {
+      if (CMAX > 0) {
+#pragma unroll
+        for (uint32_t m = 0; m + 1 <= CMAX; ++m)
+          if (m < count[kr]) put(m, value_of(kr, m));
+      } else {
+        for (uint32_t m = 0; m < count[kr]; ++m) put(m, value_of(kr, m));
+      }
+    }, kept, first);
+  }
+
+  // push with a round's elements in any order: write(kr, put) is called once
+  // for every round kr (in order, kr a constant of the unrolled loop) and
+  // calls put(m, element m) for every m < count[kr]; elements that are not
+  // kept are dropped by put.  What write reads is free once it returns, so
+  // it may load the next call's inputs there: they then arrive behind this
+  // call's write-out.
+  template <class W>
+  __device__ uint32_t push_run(const uint32_t (&count)[K], W write, uint32_t* kept = nullptr,
+                               uint64_t* first = nullptr) {
     if (!valid) return 0;
     const ArrayView& v = *view;
     const uint32_t nt = block_threads(), t = block_rank();
@@ -685,30 +739,18 @@ struct RoundsPusher {
     const bool staged = n > 0 && n + shv <= stage_elems && v.B >= VEC;   // block-uniform
     const bool whole = n == total;                                       // nothing clipped
     T* st = reinterpret_cast<T*>(stage);
+    if (staged && whole) {
+      T* const st0 = st + shv;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      if (first) first[k] = base + q[k];
-      const uint32_t c = count[k];
-      if (staged && whole && CMAX > 0) {
+      for (int k = 0; k < K; ++k) {
+        if (first) first[k] = base + q[k];
+        write(static_cast<uint32_t>(k), StagePut<T>{st0 + q[k]});
+      }
+    } else {
 #pragma unroll
-        for (uint32_t m = 0; m + 1 <= CMAX; ++m)
-          if (m < c) st[q[k] + m + shv] = static_cast<T>(value_of(static_cast<uint32_t>(k), m));
-      } else if (staged && whole) {
-        for (uint32_t m = 0; m < c; ++m) st[q[k] + m + shv] = static_cast<T>(value_of(static_cast<uint32_t>(k), m));
-      } else {
-        for (uint32_t m = 0; m < c; ++m) {
-          const uint32_t p = q[k] + m;
-          if (p >= n) break;
-          const T x = static_cast<T>(value_of(static_cast<uint32_t>(k), m));
-          if (staged) {
-            st[p + shv] = x;
-          } else {
-            uint32_t b;
-            uint64_t off;
-            bucket_of(base + p, v.log2B, b, off);
-            reinterpret_cast<T*>(sh->tab[b])[off] = x;
-          }
-        }
+      for (int k = 0; k < K; ++k) {
+        if (first) first[k] = base + q[k];
+        write(static_cast<uint32_t>(k), CheckedPut<T>{staged ? st + shv : nullptr, sh->tab, base, v.log2B, q[k], n});
       }
     }
     // Every thread is past its reads of sh->wt before the next call writes

@@ -124,20 +124,62 @@ int launch_push_generated(const ArrayView& v, const ArrayView* dview, const gga_
 
 // Memory-sourced pushes through the device API: block l appends, per
 // thread slot t and round r, counts[r][l][t] copies of inputs[r][l][t],
-// K rounds per gga::block_push_rounds call (staged, 128-bit stores).  A
+// K rounds per push of a gga::RoundsPusher (staged, 128-bit stores).  A
 // thread plays S consecutive slots S t, ..., S t + S - 1 and pushes their
 // counts together (its elements are slot S t's copies, then S t + 1's, ...,
 // which is their order in the LFVector): one scan slot and one share of
 // every barrier then serve S slots, and the blocks (512 / S threads for
 // T = 512) are small enough for all 1024 of the paper-shaped workload to
-// be resident at once.  Each thread loads its 2 K S counts and inputs of a
-// call before using any.  A call that does not fit ends the block's rounds.
+// be resident at once.  The kernel streams counts and inputs in and the
+// elements out; its rate is that of the bytes it keeps in flight.  With
+// WIDE (T a multiple of S, both buffers 16-byte aligned) a thread's S counts
+// and S inputs of a round are 128-bit loads, and a round's loads for the next
+// push are issued as soon as this push has staged the round, so they are in
+// flight during its barrier and write-out without a register more.  A push
+// that does not fit ends the block's rounds.
 // Measured on GB300 for the paper-shaped workload (1024 x 512, 512 rounds,
 // int32): one slot per thread, K = 8, 2 blocks per SM: 1.42 ms (with the
 // loads prefetched into shared memory by cp.async: 1.52 ms); S = 2, K = 4,
 // 4 per SM: 0.98 ms; S = 4, K = 2, 8 per SM: 0.90 ms; S = 4, K = 4, 8 per
-// SM: 0.84 ms.
-template <int E, int K, int S, int MINB>
+// SM: 0.84 ms, 0.80 with the write-out's bucket math per bucket; with one
+// cursor for all pushes, the wide early loads and stores without a loop 0.64 ms
+// (a loop per slot instead: 0.81).
+template <int S, typename V, bool WIDE>
+__device__ __forceinline__ void load_slots(V (&x)[S], const V* __restrict__ p, uint32_t have) {
+  constexpr uint32_t kWord = S * sizeof(V) >= 16 ? 16 : S * sizeof(V);   // bytes of a load
+  if constexpr (WIDE && kWord == 16) {
+    constexpr uint32_t kPer = 16 / sizeof(V);
+#pragma unroll
+    for (int i = 0; i < S; i += kPer) {
+      uint4 w = make_uint4(0, 0, 0, 0);
+      if (have) w = __ldcs(reinterpret_cast<const uint4*>(p + i));
+      if constexpr (sizeof(V) == 16) {
+        x[i] = w;
+      } else if constexpr (sizeof(V) == 8) {
+        x[i] = w.x | static_cast<V>(w.y) << 32;
+        x[i + 1] = w.z | static_cast<V>(w.w) << 32;
+      } else {
+        x[i] = w.x;
+        x[i + 1] = w.y;
+        x[i + 2] = w.z;
+        x[i + 3] = w.w;
+      }
+    }
+  } else if constexpr (WIDE && sizeof(V) == 4 && S == 2) {
+    uint2 w = make_uint2(0, 0);
+    if (have) w = __ldcs(reinterpret_cast<const uint2*>(p));
+    x[0] = w.x;
+    x[1] = w.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      x[i] = V();
+      if (static_cast<uint32_t>(i) < have) x[i] = __ldcs(p + i);
+    }
+  }
+}
+
+template <int E, int K, int S, int MINB, bool WIDE>
 __global__ void __launch_bounds__(512 / S, MINB) push_expand_s_kernel(const ArrayView* view,
                                                                   const uint32_t* __restrict__ counts,
                                                                   const typename Elem<E>::T* __restrict__ inputs,
@@ -145,52 +187,66 @@ __global__ void __launch_bounds__(512 / S, MINB) push_expand_s_kernel(const Arra
                                                                   uint32_t stage_bytes) {
   typedef typename Elem<E>::T V;
   extern __shared__ uint4 s_stage[];
+  __shared__ RoundsShared<K> s_rounds;
   const uint32_t l = blockIdx.x, t = S * threadIdx.x;
+  const uint32_t mine = t < T ? (T - t < S ? T - t : S) : 0u;   // slots this thread plays
+  const uint64_t at0 = static_cast<uint64_t>(l) * T + t, row = static_cast<uint64_t>(L) * T;
+  uint32_t cs[K][S];
+  V x[K][S];
+  auto load = [&](int k, uint32_t r) {
+    const uint64_t at = at0 + r * row;
+    const uint32_t have = r < R ? mine : 0u;
+    load_slots<S, uint32_t, WIDE>(cs[k], counts + at, have);
+    load_slots<S, V, WIDE>(x[k], inputs + at, have);
+  };
+#pragma unroll
+  for (int k = 0; k < K; ++k) load(k, k);
+  RoundsPusher<V, K> pusher(view, l, s_rounds, s_stage, stage_bytes);
 #pragma unroll 1
   for (uint32_t r0 = 0; r0 < R; r0 += K) {
-    uint32_t c[K], cs[K][S];
-    V x[K][S];
+    uint32_t c[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-      const uint32_t r = r0 + k;
       c[k] = 0;
 #pragma unroll
-      for (int i = 0; i < S; ++i) {
-        cs[k][i] = 0;
-        x[k][i] = V();
-        if (r < R && t + i < T) {
-          const uint64_t at = (static_cast<uint64_t>(r) * L + l) * T + t + i;
-          cs[k][i] = __ldcs(counts + at);
-          x[k][i] = __ldcs(inputs + at);
-        }
-        c[k] += cs[k][i];
-      }
+      for (int i = 0; i < S; ++i) c[k] += cs[k][i];
     }
-    const uint32_t done = block_push_rounds<V, K>(
-        view, l, c,
-        [&](uint32_t kr, uint32_t m) {
-          V v = x[kr][S - 1];
+    const uint32_t done = pusher.push_run(c, [&](uint32_t kr, auto put) {
+      // Two copies by predicated stores, the third and later ones (rare at
+      // about one copy per slot) by a loop only the threads that have some enter.
+      constexpr uint32_t kFlat = decltype(put)::kOneStore ? 2 : 0;
+      uint32_t m = 0, most = 0;
 #pragma unroll
-          for (int i = S - 2; i >= 0; --i) {
-            uint32_t before = 0;
+      for (int i = 0; i < S; ++i) {
+        const uint32_t n = cs[kr][i];
+        if constexpr (kFlat > 0) {
+          if (n > 0) put(m, x[kr][i]);
+          if (n > 1) put(m + 1, x[kr][i]);
+        }
+        m += n;
+        most = max(most, n);
+      }
+      if (most > kFlat) {
+        m = 0;
 #pragma unroll
-            for (int j = 0; j <= i; ++j) before += cs[kr][j];
-            if (m < before) v = x[kr][i];
-          }
-          return v;
-        },
-        s_stage, stage_bytes);
+        for (int i = 0; i < S; ++i) {
+          for (uint32_t j = kFlat; j < cs[kr][i]; ++j) put(m + j, x[kr][i]);
+          m += cs[kr][i];
+        }
+      }
+      load(static_cast<int>(kr), r0 + K + kr);
+    });
     if (done < static_cast<uint32_t>(K)) break;
   }
 }
 
-template <int E, int K, int S, int MINB>
-int launch_expand_s(const ArrayView& v, const ArrayView* dview, const uint32_t* counts, const void* inputs,
-                    uint32_t rounds, cudaStream_t st) {
+template <int E, int K, int S, int MINB, bool WIDE>
+int launch_expand_as(const ArrayView& v, const ArrayView* dview, const uint32_t* counts, const void* inputs,
+                     uint32_t rounds, cudaStream_t st) {
   const uint32_t NTS = ((v.T + S - 1) / S + 31) / 32 * 32;
   // Stage: twice a call's elements at one per slot of 512 (larger calls go unstaged).
   const size_t smem = static_cast<size_t>(K) * 512u * E * 2u;
-  auto kern = push_expand_s_kernel<E, K, S, MINB>;
+  auto kern = push_expand_s_kernel<E, K, S, MINB, WIDE>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   kern<<<v.L, NTS, smem, st>>>(dview, counts, static_cast<const typename Elem<E>::T*>(inputs), rounds, v.L, v.T,
                                static_cast<uint32_t>(smem));
@@ -198,11 +254,22 @@ int launch_expand_s(const ArrayView& v, const ArrayView* dview, const uint32_t* 
   return launch_finalize(v, st);
 }
 
+template <int E, int K, int S, int MINB>
+int launch_expand_s(const ArrayView& v, const ArrayView* dview, const uint32_t* counts, const void* inputs,
+                    uint32_t rounds, cudaStream_t st) {
+  // Every row of T counts and inputs then starts on a 16-byte boundary (8
+  // for two counts), and a thread plays all of its slots or none.
+  const bool wide = v.T % S == 0 &&
+                    ((reinterpret_cast<uintptr_t>(counts) | reinterpret_cast<uintptr_t>(inputs)) & 15) == 0;
+  return wide ? launch_expand_as<E, K, S, MINB, true>(v, dview, counts, inputs, rounds, st)
+              : launch_expand_as<E, K, S, MINB, false>(v, dview, counts, inputs, rounds, st);
+}
+
 int launch_push_expand(const ArrayView& v, const ArrayView* dview, const uint32_t* counts, const void* inputs,
                        uint32_t rounds, cudaStream_t st) {
   if (v.T > 512) return GGA_ERR_INVALID;
-  if (v.E == 4) return launch_expand_s<4, 4, 4, 8>(v, dview, counts, inputs, rounds, st);
-  if (v.E == 8) return launch_expand_s<8, 2, 4, 8>(v, dview, counts, inputs, rounds, st);
+  if (v.E == 4) return launch_expand_s<4, 4, 4, 7>(v, dview, counts, inputs, rounds, st);
+  if (v.E == 8) return launch_expand_s<8, 2, 4, 7>(v, dview, counts, inputs, rounds, st);
   return launch_expand_s<16, 2, 2, 4>(v, dview, counts, inputs, rounds, st);
 }
 
