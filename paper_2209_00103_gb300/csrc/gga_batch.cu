@@ -2,149 +2,38 @@
 //
 // A batch is a list of jobs: an array, the draws of its counts and values
 // (as gga_insert_generated), and a target size.  gga_batch_grow runs one
-// persistent kernel over all (array, LFVector) items, largest first, taken
-// from an atomic ticket: a block grows its LFVector in passes of several
-// rounds -- every thread draws its counts, a block scan gives positions,
-// counts are clipped at the LFVector's target by the same scan, the leader
-// reserves and allocates, the block stages the values and writes them with
-// 128-bit stores (Algorithm 1 with thread coarsening: a block of 512 threads
-// plays T <= 1024 threads).  Then one kernel folds the pool
-// pops and one finalizes every array.  Nothing allocates and nothing waits
-// on the host, so the whole step can be captured in a CUDA graph and
-// replayed (gga_batch_capture / gga_batch_replay).
+// persistent kernel per form (payload size and count distribution) over its
+// (array, LFVector) items, longest first, taken from atomic tickets
+// (gga_batch_grow.cuh): a block -- a cluster of blocks for the longest --
+// grows its LFVector in passes of several rounds: every thread draws its
+// counts, a block scan gives positions, counts are clipped at the LFVector's
+// target by the same scan, the leader reserves and allocates, the block
+// stages the pass and writes it with 128-bit stores (Algorithm 1 with thread
+// coarsening).  The forms run side by side, a form's blocks taking the SMs as
+// an earlier one's finish.  Then one kernel folds the pool pops and finalizes
+// every array.  Nothing allocates and nothing waits on the host, so the whole
+// step can be captured in a CUDA graph and replayed (gga_batch_capture /
+// gga_batch_replay).
 #include <algorithm>
 #include <new>
 #include <vector>
 
-#include "gga_gen.cuh"
+#include "gga_batch_grow.cuh"
 
 namespace gga {
-
-int launch_clear(const ArrayView& v, cudaStream_t st);
-
 namespace {
-
-// Threads per block and virtual threads per thread (T <= kBatchThreads *
-// kBatchKV = 1024) and resident blocks per SM.
-#ifndef GGA_BATCH_THREADS
-#define GGA_BATCH_THREADS 512
-#endif
-constexpr int kBatchThreads = GGA_BATCH_THREADS;
-constexpr int kBatchKV = 1024 / kBatchThreads;
-constexpr int kBatchMinBlocks = 1024 / kBatchThreads;
-// Stage of a pass: 80 KB, two blocks per SM.  Measured on GB300 for the
-// 4096-array workload (rounds per pass for 8- / 16-byte payloads): 48 KB
-// with 4 / 2 rounds 4.30 ms, 80 KB with 4 / 4 rounds 4.24 ms, 96 KB with
-// 4 / 4 4.25 ms, with 6 / 4 4.31 ms.
-constexpr uint32_t kBatchStageBytes = 81920;
-constexpr uint32_t kBatchMaxRounds = 1u << 20;
-
-struct BatchJob {
-  ArrayView v;
-  GenParams g;
-  uint64_t target;
-};
-
-struct BatchItem {
-  uint32_t job;
-  uint32_t l;
-};
-
-// Grow LFVector l of job J to its share of the target: rounds of in-thread
-// insertions in passes of K (grow_passes in gga_gen.cuh), clipped at the
-// target.  All threads of the block call it.
-#ifndef GGA_BATCH_NOINLINE
-#define GGA_BATCH_NOINLINE 0
-#endif
-// One distribution's pass loop; with GGA_BATCH_NOINLINE a function of its
-// own, register-allocated apart from the other (payload, distribution) forms.
-template <int E, int K, int DIST>
-__device__ __forceinline__ uint32_t grow_item_passes_inl(const ArrayView& v, const GenParams& g, uint32_t l,
-                                                         uint64_t target, GenShared& sh, uint4* stage, bool* done) {
-  return grow_passes<E, K, kBatchKV, true, DIST>(v, g, l, kBatchMaxRounds, target, sh, stage, kBatchStageBytes / E,
-                                                 done);
-}
-template <int E, int K, int DIST>
-__device__ __noinline__ uint32_t grow_item_passes_call(const ArrayView& v, const GenParams& g, uint32_t l,
-                                                       uint64_t target, GenShared& sh, uint4* stage, bool* done) {
-  return grow_item_passes_inl<E, K, DIST>(v, g, l, target, sh, stage, done);
-}
-template <int E, int K, int DIST>
-__device__ __forceinline__ uint32_t grow_item_passes(const ArrayView& v, const GenParams& g, uint32_t l,
-                                                     uint64_t target, GenShared& sh, uint4* stage, bool* done) {
-  return GGA_BATCH_NOINLINE ? grow_item_passes_call<E, K, DIST>(v, g, l, target, sh, stage, done)
-                            : grow_item_passes_inl<E, K, DIST>(v, g, l, target, sh, stage, done);
-}
-
-template <int E>
-__device__ void grow_item(const BatchJob& J, uint32_t l, GenShared& sh, uint4* stage) {
-  const ArrayView& v = J.v;
-  const uint64_t target = J.target / v.L + (l < J.target % v.L ? 1 : 0);
-  // Rounds per pass: a pass of T <= 1024 threads at one element per thread
-  // and round then averages <= 64 KB, inside the 80 KB stage.
-  constexpr int K = E == 4 ? 8 : 4;
-  uint32_t drawn;
-  bool done;
-  // One dispatch per item on the count distribution, none per draw.
-  switch (J.g.dist) {
-    case GGA_DIST_BERNOULLI:
-      drawn = grow_item_passes<E, K, GGA_DIST_BERNOULLI>(v, J.g, l, target, sh, stage, &done);
-      break;
-    case GGA_DIST_UNIFORM3:
-      drawn = grow_item_passes<E, K, GGA_DIST_UNIFORM3>(v, J.g, l, target, sh, stage, &done);
-      break;
-    case GGA_DIST_GEOMETRIC:
-      drawn = grow_item_passes<E, K, GGA_DIST_GEOMETRIC>(v, J.g, l, target, sh, stage, &done);
-      break;
-    default:
-      drawn = grow_item_passes<E, K, GGA_DIST_POISSON>(v, J.g, l, target, sh, stage, &done);
-      break;
-  }
-  if (threadIdx.x == 0 && !done && drawn >= kBatchMaxRounds) latch_error(v.status, GGA_ERR_TIMEOUT);
-  __syncthreads();
-}
-
-__global__ void __launch_bounds__(kBatchThreads, kBatchMinBlocks) batch_grow_kernel(const BatchJob* __restrict__ jobs,
-                                                                      const BatchItem* __restrict__ items,
-                                                                      uint32_t n_items, uint32_t* ticket) {
-  extern __shared__ uint4 s_stage4[];
-  __shared__ GenShared sh;
-  __shared__ uint32_t s_item;
-  // The item's job (its view and draws) in shared memory: the pass loop
-  // reads these fields over and over, and from here they are shared-memory
-  // loads instead of global ones.
-  __shared__ __align__(16) BatchJob s_job;
-  static_assert(sizeof(BatchJob) % 8 == 0, "job copied in 8-byte words");
-  while (true) {
-    if (threadIdx.x == 0) s_item = atomicAdd(ticket, 1u);
-    __syncthreads();
-    const uint32_t it = s_item;
-    if (it >= n_items) break;
-    const BatchItem item = items[it];
-    if (threadIdx.x < sizeof(BatchJob) / 8)
-      reinterpret_cast<unsigned long long*>(&s_job)[threadIdx.x] =
-          reinterpret_cast<const unsigned long long*>(jobs + item.job)[threadIdx.x];
-    __syncthreads();
-    const BatchJob& J = s_job;
-    switch (J.v.E) {
-      case 4: grow_item<4>(J, item.l, sh, s_stage4); break;
-      case 8: grow_item<8>(J, item.l, sh, s_stage4); break;
-      default: grow_item<16>(J, item.l, sh, s_stage4); break;
-    }
-  }
-}
 
 // The prefix sums of every job's array, one block each.  After a growth
 // (pools given) the blocks also fold the grow kernel's pops into the pools'
-// queue heads -- a batch has no more pools than jobs -- and reset the ticket
+// queue heads -- a batch has no more pools than jobs -- and reset the tickets
 // for the next run.
 __global__ void __launch_bounds__(256) batch_finalize_kernel(const BatchJob* __restrict__ jobs,
                                                              PoolState* const* pools, uint32_t n_pools,
-                                                             uint32_t* ticket) {
+                                                             uint32_t* tickets) {
   __shared__ FinalizeShared sh;
   if (pools) {
     if (blockIdx.x < n_pools) ring_fixup_class(pools[blockIdx.x], threadIdx.x);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
+    if (blockIdx.x == 0 && threadIdx.x < kBatchLaunches) tickets[threadIdx.x] = 0;
   }
   finalize_block(jobs[blockIdx.x].v, nullptr, nullptr, nullptr, 1, sh);
 }
@@ -173,24 +62,62 @@ __global__ void batch_clear_kernel(const BatchJob* __restrict__ jobs, const Batc
 
 struct gga_batch_t {
   gga::BatchJob* jobs;
-  gga::BatchItem* items;
+  gga::BatchItem* items;      // form by form
   gga::PoolState** pools;
-  uint32_t* ticket;
+  uint32_t* tickets;          // one per launch
   uint32_t n_jobs, n_items, n_pools;
-  int num_sms;
-  unsigned grid;
+  uint32_t n_launches;
+  gga::BatchLaunch launch[gga::kBatchLaunches];
+  // Streams of the second and later launches, forked from and joined to the
+  // caller's stream by events.
+  cudaStream_t side[gga::kBatchLaunches];
+  cudaEvent_t fork, join[gga::kBatchLaunches];
   cudaGraphExec_t graph;
   bool has_graph;
 };
 
 namespace {
 
+// Passes one block takes to draw an LFVector of `target` elements: rounds
+// at the distribution's mean count, batch_rounds a pass.
+uint64_t expected_passes(const gga::BatchJob& J, uint64_t target) {
+  double mean = J.g.dist == GGA_DIST_BERNOULLI ? 0.5 : 1.0;
+  if (J.g.dist == GGA_DIST_POISSON) {
+    mean = 0;
+    for (uint32_t k = 0; k < J.g.nthr; ++k) mean += 1.0 - J.g.thr[k] / 4294967296.0;
+  }
+  const double per_pass = mean * J.v.T * gga::batch_rounds(static_cast<int>(J.v.E), J.g.dist);
+  const double p = per_pass > 0 ? static_cast<double>(target) / per_pass : 1e12;
+  return p < 1e12 ? static_cast<uint64_t>(p) + 1 : static_cast<uint64_t>(1e12);
+}
+
+void launch_form(const gga::BatchLaunch& a, cudaStream_t st) {
+  switch (a.form >> 2) {
+    case 0: gga::launch_batch_form<4>(a, st); break;
+    case 1: gga::launch_batch_form<8>(a, st); break;
+    default: gga::launch_batch_form<16>(a, st); break;
+  }
+}
+
+int blocks_per_sm(uint32_t form, bool clusters) {
+  return form >> 2 == 0 ? gga::batch_blocks_per_sm<4>(form, clusters)
+                        : (form >> 2 == 1 ? gga::batch_blocks_per_sm<8>(form, clusters)
+                                          : gga::batch_blocks_per_sm<16>(form, clusters));
+}
+
 int batch_grow(gga_batch_t* b, cudaStream_t st) {
-  if (b->n_items)
-    gga::batch_grow_kernel<<<b->grid, gga::kBatchThreads, gga::kBatchStageBytes, st>>>(b->jobs, b->items,
-                                                                                         b->n_items, b->ticket);
-  if (b->n_jobs) gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs, b->pools, b->n_pools, b->ticket);
-  return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
+  bool ok = true;
+  if (b->n_launches > 1) ok = cudaEventRecord(b->fork, st) == cudaSuccess;
+  for (uint32_t i = 0; i < b->n_launches && ok; ++i) {
+    cudaStream_t s = i == 0 ? st : b->side[i];
+    if (i) ok = cudaStreamWaitEvent(s, b->fork, 0) == cudaSuccess;
+    launch_form(b->launch[i], s);
+    if (i) ok = cudaEventRecord(b->join[i], s) == cudaSuccess && ok;
+  }
+  for (uint32_t i = 1; i < b->n_launches && ok; ++i) ok = cudaStreamWaitEvent(st, b->join[i], 0) == cudaSuccess;
+  if (b->n_jobs)
+    gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs, b->pools, b->n_pools, b->tickets);
+  return ok && cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 
 int batch_clear(gga_batch_t* b, cudaStream_t st) {
@@ -206,8 +133,13 @@ extern "C" {
 int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, gga_batch* out) {
   if (!out || (n_jobs && !jobs)) return GGA_ERR_INVALID;
   *out = nullptr;
+  struct Item {
+    uint32_t form;
+    uint64_t passes;
+    gga::BatchItem it;
+  };
   std::vector<gga::BatchJob> hj(n_jobs);
-  std::vector<std::pair<uint64_t, gga::BatchItem>> hi;
+  std::vector<Item> hi;
   std::vector<gga::PoolState*> hp;
   int num_sms = 0;
   for (uint32_t j = 0; j < n_jobs; ++j) {
@@ -220,48 +152,61 @@ int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, g
       return GGA_ERR_INVALID;
     hj[j].g = gga::make_gen_params(sp);
     hj[j].target = jobs[j].target;
-    const uint32_t L = hj[j].v.L;
+    const uint32_t L = hj[j].v.L, E = hj[j].v.E;
+    const uint32_t form = (E == 4 ? 0u : (E == 8 ? 4u : 8u)) + sp.dist;
     for (uint32_t l = 0; l < L; ++l) {
       const uint64_t tl = jobs[j].target / L + (l < jobs[j].target % L ? 1 : 0);
-      if (tl) hi.push_back({tl, gga::BatchItem{j, l}});
+      if (tl) hi.push_back({form, expected_passes(hj[j], tl), gga::BatchItem{j, l}});
     }
     if (std::find(hp.begin(), hp.end(), hj[j].v.pool) == hp.end()) hp.push_back(hj[j].v.pool);
   }
-  // Largest LFVectors first: the ticket then balances the tail.
-  std::stable_sort(hi.begin(), hi.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  // Form by form, longest chains first: the tickets then balance
+  // the tail.
+  std::stable_sort(hi.begin(), hi.end(), [](const Item& a, const Item& b) {
+    return a.form != b.form ? a.form < b.form : a.passes > b.passes;
+  });
   std::vector<gga::BatchItem> items(hi.size());
-  for (size_t i = 0; i < hi.size(); ++i) items[i] = hi[i].second;
+  uint64_t sum = 0;
+  for (size_t i = 0; i < hi.size(); ++i) {
+    items[i] = hi[i].it;
+    sum += hi[i].passes;
+  }
 
-  gga_batch_t* b = new (std::nothrow) gga_batch_t();
+  gga_batch_t* b = new (std::nothrow) gga_batch_t();   // zeroed
   if (!b) return GGA_ERR_CUDA;
   b->n_jobs = n_jobs;
   b->n_items = static_cast<uint32_t>(items.size());
   b->n_pools = static_cast<uint32_t>(hp.size());
-  b->has_graph = false;
-  b->jobs = nullptr;
-  b->items = nullptr;
-  b->pools = nullptr;
-  b->ticket = nullptr;
-  if (num_sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+  // A form's items grown by clusters: those whose chain is long enough for
+  // the cluster's larger passes (of which the target clips the last), and
+  // longer than a quarter of a block's average load over the whole batch.
+  // (The rest then ends within a quarter of that load.)
+  struct Form {
+    uint32_t id, first, n, big;
+    uint64_t passes, big_passes;
+  };
+  std::vector<Form> forms;
+  uint64_t big_sum = 0;
+  const uint64_t blocks = static_cast<uint64_t>(std::max(num_sms, 1)) * gga::kBatchMinBlocks;
+  for (uint32_t i = 0; i < b->n_items; ++i) {
+    if (forms.empty() || forms.back().id != hi[i].form) forms.push_back({hi[i].form, i, 0, 0, 0, 0});
+    Form& f = forms.back();
+    if (f.big == f.n && hi[i].passes >= 4 * gga::kBatchCluster && hi[i].passes * 4 > sum / blocks) {
+      ++f.big;
+      f.big_passes += hi[i].passes;
+      big_sum += hi[i].passes;
+    }
+    ++f.n;
+    f.passes += hi[i].passes;
   }
-  b->num_sms = num_sms;
-  int per_sm = 0;
-  cudaFuncSetAttribute(gga::batch_grow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       static_cast<int>(gga::kBatchStageBytes));
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gga::batch_grow_kernel, gga::kBatchThreads,
-                                                    gga::kBatchStageBytes) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  b->grid = static_cast<unsigned>(num_sms * per_sm);
+  // The form with most work first.
+  std::stable_sort(forms.begin(), forms.end(), [](const Form& x, const Form& y) { return x.passes > y.passes; });
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = GGA_OK;
   if (cudaMalloc(&b->jobs, sizeof(gga::BatchJob) * (n_jobs ? n_jobs : 1)) != cudaSuccess ||
       cudaMalloc(&b->items, sizeof(gga::BatchItem) * (items.empty() ? 1 : items.size())) != cudaSuccess ||
       cudaMalloc(&b->pools, sizeof(gga::PoolState*) * (hp.empty() ? 1 : hp.size())) != cudaSuccess ||
-      cudaMalloc(&b->ticket, sizeof(uint32_t)) != cudaSuccess)
+      cudaMalloc(&b->tickets, gga::kBatchLaunches * sizeof(uint32_t)) != cudaSuccess)
     rc = GGA_ERR_CUDA;
   if (rc == GGA_OK &&
       ((n_jobs && cudaMemcpyAsync(b->jobs, hj.data(), sizeof(gga::BatchJob) * n_jobs, cudaMemcpyHostToDevice, st) !=
@@ -270,8 +215,29 @@ int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, g
                                           cudaMemcpyHostToDevice, st) != cudaSuccess) ||
        (!hp.empty() && cudaMemcpyAsync(b->pools, hp.data(), sizeof(gga::PoolState*) * hp.size(),
                                        cudaMemcpyHostToDevice, st) != cudaSuccess) ||
-       cudaMemsetAsync(b->ticket, 0, sizeof(uint32_t), st) != cudaSuccess ||
+       cudaMemsetAsync(b->tickets, 0, gga::kBatchLaunches * sizeof(uint32_t), st) != cudaSuccess ||
        cudaStreamSynchronize(st) != cudaSuccess))
+    rc = GGA_ERR_CUDA;
+  // The cluster kernels first, then the block kernels.
+  for (int clusters = 1; clusters >= 0; --clusters) {
+    for (size_t k = 0; k < forms.size() && rc == GGA_OK; ++k) {
+      const Form& f = forms[k];
+      const uint32_t n = clusters ? f.big : f.n - f.big, unit = clusters ? gga::kBatchCluster : 1;
+      if (n == 0) continue;
+      // As many units as are resident at once -- for the cluster kernels the
+      // form's share of them by its passes, so that every form's longest
+      // chains start at once -- or as there are items.
+      uint64_t fit = static_cast<uint64_t>(num_sms) * blocks_per_sm(f.id, clusters != 0) / unit;
+      if (clusters) fit = fit * f.big_passes / big_sum;
+      const uint32_t i = b->n_launches++;
+      b->launch[i] = gga::BatchLaunch{f.id, clusters != 0, b->jobs, b->items + f.first + (clusters ? 0 : f.big),
+                                      n, b->tickets + i, static_cast<uint32_t>(std::max<uint64_t>(1, std::min<uint64_t>(fit, n))) * unit};
+      if (i && (cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+                cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming) != cudaSuccess))
+        rc = GGA_ERR_CUDA;
+    }
+  }
+  if (rc == GGA_OK && b->n_launches > 1 && cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess)
     rc = GGA_ERR_CUDA;
   if (rc != GGA_OK) {
     gga_batch_destroy(b);
@@ -324,10 +290,15 @@ int gga_batch_destroy(gga_batch b) {
   int rc = GGA_OK;
   if (cudaDeviceSynchronize() != cudaSuccess) rc = GGA_ERR_CUDA;
   if (b->has_graph) cudaGraphExecDestroy(b->graph);
+  for (int i = 0; i < gga::kBatchLaunches; ++i) {
+    if (b->side[i]) cudaStreamDestroy(b->side[i]);
+    if (b->join[i]) cudaEventDestroy(b->join[i]);
+  }
+  if (b->fork) cudaEventDestroy(b->fork);
   if (b->jobs) cudaFree(b->jobs);
   if (b->items) cudaFree(b->items);
   if (b->pools) cudaFree(b->pools);
-  if (b->ticket) cudaFree(b->ticket);
+  if (b->tickets) cudaFree(b->tickets);
   delete b;
   return rc;
 }

@@ -285,41 +285,56 @@ __host__ __device__ constexpr uint32_t max_count() {
   return DIST == GGA_DIST_BERNOULLI ? 1u : (DIST == GGA_DIST_UNIFORM3 ? 2u : 0u);
 }
 
-// Threshold counts (ascending thresholds) per interval of 2^24 draws, in
-// shared memory: ptab[i] holds c_i = #{k : thr[k] <= i * 2^24} in its top 7
-// bits and, in its low 25, the offset of the next threshold thr[c_i] from
-// i * 2^24 when that threshold lies inside the interval, else 2^24 (no draw
-// of the interval reaches it).  A draw u of interval i counts c_i when its
-// low 24 bits stay below that offset -- one table load -- and otherwise
-// steps over the thresholds from c_i + 1.
+// Threshold counts (ascending thresholds) per interval of 2^23 draws, in
+// shared memory: entry i is {c_i, next_i}, c_i = #{k : thr[k] <= i * 2^23}
+// and next_i the threshold after those if it lies inside the interval (else
+// 2^32 - 1).  A draw u of interval i counts c_i + (u >= next_i): one table
+// load and no branch, unless u reaches `second`, the least value at which
+// that could be wrong (the second threshold inside some interval, or
+// 2^32 - 1), where the thresholds are stepped over.  (Poisson(1): thr[6], one
+// draw in 12,000; with 256 intervals it is thr[5], one in 1,700, and a warp
+// of eight draws per thread takes the slow way every seventh time.)
 struct ThresholdTable {
+  static constexpr uint32_t kShift = 23, kEntries = 1u << (32 - kShift);
   uint32_t thr[GGA_MAX_THRESHOLDS];
-  uint32_t ptab[256];
+  uint2 tab[kEntries];
+  uint32_t second;
 
   // Fill from ascending g.thr[0 .. nthr) (every thread of the block; a
   // barrier must follow).
   __device__ __forceinline__ void fill(const GenParams& g, uint32_t t, uint32_t nt) {
     for (uint32_t i = t; i < GGA_MAX_THRESHOLDS; i += nt) thr[i] = g.thr[i];
-    for (uint32_t i = t; i < 256; i += nt) {
+    for (uint32_t i = t; i < kEntries; i += nt) {
       uint32_t c = 0;
-      for (uint32_t k = 0; k < g.nthr; ++k) c += g.thr[k] <= (i << 24) ? 1u : 0u;
-      const uint64_t lo = static_cast<uint64_t>(i) << 24;
-      const uint32_t rel = c < g.nthr && g.thr[c] < lo + (1u << 24) ? static_cast<uint32_t>(g.thr[c] - lo) : (1u << 24);
-      ptab[i] = (c << 25) | rel;
+      for (uint32_t k = 0; k < g.nthr; ++k) c += g.thr[k] <= (i << kShift) ? 1u : 0u;
+      tab[i] = make_uint2(c, c < g.nthr && g.thr[c] >> kShift == i ? g.thr[c] : ~0u);
+    }
+    if (t == 0) {
+      second = ~0u;
+      for (uint32_t k = g.nthr; k-- > 1;)
+        if (g.thr[k] >> kShift == g.thr[k - 1] >> kShift && (g.thr[k - 1] & ((1u << kShift) - 1u)) != 0)
+          second = g.thr[k];
     }
   }
 
-  // #{k < nthr : u >= thr[k]} for the high word u of a draw.
+  // The count of a draw with high word u < second.
+  __device__ __forceinline__ uint32_t first_count(uint32_t u) const {
+    const uint2 e = tab[u >> kShift];
+    return e.x + (u >= e.y ? 1u : 0u);
+  }
+
+  // #{k < nthr : u >= thr[k]} for the high word u of any draw.
   __device__ __forceinline__ uint32_t count(uint32_t nthr, uint32_t u) const {
-    const uint32_t e = ptab[u >> 24];
-    uint32_t c = e >> 25;
-    if ((u & 0xFFFFFFu) >= (e & 0x1FFFFFFu)) {
-      ++c;
+    uint32_t c = first_count(u);
+    if (u >= second) {
+      c = 0;
       while (c < nthr && u >= thr[c]) ++c;
     }
     return c;
   }
 };
+
+constexpr int kMaxCluster = 8;
 
 struct GenShared {
   uint32_t wt[4][32];         // packed warp prefixes (K / 2 <= 4 words)
@@ -329,25 +344,181 @@ struct GenShared {
   int stop;                   // 1: pool exhausted, 2: target reached
   uint64_t tab[kMaxBuckets];  // the LFVector's bucket table (copy)
   ThresholdTable thr;
+  // Clusters only, written by the peers: the blocks' pass totals (by pass
+  // parity) and the allocated buckets after a growth.
+  uint32_t peer_total[2][kMaxCluster];
+  uint32_t peer_nb;
 };
+
+// Thread-block cluster operations (the blocks of a cluster are co-resident,
+// so their barrier always completes).
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Store x to block `rank`'s copy of this block's shared variable *p.
+__device__ __forceinline__ void cluster_store(uint32_t* p, uint32_t rank, uint32_t x) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+}
+
+// *p = x in shared memory if `cond`, as a predicated store.  (As an `if` the
+// generated insertion of 4-byte uniform counts took 53.5 instructions per
+// draw against 49.9, 80 us against 72 for 2^25 draws on GB300.)
+template <int E>
+__device__ __forceinline__ void store_shared_if(typename Elem<E>::T* p, typename Elem<E>::T x, bool cond) {
+  const uint32_t a = smem_u32(p), c = cond ? 1u : 0u;
+  if constexpr (E == 4) {
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; @q st.shared.u32 [%0], %1;}" ::"r"(a), "r"(x), "r"(c) : "memory");
+  } else if constexpr (E == 8) {
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; @q st.shared.u64 [%0], %1;}" ::"r"(a), "l"(x), "r"(c) : "memory");
+  } else {
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %5, 0; @q st.shared.v4.u32 [%0], {%1, %2, %3, %4};}" ::"r"(a), "r"(x.x),
+                 "r"(x.y), "r"(x.z), "r"(x.w), "r"(c)
+                 : "memory");
+  }
+}
+
+// Marks.  A thread whose counts have no small bound would store its elements
+// one by one in a loop that runs as often as the largest count of its warp,
+// most lanes idle, and compute every value there.  Such a pass stages one
+// 32-bit mark per non-empty draw instead, at its first element's stage index
+// si: ((si + 1) << 13) | (round of the pass << 10) | (virtual thread).  Marks
+// grow with si, so the draw an element belongs to is the largest mark at or
+// before it: a running maximum, which the write-out takes with a warp scan
+// and from which every lane computes its own elements' values.  Indices with
+// no mark hold zero.  Measured on GB300 for 2^25 draws (1024 LFVectors x 512
+// threads), elements stored in loops / by marks: geometric counts 219 / 117
+// us (4 bytes), 378 / 133 (8), 337 / 157 (16); Poisson 216 / 125, 278 / 139,
+// 296 / 161.
+constexpr uint32_t kMarkBits = 13;   // 3 of the round, 10 of the virtual thread
+constexpr uint32_t kMarkMaxStage = (1u << (32 - kMarkBits)) - 2u;
+// Consecutive elements of a lane in a step of the write-out: as many as its
+// 128-bit stores still cover whole 32-byte sectors with.  (Four records a
+// lane: 197 us against 161 for 2^25 draws on GB300.)
+constexpr uint32_t mark_group(int E) { return E == 16 ? 2 : 4; }
+
+// Writes the n elements of a marked pass (stage indices shv .. shv + n - 1,
+// position base at shv, shv = base mod mark_group(E)) to
+// their buckets; all threads of the block, after a barrier that follows the
+// marks.  Element m of draw (k, vt) is v0 + va * vt + vb * k + vc * m.  A warp
+// takes a contiguous span of each bucket's part, a lane mark_group(E)
+// consecutive elements at a time.
+template <int E, typename V>
+__device__ __forceinline__ void marks_to_buckets(const uint64_t* tab, uint32_t log2B, uint64_t base, uint32_t n,
+                                                 uint32_t shv, const uint32_t* marks, V v0, V va, V vb, V vc,
+                                                 uint32_t t, uint32_t nt) {
+  typedef typename Elem<E>::T T;
+  constexpr uint32_t G = mark_group(E);
+  const uint32_t lane = t & 31, warp = t >> 5, nw = nt >> 5;
+  const uint64_t gbeg = base - shv;
+  const uint32_t end = n + shv;
+  for (uint32_t s0 = 0; s0 < end;) {       // block-uniform: the part in one bucket
+    uint32_t bb;
+    uint64_t off;
+    bucket_of(gbeg + s0, log2B, bb, off);
+    const uint64_t room = bucket_len(bb, log2B) - off;
+    const uint32_t s1 = room < end - s0 ? s0 + static_cast<uint32_t>(room) : end;
+    T* const dst = reinterpret_cast<T*>(tab[bb] + off * sizeof(T));   // element s0's place
+    const uint32_t steps = (s1 - s0 + 32 * G - 1) / (32 * G), per = (steps + nw - 1) / nw;
+    uint32_t c = s0 + warp * per * (32 * G);
+    const uint32_t cend = min(s1, c + per * (32 * G));
+    // The last mark before the span: a draw has at most 63 elements, so it
+    // lies within the 64 indices before (or there is none: the run's start).
+    uint32_t carry = 0;
+    if (c < cend) {
+#pragma unroll
+      for (uint32_t back = 0; back < 64; back += 32) {
+        const uint32_t d = back + 1 + lane;
+        const uint32_t w = d <= c ? marks[c - d] : 0u;
+        if (carry == 0) carry = __reduce_max_sync(0xffffffffu, w);
+      }
+    }
+    for (; c < cend; c += 32 * G) {        // warp-uniform
+      const uint32_t si = c + lane * G;
+      uint32_t w[G];
+      if constexpr (G == 4) {
+        const uint4 x = *reinterpret_cast<const uint4*>(marks + si);
+        w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
+      } else {
+        const uint2 x = *reinterpret_cast<const uint2*>(marks + si);
+        w[0] = x.x; w[1] = x.y;
+      }
+#pragma unroll
+      for (uint32_t e = 1; e < G; ++e) w[e] = max(w[e], w[e - 1]);
+      uint32_t inc = w[G - 1];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) inc = max(inc, __shfl_up_sync(0xffffffffu, inc, o));   // own value below lane o
+      uint32_t ex = __shfl_up_sync(0xffffffffu, inc, 1);
+      if (lane == 0) ex = 0;
+      ex = max(ex, carry);
+      carry = max(carry, __shfl_sync(0xffffffffu, inc, 31));
+      if (si >= s1) continue;
+      union {
+        T e[G];
+        uint4 q[sizeof(T) * G / 16];
+      } x;
+#pragma unroll
+      for (uint32_t e = 0; e < G; ++e) {
+        const uint32_t m = max(w[e], ex);
+        x.e[e] = gen_value<E>(v0 + va * static_cast<V>(m & 1023u) + vb * static_cast<V>((m >> 10) & 7u) +
+                              vc * static_cast<V>(si + e + 1 - (m >> kMarkBits)));
+      }
+      T* const p = dst + (si - s0);
+      if (si >= shv && si + G <= s1) {
+#pragma unroll
+        for (uint32_t i = 0; i < sizeof(T) * G / 16; ++i) __stcs(reinterpret_cast<uint4*>(p) + i, x.q[i]);
+      } else {
+#pragma unroll
+        for (uint32_t e = 0; e < G; ++e)
+          if (si + e >= shv && si + e < s1) p[e] = x.e[e];
+      }
+    }
+    s0 = s1;
+  }
+}
+
+// Zero for marks[0 .. n), by all threads of the block.
+__device__ __forceinline__ void clear_marks(uint4* marks4, uint32_t n, uint32_t t, uint32_t nt) {
+  for (uint32_t i = t; i < (n + 3) / 4; i += nt) marks4[i] = make_uint4(0, 0, 0, 0);
+}
 
 // Returns the number of rounds it drew; *done is set when the LFVector
 // reached `target` or the pool ran out.  Every thread of the block calls
 // it.  SEARCH as for gen_count (g in shared memory); DIST as for
 // gen_count_state (-1: g.dist at run time).
-template <int E, int K, int KV, bool SEARCH = false, int DIST = -1>
+//
+// C > 1: the C blocks of a cluster grow the LFVector together, block q of a
+// pass drawing its rounds q K .. q K + K - 1 of the pass's C K.  The blocks
+// store their totals into one another's shared memory, one cluster barrier
+// takes the place of the pass's second block barrier, and every block then
+// knows where its run starts and whether the pass stays inside the allocated
+// buckets; only when it does not, block 0 allocates behind a second cluster
+// barrier.  Draws, positions, clipping and the rounds kept when the pool
+// runs out are those of one block drawing the same rounds one after another.
+template <int E, int K, int KV, bool SEARCH = false, int DIST = -1, int C = 1>
 __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t l, uint32_t R, uint64_t target,
                                 GenShared& sh, uint4* stage4, uint32_t cap, bool* done) {
   typedef typename Elem<E>::T T;
   constexpr uint32_t VEC = 16 / E;
   constexpr int KP = K / 2;
   static_assert(K % 2 == 0 && K <= 8, "K rounds per pass: even, at most 8");
+  static_assert(KV == 1 || KV == 4, "a round's counts in one word");
   T* stage = reinterpret_cast<T*>(stage4);
   const uint32_t t0 = threadIdx.x, NT = blockDim.x;
   const int lane = t0 & 31, warp = t0 >> 5, nwarps = NT >> 5;
   const uint32_t kv = KV == 1 ? 1u : (v.T + NT - 1) / NT;
   const uint64_t tfirst = static_cast<uint64_t>(t0) * kv;        // first virtual thread
   const uint32_t nvt = tfirst < v.T ? min(kv, v.T - static_cast<uint32_t>(tfirst)) : 0u;   // virtual threads played
+  const uint32_t played = nvt >= 4 ? ~0u : (1u << (8 * nvt)) - 1u;   // a byte of ones per virtual thread
   const uint64_t gfirst = static_cast<uint64_t>(l) * v.T + tfirst;
   const uint64_t* bk = v.buckets + static_cast<uint64_t>(l) * kMaxBuckets;
   RoundDraws dv[KV];   // virtual threads gfirst, ..., gfirst + KV - 1
@@ -365,47 +536,80 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
   const bool tabled = DIST == GGA_DIST_POISSON && g.thr_sorted;   // uniform
   if (tabled) sh.thr.fill(g, t0, NT);
   __syncthreads();
-  uint32_t r0 = 0;
+  const uint32_t rank = C > 1 ? cluster_rank() : 0u;
+  uint32_t par = 0;
+  // Counts without a small bound are staged as marks (buckets must hold a
+  // lane's group); `dirty` marks of the last pass are still set.
+  constexpr bool kMarks = !(DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2);
+  constexpr uint32_t kGroup = mark_group(E);
+  uint32_t* const marks = reinterpret_cast<uint32_t*>(stage4);
+  const uint32_t mark_cap = v.B < kGroup ? 0u : min(cap * static_cast<uint32_t>(E / 4) - 32 * kGroup, kMarkMaxStage);
+  // (a warp's last step of the write-out reads up to 32 groups past the end)
+  uint32_t dirty = 0;
+  if (kMarks) clear_marks(stage4, cap * (E / 4), t0, NT);   // (the pass's barriers come before the first mark)
+  uint32_t r0 = 0;   // the pass's first round
   while (r0 < R && sh.stop == 0) {
-    const uint32_t kk = min(static_cast<uint32_t>(K), R - r0);
-    // pk: the thread's per-round sums, two rounds per word.  cw: with KV
-    // virtual threads, the counts of the first KV - 1 of them, one byte
-    // each (round k, virtual thread i at byte k * (KV - 1) + i; the last
-    // one's count is the sum minus theirs); with one, the count is pk's
-    // half-word.
-    constexpr int KC = KV > 1 ? (K * (KV - 1) + 3) / 4 : 1;
-    uint32_t pk[KP], inc[KP], cw[KC];
+    const uint32_t rb0 = r0 + rank * K;   // this block's first round of the pass
+    const uint32_t kk = rb0 < R ? min(static_cast<uint32_t>(K), R - rb0) : 0u;
+    // exw: the thread's offsets in its warp, two rounds per word; cw: its
+    // counts, one byte each (round k, virtual thread i at byte k * KV + i).
+    constexpr int KC = (K * KV + 3) / 4;
+    uint32_t exw[KP], cw[KC];
 #pragma unroll
     for (int q = 0; q < KC; ++q) cw[q] = 0;
+    auto count_of = [&](uint32_t k, uint32_t i) { return (cw[(k * KV + i) / 4] >> (8 * ((k * KV + i) % 4))) & 0xFFu; };
 #pragma unroll
     for (int j = 0; j < KP; ++j) {
-      uint32_t c[2];
+      // The counts of rounds 2 j and 2 j + 1, drawn for every virtual thread
+      // and masked a round at a time (a branch or a test around every draw
+      // costs more than the draws of the threads and rounds past the end).
+      uint32_t w[2] = {0, 0}, top = 0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint64_t r = static_cast<uint64_t>(g.round0) + rb0 + 2 * j + h;
+#pragma unroll
+        for (int i = 0; i < KV; ++i) {
+          uint32_t ci;
+          if (DIST == GGA_DIST_POISSON && tabled) {
+            const uint32_t u = splitmix_mix_hi(dv[i].state(r));
+            top = max(top, u);
+            ci = sh.thr.first_count(u);
+          } else {
+            ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r));
+          }
+          w[h] |= ci << (8 * i);
+        }
+      }
+      if (DIST == GGA_DIST_POISSON && tabled && top >= sh.thr.second) {
+        // A draw among the thresholds the table does not tell apart: all of
+        // this thread's draws of the two rounds again, threshold by threshold.
+        uint64_t both = 0;
+#pragma unroll 1
+        for (uint32_t q = 0; q < 2 * KV; ++q) {
+          const uint32_t h = q / KV, i = q % KV;
+          const uint64_t r = static_cast<uint64_t>(g.round0) + rb0 + 2 * j + h;
+          const uint32_t u = splitmix_mix_hi(RoundDraws(g.seed, gfirst + i).state(r));
+          uint32_t c = 0;
+          while (c < g.nthr && u >= sh.thr.thr[c]) ++c;
+          both |= static_cast<uint64_t>(c) << (32 * h + 8 * i);
+        }
+        w[0] = static_cast<uint32_t>(both);
+        w[1] = static_cast<uint32_t>(both >> 32);
+      }
+      uint32_t pk = 0;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint32_t k = 2 * j + h;
-        const uint64_t r = static_cast<uint64_t>(g.round0) + r0 + k;
-        uint32_t sum = 0;
-#pragma unroll
-        for (int i = 0; i < KV; ++i) {
-          // Drawn unconditionally and masked: a branch around every draw
-          // costs more than the draws of the threads and rounds past the end.
-          uint32_t ci;
-          if (DIST == GGA_DIST_POISSON && tabled) ci = sh.thr.count(g.nthr, splitmix_mix_hi(dv[i].state(r)));
-          else ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r));
-          if (!(k < kk && static_cast<uint32_t>(i) < nvt)) ci = 0;
-          if (KV > 1 && i < KV - 1) {
-            const int q = static_cast<int>(k) * (KV - 1) + i;
-            cw[KV > 1 ? q / 4 : 0] |= ci << (8 * (q % 4));
-          }
-          sum += ci;
-        }
-        c[h] = sum;
+        w[h] &= k < kk ? played : 0u;
+        cw[k * KV / 4] |= w[h] << (8 * (k * KV % 4));
+        pk |= (KV == 1 ? w[h] : __dp4a(w[h], 0x01010101u, 0u)) << (16 * h);
       }
-      pk[j] = c[0] | (c[1] << 16);
-      inc[j] = warp_incl_scan_u32(pk[j]);
-      if (lane == 31) sh.wt[j][warp] = inc[j];
+      const uint32_t inc = warp_incl_scan_u32(pk);
+      exw[j] = inc - pk;
+      if (lane == 31) sh.wt[j][warp] = inc;
     }
     __syncthreads();
+    if (kMarks) clear_marks(stage4, dirty, t0, NT);   // the last pass's write-out is over
     if (warp == 0) {
       uint32_t rb = 0;
 #pragma unroll
@@ -421,7 +625,11 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
           rb += tot >> 16;
         }
       }
-      if (lane == 0) {
+      if constexpr (C > 1) {
+        if (lane == 0) sh.rb[K] = rb;
+        rb = __shfl_sync(0xffffffffu, rb, 0);
+        if (lane < C) cluster_store(&sh.peer_total[par][rank], lane, rb);
+      } else if (lane == 0) {
         sh.rb[K] = rb;
         const uint64_t base = sh.base;
         const uint64_t rem = target - base;   // > 0 while the loop runs
@@ -449,113 +657,137 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
         v.sizes[l] = base + commit;
       }
     }
-    __syncthreads();   // synchronize(): the buckets exist before any write
-
-    const uint64_t base = sh.base;
-    const uint32_t commit = sh.commit;
-    const uint32_t shv = static_cast<uint32_t>(base & (VEC - 1));   // stage index = pass position + shv
-    const bool staged = commit + shv <= cap;
+    uint64_t base;     // position of this block's first element of the pass
+    uint32_t commit;   // elements of this block the pass keeps
+    uint64_t next;     // the LFVector's size after the pass
+    if constexpr (C > 1) {
+      cluster_barrier();   // every block's total is here; this block's scan too
+      const uint64_t size = sh.base, rem = target - size;
+      uint32_t pre = 0, sum = 0;
+#pragma unroll
+      for (uint32_t q = 0; q < C; ++q) {
+        const uint32_t tq = sh.peer_total[par][q];
+        if (q < rank) pre += tq;
+        sum += tq;
+      }
+      par ^= 1u;
+      const uint32_t kept = sum < rem ? sum : static_cast<uint32_t>(rem);
+      const uint32_t mine = sh.rb[K];
+      commit = pre >= kept ? 0u : min(mine, kept - pre);
+      base = size + pre;
+      next = size + kept;
+      const uint32_t nb = sh.nb;
+      const uint32_t need = kept ? buckets_for(next, v.log2B) : 0u;
+      bool full = false;
+      if (need > nb) {   // the same in every thread of the cluster
+        if (rank == 0 && t0 == 0) {
+          const uint32_t got = grow_buckets(v, l, nb, need);
+          v.nbuckets[l] = got;
+          for (uint32_t q = 0; q < C; ++q) cluster_store(&sh.peer_nb, q, got);
+        }
+        cluster_barrier();   // synchronize(): the buckets exist before any write
+        const uint32_t got = sh.peer_nb;
+        for (uint32_t i = nb + t0; i < got; i += NT) sh.tab[i] = __ldcg(bk + i);
+        full = got < need;
+        if (full) {          // keep the longest prefix of whole rounds that fits
+          const uint64_t capg = bucket_first(got, v.log2B);
+          uint32_t kf = 0;
+          while (kf < static_cast<uint32_t>(K) && base + sh.rb[kf + 1] <= capg) ++kf;
+          commit = base > capg ? 0u : min(commit, sh.rb[kf]);
+          if (t0 == 0) {
+            if (commit) atomicMax(reinterpret_cast<unsigned long long*>(v.sizes + l), base + commit);
+            if (rank == 0) latch_error(v.status, GGA_ERR_POOL_EXHAUSTED);
+          }
+        }
+        __syncthreads();     // the table is filled, and every thread has read sh.nb
+        if (t0 == 0) sh.nb = got;
+      }
+      if (t0 == 0) {         // read by the others after the stage's barrier
+        if (rank == 0 && !full) v.sizes[l] = next;
+        sh.stop = full ? 1 : (next >= target ? 2 : 0);
+      }
+    } else {
+      __syncthreads();   // synchronize(): the buckets exist before any write
+      base = sh.base;
+      commit = sh.commit;
+      next = base + commit;
+    }
+    // Stage index = pass position + shv.
+    const bool marked = kMarks && sh.rb[K] + static_cast<uint32_t>(base & (kGroup - 1)) <= mark_cap;
+    const uint32_t shv = static_cast<uint32_t>(base & ((marked ? kGroup : VEC) - 1));
+    const bool staged = !marked && commit + shv <= cap;
     // Fast path (block-uniform): the whole pass is kept and staged, so no
     // element needs the clipping test or the bucket math.
-    const bool whole = staged && commit == sh.rb[K];
+    const bool whole = !kMarks && staged && commit == sh.rb[K];
     typedef typename std::conditional<E == 4, uint32_t, uint64_t>::type V;
-    // Element m of virtual thread i in round k: va * gid + vb * round + vc * m
-    // (a 4-byte element keeps the low 32 bits, which 32-bit arithmetic gives
-    // exactly).
-    // The value parameters in registers: g may live in shared memory, where
-    // the stage stores below could alias it and force a reload per element.
-    const V va = static_cast<V>(g.va), vb = static_cast<V>(g.vb), vc = static_cast<V>(g.vc);
-    const V vr = va * static_cast<V>(gfirst) + vb * static_cast<V>(static_cast<uint64_t>(g.round0) + r0);
-    // Counts without a small bound, two virtual threads per thread (below):
-    // one store loop over the run of both.  (With four the switch points
-    // cost registers the kernels do not have.)
-    constexpr bool kMergedRun = KV == 2 && !(DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2);
-    if (whole) {
-      T* const st0 = stage + shv;
+    if (marked) {
 #pragma unroll
       for (int j = 0; j < KP; ++j) {
-        const uint32_t ex = sh.wt[j][warp] + inc[j] - pk[j];
+        const uint32_t ex = sh.wt[j][warp] + exw[j];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const uint32_t k = 2 * j + h;
-          T* st = st0 + sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
-          const uint32_t csum = (pk[j] >> (16 * h)) & 0xFFFFu;
-          const V v0 = vr + vb * static_cast<V>(k);
-          if (kMergedRun) {
-            // The thread's virtual threads own consecutive positions of the
-            // round, so their elements form one run of csum positions: one
-            // loop over the run, moving to the next virtual thread's values
-            // at its first position (an empty virtual thread's switch point
-            // equals the next one's, and the later switch wins).  One
-            // shared-memory store per warp iteration over the run, against
-            // one per iteration of each virtual thread's own loop.
-            uint32_t sw[KV > 1 ? KV - 1 : 1];
-            uint32_t acc = 0;
-#pragma unroll
-            for (int i = 0; i < KV - 1; ++i) {
-              const int q = static_cast<int>(k) * (KV - 1) + i;
-              acc += (cw[q / 4] >> (8 * (q % 4))) & 0xFFu;
-              sw[i] = acc;
-            }
-            V val = v0;
-            for (uint32_t m = 0; m < csum; ++m, val += vc) {
-#pragma unroll
-              for (int i = 0; i < KV - 1; ++i)
-                if (m == sw[i]) val = v0 + va * static_cast<V>(i + 1);
-              st[m] = gen_value<E>(val);
-            }
-            continue;
-          }
-          uint32_t before = 0;   // elements of the earlier virtual threads of this round
+          uint32_t si = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu) + shv;
 #pragma unroll
           for (int i = 0; i < KV; ++i) {
-            uint32_t c = csum - before;
-            if (KV > 1 && i < KV - 1) {
-              const int q = static_cast<int>(k) * (KV - 1) + i;
-              c = (cw[KV > 1 ? q / 4 : 0] >> (8 * (q % 4))) & 0xFFu;
-            }
-            before += c;
-            V val = v0 + va * static_cast<V>(i);
-            if (DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2) {
-              // At most two elements: predicated stores, no loop.
-              if (c > 0) st[0] = gen_value<E>(val);
-              if (max_count<DIST>() > 1 && c > 1) st[1] = gen_value<E>(val + vc);
-            } else {
-              for (uint32_t m = 0; m < c; ++m, val += vc) st[m] = gen_value<E>(val);
-            }
-            st += c;
+            const uint32_t c = count_of(k, i);
+            if (c) marks[si] = ((si + 1) << kMarkBits) + ((k << 10) + static_cast<uint32_t>(tfirst) + i);
+            si += c;
           }
         }
       }
     } else {
-      // A clipped or unstaged pass: element by element.
+      // Element m of virtual thread i in round k: va * gid + vb * round + vc * m
+      // (a 4-byte element keeps the low 32 bits, which 32-bit arithmetic gives
+      // exactly).
+      // The value parameters in registers: g may live in shared memory, where
+      // the stage stores below could alias it and force a reload per element.
+      const V va = static_cast<V>(g.va), vb = static_cast<V>(g.vb), vc = static_cast<V>(g.vc);
+      const V vr = va * static_cast<V>(gfirst) + vb * static_cast<V>(static_cast<uint64_t>(g.round0) + rb0);
+      if (whole) {
+        T* const st0 = stage + shv;
 #pragma unroll
-      for (int j = 0; j < KP; ++j) {
-        const uint32_t ex = sh.wt[j][warp] + inc[j] - pk[j];
+        for (int j = 0; j < KP; ++j) {
+          const uint32_t ex = sh.wt[j][warp] + exw[j];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t k = 2 * j + h;
-          uint32_t q = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
-          const uint32_t csum = (pk[j] >> (16 * h)) & 0xFFFFu;
-          uint32_t before = 0;
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t k = 2 * j + h;
+            T* st = st0 + sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
+            const V v0 = vr + vb * static_cast<V>(k);
 #pragma unroll
-          for (int i = 0; i < KV; ++i) {
-            uint32_t c = csum - before;
-            if (KV > 1 && i < KV - 1) {
-              const int qq = static_cast<int>(k) * (KV - 1) + i;
-              c = (cw[KV > 1 ? qq / 4 : 0] >> (8 * (qq % 4))) & 0xFFu;
+            for (int i = 0; i < KV; ++i) {
+              const uint32_t c = count_of(k, i);
+              V val = v0 + va * static_cast<V>(i);
+              // At most two elements: predicated stores, no loop.
+              store_shared_if<E>(st, gen_value<E>(val), c > 0);
+              if (max_count<DIST>() > 1) store_shared_if<E>(st + 1, gen_value<E>(val + vc), c > 1);
+              st += c;
             }
-            before += c;
-            V val = vr + va * static_cast<V>(i) + vb * static_cast<V>(k);
-            for (uint32_t m = 0; m < c; ++m, ++q, val += vc) {
-              if (q >= commit) continue;
-              if (staged) {
-                stage[q + shv] = gen_value<E>(val);
-              } else {
-                uint32_t bb;
-                uint64_t off;
-                bucket_of(base + q, v.log2B, bb, off);
-                reinterpret_cast<T*>(sh.tab[bb])[off] = gen_value<E>(val);
+          }
+        }
+      } else {
+        // A clipped or unstaged pass: element by element.
+#pragma unroll
+        for (int j = 0; j < KP; ++j) {
+          const uint32_t ex = sh.wt[j][warp] + exw[j];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t k = 2 * j + h;
+            uint32_t q = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
+#pragma unroll
+            for (int i = 0; i < KV; ++i) {
+              const uint32_t c = count_of(k, i);
+              V val = vr + va * static_cast<V>(i) + vb * static_cast<V>(k);
+              for (uint32_t m = 0; m < c; ++m, ++q, val += vc) {
+                if (q >= commit) continue;
+                if (staged) {
+                  stage[q + shv] = gen_value<E>(val);
+                } else {
+                  uint32_t bb;
+                  uint64_t off;
+                  bucket_of(base + q, v.log2B, bb, off);
+                  reinterpret_cast<T*>(sh.tab[bb])[off] = gen_value<E>(val);
+                }
               }
             }
           }
@@ -563,15 +795,25 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
       }
     }
     __syncthreads();
-    if (staged && commit) stage_to_buckets<T>(sh.tab, v.log2B, v.B, base, commit, shv, stage4, t0, NT);
+    if (marked) {
+      dirty = sh.rb[K] + shv;
+      if (commit)
+        marks_to_buckets<E, V>(sh.tab, v.log2B, base, commit, shv, marks,
+                               static_cast<V>(g.va * (static_cast<uint64_t>(l) * v.T) +
+                                              g.vb * (static_cast<uint64_t>(g.round0) + rb0)),
+                               static_cast<V>(g.va), static_cast<V>(g.vb), static_cast<V>(g.vc), t0, NT);
+    } else {
+      dirty = staged ? (commit + shv) * (E / 4) : 0u;
+      if (staged && commit) stage_to_buckets<T>(sh.tab, v.log2B, v.B, base, commit, shv, stage4, t0, NT);
+    }
     // No barrier here: the next pass writes the stage, sh.wt, sh.rb and
     // sh.commit only after its first two barriers, which every thread reaches
     // after finishing this pass; sh.base is written by thread 0 and read by
     // thread 0 (the leader) before the next pass's second barrier and by the
     // others after it; sh.stop was set before this pass's second barrier;
     // sh.tab only gains entries past those this pass reads.
-    if (t0 == 0) sh.base = base + commit;
-    r0 += kk;
+    if (t0 == 0) sh.base = next;
+    r0 = R - r0 > static_cast<uint32_t>(C * K) ? r0 + C * K : R;
   }
   *done = sh.stop != 0;
   __syncthreads();   // the caller may reuse the stage and sh

@@ -797,33 +797,27 @@ int launch_finalize(const ArrayView& v, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // In-kernel generated insertion.
 
-// A pass's values are staged in shared memory (a pass averages 16 KB at
-// K = 8 rounds, 512 threads, one int32 per thread and round; a pass that
-// does not fit writes directly).  T in (256, 512] is played by blocks of
-// T / GGA_GEN_VT threads, GGA_GEN_VT virtual threads each (one scan word
-// and one share of every barrier serve them), GGA_GEN_MINB_VT resident per
-// SM with a GGA_GEN_STAGE_VT-byte stage: measured on GB300 for the
-// paper-shaped workload (1024 LFVectors x 512 threads x 512 rounds, int32),
-// 128 threads x 4, 8 per SM: 0.737 ms (0.545 ms since the draws are branch-free
-// and the write-out does its bucket math per bucket); 256 x 2, 4 per SM: 0.753 ms; 512 x 1,
-// 3 per SM (40 registers, 48 KB stage): 0.816 ms.  Other T use one virtual
-// thread per thread, blocks of up to 512 threads 3 per SM (up to 1024: 1).
-#ifndef GGA_GEN_VT
-#define GGA_GEN_VT 4
-#endif
-#ifndef GGA_GEN_MINB_VT
-#define GGA_GEN_MINB_VT 8
-#endif
-#ifndef GGA_GEN_MINB512
-#define GGA_GEN_MINB512 3
-#endif
-#ifndef GGA_GEN_STAGE_VT
-#define GGA_GEN_STAGE_VT 24576
-#endif
-constexpr uint32_t kGenStageBytes = 49152;
-constexpr uint32_t kGenStageBytesVT = GGA_GEN_STAGE_VT;
+// A pass's elements (or marks) are staged in shared memory, its rounds
+// chosen so that at one element per thread and round a pass fills about
+// two thirds of the stage; a pass that does not fit writes directly, element
+// by element, which costs twice the instructions (8-byte uniform counts at 8
+// rounds in a 24 KB stage: 126 per draw and 250 us for 2^25 draws, at 4
+// rounds 87 us).  T > 256 is played by blocks of T / 4 threads, four
+// virtual threads each: one scan word and one share of every barrier serve
+// them, and eight blocks (four for T > 512) are resident per SM.  Measured
+// on GB300 for the paper-shaped workload (1024 LFVectors x 512 threads x 512
+// rounds, int32) when this was chosen: 128 threads x 4, 8 per SM: 0.737 ms
+// (0.47 ms now); 256 x 2, 4 per SM: 0.753 ms; 512 x 1, 3 per SM (40
+// registers, 48 KB stage): 0.816 ms.  Other T use one virtual thread per
+// thread and a stage sized by T, so that small blocks fill the SM.
+constexpr int kGenVT = 4;
 
-template <int E> struct GenK { static constexpr int value = E == 16 ? 4 : 8; };
+// Rounds per pass: counts without a small bound stage 4-byte marks.
+template <int E, int DIST>
+struct GenRounds {
+  static constexpr bool kMarks = max_count<DIST>() == 0;
+  static constexpr int value = E == 4 ? 8 : (kMarks ? (E == 8 ? 8 : 4) : (E == 8 ? 4 : 2));
+};
 
 // One block per LFVector, R rounds in passes of K (grow_passes in
 // gga_gen.cuh), with no target.
@@ -837,44 +831,47 @@ __global__ void __launch_bounds__(MAXT, MINB) gen_insert_kernel(const __grid_con
   grow_passes<E, K, KV, false, DIST>(v, g, blockIdx.x, R, ~0ull, sh, s_stage4, stage_bytes / E, &done);
 }
 
+template <int E, int DIST>
+static void launch_gen_as(const ArrayView& v, const GenParams& g, uint32_t R, cudaStream_t st) {
+  constexpr int K = GenRounds<E, DIST>::value;
+  const bool vt = v.T > 256;
+  const uint32_t per = vt ? kGenVT : 1;
+  const uint32_t nt = ((v.T + per - 1) / per + 31) / 32 * 32;
+  // A pass of one element per thread and round and a quarter more, in
+  // whole 16-byte words, and a warp's overhang (41,984 bytes at most; eight
+  // blocks of T = 512 fit an SM).
+  const uint32_t esize = GenRounds<E, DIST>::kMarks ? 4 : E;
+  const size_t smem = (static_cast<size_t>(K) * v.T * esize * 5 / 4 + 1024 + 15) & ~static_cast<size_t>(15);
+#define GGA_GEN(KV, MT, MB)                                                                                  \
+  do {                                                                                                       \
+    auto kern = gen_insert_kernel<E, K, KV, MT, MB, DIST>;                                                   \
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));         \
+    kern<<<v.L, nt, smem, st>>>(v, g, R, static_cast<uint32_t>(smem));                                       \
+  } while (0)
+  if (!vt) GGA_GEN(1, 256, 6);
+  else if (v.T <= 512) GGA_GEN(kGenVT, 128, 8);
+  else GGA_GEN(kGenVT, 256, 4);
+#undef GGA_GEN
+}
+
+template <int E>
+static void launch_gen(const ArrayView& v, const GenParams& g, uint32_t R, cudaStream_t st) {
+  // The count distribution is a template argument: the draw loop then has
+  // no per-draw dispatch.
+  switch (g.dist) {
+    case GGA_DIST_BERNOULLI: launch_gen_as<E, GGA_DIST_BERNOULLI>(v, g, R, st); break;
+    case GGA_DIST_UNIFORM3: launch_gen_as<E, GGA_DIST_UNIFORM3>(v, g, R, st); break;
+    case GGA_DIST_GEOMETRIC: launch_gen_as<E, GGA_DIST_GEOMETRIC>(v, g, R, st); break;
+    default: launch_gen_as<E, GGA_DIST_POISSON>(v, g, R, st); break;
+  }
+}
+
 int launch_insert_generated(const ArrayView& v, const gga_gen_spec& spec, uint32_t R, uint32_t* /*done*/,
                             int /*num_sms*/, cudaStream_t st) {
   const GenParams g = make_gen_params(spec);
-  const bool vt = GGA_GEN_VT > 1 && v.T > 256 && v.T <= 512;
-  const uint32_t NT = vt ? ((v.T + GGA_GEN_VT - 1) / GGA_GEN_VT + 31) / 32 * 32 : (v.T + 31) / 32 * 32;
-  const size_t smem = vt ? kGenStageBytesVT : kGenStageBytes;
-#define GGA_GEN_AD(EE, KK, KV, MT, MB, DD)                                                                   \
-  do {                                                                                                       \
-    cudaFuncSetAttribute(gen_insert_kernel<EE, KK, KV, MT, MB, DD>,                                          \
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));               \
-    gen_insert_kernel<EE, KK, KV, MT, MB, DD><<<v.L, NT, smem, st>>>(v, g, R, static_cast<uint32_t>(smem));   \
-  } while (0)
-  // The count distribution is a template argument: the draw loop then has
-  // no per-draw dispatch.
-#define GGA_GEN_AS(EE, KK, KV, MT, MB)                                                                       \
-  do {                                                                                                       \
-    switch (g.dist) {                                                                                        \
-      case GGA_DIST_BERNOULLI: GGA_GEN_AD(EE, KK, KV, MT, MB, GGA_DIST_BERNOULLI); break;                    \
-      case GGA_DIST_UNIFORM3: GGA_GEN_AD(EE, KK, KV, MT, MB, GGA_DIST_UNIFORM3); break;                      \
-      case GGA_DIST_GEOMETRIC: GGA_GEN_AD(EE, KK, KV, MT, MB, GGA_DIST_GEOMETRIC); break;                    \
-      default: GGA_GEN_AD(EE, KK, KV, MT, MB, GGA_DIST_POISSON); break;                                      \
-    }                                                                                                        \
-  } while (0)
-  // Rounds per pass: a pass then averages <= 32 KB at one element per thread
-  // and round (K halves for blocks of more than 512 threads beyond 4 bytes).
-#define GGA_GEN(EE)                                                                                          \
-  do {                                                                                                       \
-    if (vt) GGA_GEN_AS(EE, GenK<EE>::value, (GGA_GEN_VT > 1 ? GGA_GEN_VT : 2), 512 / (GGA_GEN_VT > 1 ? GGA_GEN_VT : 2),   \
-                       GGA_GEN_MINB_VT);                                                                     \
-    else if (NT <= 512) GGA_GEN_AS(EE, GenK<EE>::value, 1, 512, GGA_GEN_MINB512);                            \
-    else GGA_GEN_AS(EE, (EE == 4 ? 8 : GenK<EE>::value / 2), 1, 1024, 1);                                    \
-  } while (0)
-  if (v.E == 4) GGA_GEN(4);
-  else if (v.E == 8) GGA_GEN(8);
-  else GGA_GEN(16);
-#undef GGA_GEN
-#undef GGA_GEN_AS
-#undef GGA_GEN_AD
+  if (v.E == 4) launch_gen<4>(v, g, R, st);
+  else if (v.E == 8) launch_gen<8>(v, g, R, st);
+  else launch_gen<16>(v, g, R, st);
   finalize_kernel<<<1, 1024, 0, st>>>(v);
   return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }

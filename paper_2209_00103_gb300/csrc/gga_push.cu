@@ -95,21 +95,21 @@ template <int E>
 void launch_push_generated_as(const ArrayView& v, const ArrayView* dview, const GenParams& g, uint32_t rounds,
                               cudaStream_t st) {
   const uint32_t nt = ((v.T + kPushSlots - 1) / kPushSlots + 31) / 32 * 32;
-  const uint32_t smem = 2 * push_half_elems(v.T, E) * E;   // two halves: at most 43 KB (T = 1024, 16-byte elements)
+  const uint32_t smem = 2 * push_half_elems(v.T, E) * E;   // two halves: at most 44 KB (T = 1024, 16-byte elements)
+#define GGA_PUSH(D)                                                                                         \
+  do {                                                                                                      \
+    auto kern = push_generated_kernel<E, D>;                                                                \
+    if (smem > 32768u)   /* with the count table the block's shared memory may pass 48 KB */                \
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));      \
+    kern<<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);                                               \
+  } while (0)
   switch (g.dist) {
-    case GGA_DIST_BERNOULLI:
-      push_generated_kernel<E, GGA_DIST_BERNOULLI><<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);
-      break;
-    case GGA_DIST_UNIFORM3:
-      push_generated_kernel<E, GGA_DIST_UNIFORM3><<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);
-      break;
-    case GGA_DIST_GEOMETRIC:
-      push_generated_kernel<E, GGA_DIST_GEOMETRIC><<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);
-      break;
-    default:
-      push_generated_kernel<E, GGA_DIST_POISSON><<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);
-      break;
+    case GGA_DIST_BERNOULLI: GGA_PUSH(GGA_DIST_BERNOULLI); break;
+    case GGA_DIST_UNIFORM3: GGA_PUSH(GGA_DIST_UNIFORM3); break;
+    case GGA_DIST_GEOMETRIC: GGA_PUSH(GGA_DIST_GEOMETRIC); break;
+    default: GGA_PUSH(GGA_DIST_POISSON); break;
   }
+#undef GGA_PUSH
 }
 
 int launch_push_generated(const ArrayView& v, const ArrayView* dview, const gga_gen_spec& spec, uint32_t rounds,
