@@ -279,7 +279,14 @@ int gga_push_expand(gga_handle h, const uint32_t* counts_dev, const void* inputs
  * the proportional guess i * L / N --, then the bucket and offset of the
  * LFVector-local index).  idx_dev: uint64 [n], 8-byte aligned; out_dev: n
  * elements of E bytes.  An index >= size latches GGA_ERR_OUT_OF_RANGE and
- * its output element is zeroed.
+ * its output element is zeroed.  A batch of 2^25 reads or more of 4- or
+ * 8-byte elements, from a slab of 512 MB or more and at most 48 bytes per
+ * read, is grouped by ranges of global indices first (the values come back in
+ * the order of idx_dev).  That takes 6.4 bytes (E = 8: 14.4) of
+ * device memory per read during the call, stream-ordered, from a pool of the
+ * library that keeps up to 1 GB between calls while any handle of the device
+ * lives; without that memory, and while `stream` is captured, the batch is
+ * read directly.
  */
 int gga_read(gga_handle h, const uint64_t* idx_dev, uint64_t n, void* out_dev, void* stream);
 

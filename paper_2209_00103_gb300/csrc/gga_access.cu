@@ -412,6 +412,363 @@ __global__ void __launch_bounds__(kWbinThreads) wbin_apply_kernel(ArrayView v, c
 }
 
 // ---------------------------------------------------------------------------
+// Binned random reads (large batches into large arrays).
+//
+// A random read of an array far larger than the L2 is one DRAM access, and
+// the rate of those bounds the direct kernel (48 G reads/s on GB300, 1.38 ms
+// for 2^26 of 1.07 GB) while the bytes would take a seventh of that.  As for
+// the writes, a large batch is therefore grouped by ranges of global indices
+// and read range by range, each range streamed into L2 ahead of its reads;
+// the values then go back to their places through the tiles they came from:
+//   count:   per-bin totals; a tile whose indices are local (a sorted batch,
+//            a window) is read here, directly, and takes no further part
+//   scan:    bin cursors (wbin_scan_kernel)
+//   scatter: a tile's indices, 32 bits each, sorted by bin in shared memory
+//            go to the bins, and the tile keeps where its runs lie and each
+//            sorted index's place in the tile
+//   apply:   every index is replaced by the element it names (8-byte elements:
+//            written beside it), bins ahead prefetched into L2
+//   return:  a tile gathers its runs, sorts the elements back in shared
+//            memory and writes them out
+// Per read 16 bytes of indices, 4 of places, 8 of 32-bit indices and 3 E of
+// elements, all in streams, plus the array once.  Measured on GB300 for 2^26
+// int32 reads of 1.07 GB: 0.89 ms (count 0.09, scatter 0.21, apply 0.39, return
+// 0.18) against 1.38 direct.
+
+// Which batches: 4- and 8-byte elements, 2^25 reads and more, a slab of 512
+// MB and more, at most 48 bytes of it per read (the array's size is on the
+// device; the slab's bounds it).  Measured on GB300, direct / binned (us),
+// uniform indices: 2^26 reads of 1.07 GB 1385 / 890 (int32), 1436 / 1010
+// (int64), 1489 / 1511 (records: their values move 48 bytes per read, so they
+// are read directly); 2^25 reads of 1.07 GB 700 / 577, of 4.2 GB 748 / 882;
+// 2^24 of 1.07 GB 359 / 403; 2^26 of 0.27 GB 1045 / 1019.  A sorted batch, read
+// directly by the count: 305 / 317; indices within a window of 2 MB that
+// moves over the array: 525 / 403.
+constexpr uint64_t kRbinMin = 1ull << 25;
+constexpr uint64_t kRbinMax = 1ull << 30;         // (run places are 32 bits)
+constexpr uint64_t kRbinSlabMin = 512ull << 20;
+constexpr uint64_t kRbinBytesPerRead = 48;
+constexpr uint64_t kRbinArrayMin = 192ull << 20;  // arrays the L2 (129 MB) mostly holds: direct, decided on the device
+
+constexpr uint64_t kRbinTilesPerBlock = 2;        // scatter and return (1: 2% faster, but a sorted batch, with no tile left
+                                                  // to do, pays 22 us for empty blocks instead of 12)
+constexpr int kRbinApplyThreads = 512;
+constexpr int kRbinApplyPer = 8;                   // reads per thread of the apply
+constexpr int kRbinPer = 16;                      // indices per thread of a tile
+constexpr uint64_t kRbinTile = static_cast<uint64_t>(kWbinThreads) * kRbinPer;
+
+// Workspace of a binned read: the header of the binned writes, then per
+// tile its runs (first place in the tile: 16 bits, first place in the bins: 32)
+// and whether it was read directly, per read its place in its tile, offset
+// and (8- and 16-byte elements) element.
+struct RbinScratch {
+  uint8_t* head;
+  uint32_t* run_at;     // [tiles][256]
+  uint16_t* run_off;    // [tiles][256]
+  uint16_t* valid;      // [tiles] indices in range
+  uint8_t* direct;      // [tiles]
+  uint16_t* place;      // [tiles][tile]
+  uint32_t* off;        // [n]
+  uint8_t* val;         // [n] elements (E = 4: the offsets' array)
+};
+
+template <int E>
+static uint64_t rbin_layout(uint64_t n, uint8_t* base, RbinScratch* s) {
+  const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
+  uint64_t at = kWbinHeader;
+  auto take = [&](uint64_t bytes) {
+    const uint64_t a = at;
+    at = (at + bytes + 255) & ~255ull;
+    return base + a;
+  };
+  RbinScratch r;
+  r.head = base;
+  r.run_at = reinterpret_cast<uint32_t*>(take(tiles * kWbinMaxBins * 4));
+  r.run_off = reinterpret_cast<uint16_t*>(take(tiles * kWbinMaxBins * 2));
+  r.valid = reinterpret_cast<uint16_t*>(take(tiles * 2));
+  r.direct = take(tiles);
+  r.place = reinterpret_cast<uint16_t*>(take(tiles * kRbinTile * 2));
+  r.off = reinterpret_cast<uint32_t*>(take(n * 4));
+  r.val = E == 4 ? reinterpret_cast<uint8_t*>(r.off) : take(n * E);
+  if (s) *s = r;
+  return at;
+}
+
+// Bin of global index g: g >> shift, bins of ~4 MB (2^26 reads of 1.07 GB: 940
+// us, with the writes' 8 MB 961), at most kWbinMaxBins of them.
+__device__ __forceinline__ uint32_t rbin_shift(uint64_t N, uint32_t E) {
+  uint32_t s = 22 - (31 - __clz(static_cast<int>(E)));
+  while (N > 0 && ((N - 1) >> s) >= kWbinMaxBins) ++s;
+  return s;
+}
+
+template <int E>
+__global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, const uint64_t* __restrict__ idx,
+                                                                  uint64_t n, RbinScratch s,
+                                                                  typename Elem<E>::T* __restrict__ out) {
+  typedef typename Elem<E>::T T;
+  constexpr int kPer = kRbinPer;
+  __shared__ uint32_t h[kWbinMaxBins];
+  const uint64_t N = __ldg(v.offsets + v.L);
+  const uint32_t shift = rbin_shift(N, E);
+  // Arrays that the L2 mostly holds are read directly, and those of 2^32
+  // elements and more (the bins hold 32-bit indices).
+  const bool never = N * E < kRbinArrayMin || N > 0xFFFFFFFFull;
+  for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x) h[b] = 0;
+  bool bad = false;
+  const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
+  for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const uint64_t base = tile * kRbinTile;
+    uint64_t g[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint64_t i = base + static_cast<uint64_t>(u) * kWbinThreads + threadIdx.x;
+      g[u] = i < n ? __ldcs(idx + i) : ~0ull;
+    }
+    // Local, by a sample of the tile: most indices lie within 128 bytes of
+    // their neighbour (they share sectors), or in the first one's bin or the
+    // next to it (they stay in L2 without being sorted).
+    const uint64_t d = g[kPer / 2] - __shfl_up_sync(0xffffffffu, g[kPer / 2], 1) + 128 / E;
+    const uint64_t db = (g[kPer / 2] >> shift) - (__ldg(idx + base) >> shift) + 1;
+    const bool near = ((threadIdx.x & 31) != 0 && d <= 2 * (128 / E)) || db <= 2;
+    const bool direct = __syncthreads_count(near) * 2 > kWbinThreads || never;
+    if (threadIdx.x == 0) s.direct[tile] = direct ? 1 : 0;
+    if (direct) {
+      T x[kPer];
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const uint64_t i = base + static_cast<uint64_t>(u) * kWbinThreads + threadIdx.x;
+        x[u] = T();
+        if (g[u] < N) x[u] = *reinterpret_cast<const T*>(element_addr(v, N, g[u]));
+        else if (i < n) bad = true;
+      }
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const uint64_t i = base + static_cast<uint64_t>(u) * kWbinThreads + threadIdx.x;
+        if (i < n) __stcs(out + i, x[u]);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        if (g[u] < N) atomicAdd(&h[static_cast<uint32_t>(g[u] >> shift)], 1u);
+        else if (base + static_cast<uint64_t>(u) * kWbinThreads + threadIdx.x < n) bad = true;
+      }
+    }
+  }
+  if (bad) latch_error(v.status, GGA_ERR_OUT_OF_RANGE);
+  __syncthreads();
+  uint32_t* tot = wbin_totals(s.head);
+  for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x)
+    if (h[b]) atomicAdd(tot + b, h[b]);
+}
+
+template <int E>
+__global__ void __launch_bounds__(kWbinThreads, 4) rbin_scatter_kernel(ArrayView v, const uint64_t* __restrict__ idx,
+                                                                    uint64_t n, RbinScratch s) {
+  constexpr int kPer = kRbinPer;
+  constexpr uint32_t kTile = kWbinThreads * kPer;
+  __shared__ uint32_t h[kWbinMaxBins];
+  __shared__ uint32_t off[kWbinMaxBins];
+  __shared__ uint32_t at[kWbinMaxBins];   // the run's place in the bins, less its place in the tile
+  __shared__ uint32_t wsum[kWbinThreads / 32];
+  __shared__ uint32_t s_off[kTile];
+  __shared__ alignas(16) uint16_t s_place[kTile];
+  const uint64_t N = __ldg(v.offsets + v.L);
+  const uint32_t shift = rbin_shift(N, E);
+  const uint64_t tiles = *wbin_valid(s.head) ? (n + kTile - 1) / kTile : 0;   // none when all were read directly
+  for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    if (s.direct[tile]) continue;   // block-uniform
+    for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x) h[b] = 0;
+    __syncthreads();
+    const uint64_t base = tile * kTile;
+    uint64_t g[kPer];
+    uint32_t rank[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint64_t i = base + static_cast<uint64_t>(u) * kWbinThreads + threadIdx.x;
+      g[u] = i < n ? __ldcs(idx + i) : ~0ull;
+      if (g[u] >= N) g[u] = ~0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+      rank[u] = g[u] != ~0ull ? atomicAdd(&h[static_cast<uint32_t>(g[u] >> shift)], 1u) : 0u;
+    __syncthreads();
+    {
+      // Exclusive scan of the tile's bin counts (one bin per thread) and one
+      // reservation per non-empty bin in the bins.
+      const uint32_t c = h[threadIdx.x];
+      const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+      uint32_t sc = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, sc, o);
+        if (lane >= o) sc += t;
+      }
+      if (lane == 31) wsum[w] = sc;
+      const uint32_t to = c ? static_cast<uint32_t>(atomicAdd(wbin_cursors(s.head) + threadIdx.x,
+                                                              static_cast<unsigned long long>(c)))
+                            : 0u;
+      __syncthreads();
+      uint32_t add = 0;
+      for (int k = 0; k < w; ++k) add += wsum[k];
+      const uint32_t o = sc - c + add;
+      off[threadIdx.x] = o;
+      at[threadIdx.x] = to - o;
+      s.run_at[tile * kWbinMaxBins + threadIdx.x] = to - o;
+      s.run_off[tile * kWbinMaxBins + threadIdx.x] = static_cast<uint16_t>(o);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      if (g[u] == ~0ull) continue;
+      const uint32_t b = static_cast<uint32_t>(g[u] >> shift);
+      const uint32_t p = off[b] + rank[u];
+      s_off[p] = static_cast<uint32_t>(g[u]);
+      s_place[p] = static_cast<uint16_t>(u * kWbinThreads + threadIdx.x);
+    }
+    __syncthreads();
+    const uint32_t valid = off[kWbinMaxBins - 1] + h[kWbinMaxBins - 1];
+    if (threadIdx.x == 0) s.valid[tile] = static_cast<uint16_t>(valid);
+    for (uint32_t p = threadIdx.x; p < valid; p += blockDim.x) {
+      const uint32_t o = s_off[p];
+      s.off[at[o >> shift] + p] = o;
+    }
+    for (uint32_t p = 2 * threadIdx.x; p < valid; p += 2 * blockDim.x)   // two places a store (the last may be stale)
+      *reinterpret_cast<uint32_t*>(s.place + tile * kTile + p) = *reinterpret_cast<const uint32_t*>(s_place + p);
+    __syncthreads();   // the tile's shared arrays are read before the next tile fills them
+  }
+}
+
+// Address of global element g < N < 2^32 for the apply kernels, which take g
+// from 32-bit bins: element_addr in 32-bit arithmetic where the positions
+// allow (`scale` = L / N; the search starts from the same proportional guess).
+template <int E>
+__device__ __forceinline__ uint64_t element_addr_32(const ArrayView& v, uint64_t N, float scale, uint32_t g) {
+  uint32_t l = __float2uint_rz(__uint2float_rz(g) * scale);
+  if (l >= v.L) l = v.L - 1;
+  uint64_t lo = __ldg(v.offsets + l), hi = __ldg(v.offsets + l + 1);
+  if (g < lo || g >= hi) {
+    l = find_lfv(v.offsets, v.L, N, g);
+    lo = __ldg(v.offsets + l);
+  }
+  const uint64_t x = static_cast<uint64_t>(g - static_cast<uint32_t>(lo)) + (1ull << v.log2B);
+  const uint32_t hb = 63u - static_cast<uint32_t>(__clzll(static_cast<long long>(x)));
+  return __ldg(v.buckets + static_cast<uint64_t>(l) * kMaxBuckets + (hb - v.log2B)) + (x - (1ull << hb)) * E;
+}
+
+// Prefetches of the tile of positions [t0, t1) of an apply kernel, by warp 0:
+// see kWbinAheadBytes.
+template <int E>
+__device__ __forceinline__ void apply_prefetch(const ArrayView& v, uint64_t N, uint32_t shift, uint32_t nbins,
+                                               const unsigned long long* ends, uint64_t t0, uint64_t t1,
+                                               uint32_t block) {
+  const uint64_t bin_bytes = static_cast<uint64_t>(E) << shift;
+  const uint32_t ahead = bin_bytes >= kWbinAheadBytes ? 1u : static_cast<uint32_t>(kWbinAheadBytes / bin_bytes);
+  // Blocks 0 .. ahead - 1 fetch the first bins, one each.
+  if (block < ahead && block < nbins)
+    prefetch_range_l2_warp<E>(v, N, static_cast<uint64_t>(block) << shift,
+                              min(static_cast<uint64_t>(block + 1) << shift, N));
+  // First bin starting at or after t0 (bin starts ascend): binary search.
+  uint32_t lo = 0, hi = nbins;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if ((mid ? ends[mid - 1] : 0) < t0) lo = mid + 1;
+    else hi = mid;
+  }
+  for (uint32_t b = lo; b < nbins; ++b) {
+    const uint64_t start = b ? ends[b - 1] : 0;
+    if (start >= t1) break;
+    const uint32_t pb = b + ahead;   // this tile holds bin b's first access
+    if (ends[b] != start && pb < nbins)
+      prefetch_range_l2_warp<E>(v, N, static_cast<uint64_t>(pb) << shift, min(static_cast<uint64_t>(pb + 1) << shift, N));
+  }
+}
+
+template <int E>
+__global__ void __launch_bounds__(kRbinApplyThreads) rbin_apply_kernel(ArrayView v, RbinScratch s) {
+  typedef typename Elem<E>::T T;
+  constexpr int kPer = kRbinApplyPer;
+  const uint64_t total = *wbin_valid(s.head);
+  const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kRbinApplyThreads * kPer;
+  if (base >= total) return;
+  const uint64_t N = __ldg(v.offsets + v.L);   // > 0: some read was binned
+  const uint32_t shift = rbin_shift(N, E);
+  const uint32_t nbins = static_cast<uint32_t>(((N - 1) >> shift) + 1);
+  const unsigned long long* ends = wbin_cursors(s.head);   // advanced to the bin ends by the scatter
+  if (threadIdx.x < 32)
+    apply_prefetch<E>(v, N, shift, nbins, ends, base, base + kRbinApplyThreads * kPer, blockIdx.x);
+  uint32_t o[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const uint64_t i = base + static_cast<uint64_t>(u) * kRbinApplyThreads + threadIdx.x;
+    o[u] = i < total ? __ldcs(s.off + i) : 0u;
+  }
+  uint64_t addr[kPer];
+  const float scale = static_cast<float>(v.L) / __ull2float_rz(N);
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const uint64_t i = base + static_cast<uint64_t>(u) * kRbinApplyThreads + threadIdx.x;
+    addr[u] = i < total ? element_addr_32<E>(v, N, scale, o[u]) : 0;
+  }
+  T x[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u)
+    if (addr[u]) x[u] = *reinterpret_cast<const T*>(addr[u]);
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const uint64_t i = base + static_cast<uint64_t>(u) * kRbinApplyThreads + threadIdx.x;
+    if (addr[u]) __stcs(reinterpret_cast<T*>(s.val) + i, x[u]);
+  }
+}
+
+template <int E>
+__global__ void __launch_bounds__(kWbinThreads, 6) rbin_return_kernel(RbinScratch s, uint64_t n,
+                                                                   typename Elem<E>::T* __restrict__ out) {
+  typedef typename Elem<E>::T T;
+  constexpr int kPer = kRbinPer;
+  constexpr uint32_t kTile = kWbinThreads * kPer;
+  extern __shared__ __align__(16) uint8_t s_dyn[];
+  T* s_out = reinterpret_cast<T*>(s_dyn);                                  // [kTile]
+  uint8_t* s_bin = s_dyn + static_cast<size_t>(kTile) * E;                 // [kTile]
+  __shared__ uint32_t at[kWbinMaxBins];
+  __shared__ uint16_t off[kWbinMaxBins];
+  const uint64_t tiles = *wbin_valid(s.head) ? (n + kTile - 1) / kTile : 0;   // none when all were read directly
+  for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    if (s.direct[tile]) continue;   // block-uniform
+    const uint64_t base = tile * kTile;
+    const uint32_t m = static_cast<uint32_t>(n - base < kTile ? n - base : kTile);
+    const uint32_t valid = s.valid[tile];   // out-of-range indices are in no run
+    at[threadIdx.x] = s.run_at[tile * kWbinMaxBins + threadIdx.x];
+    off[threadIdx.x] = s.run_off[tile * kWbinMaxBins + threadIdx.x];
+    uint32_t place[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) place[u] = s.place[base + u * kWbinThreads + threadIdx.x];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) s_out[u * kWbinThreads + threadIdx.x] = T();   // out-of-range reads: zero
+    __syncthreads();
+    const uint32_t end = threadIdx.x + 1 < kWbinMaxBins ? off[threadIdx.x + 1] : valid;
+    for (uint32_t p = off[threadIdx.x]; p < end; ++p) s_bin[p] = static_cast<uint8_t>(threadIdx.x);
+    __syncthreads();
+    T x[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint32_t p = u * kWbinThreads + threadIdx.x;
+      if (p < valid) x[u] = reinterpret_cast<const T*>(s.val)[at[s_bin[p]] + p];
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+      if (u * kWbinThreads + threadIdx.x < valid) s_out[place[u]] = x[u];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint32_t p = u * kWbinThreads + threadIdx.x;
+      if (p < m) __stcs(out + base + p, s_out[p]);
+    }
+    __syncthreads();   // the tile's shared arrays are read before the next tile fills them
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Sweeps.
 
 template <int E>
@@ -815,6 +1172,38 @@ static void write_as(const ArrayView& v, const uint64_t* idx, uint64_t n, const 
   const uint64_t tiles_a = (n + kTileA - 1) / kTileA;
   const unsigned grid_a = static_cast<unsigned>(tiles_a > 0x7FFFFFFFull ? 0x7FFFFFFFull : tiles_a);
   wbin_apply_kernel<E><<<grid_a, kWbinThreads, 0, st>>>(v, out_off, out_val, scr);
+}
+
+template <int E>
+static void read_binned_as(const ArrayView& v, const uint64_t* idx, uint64_t n, void* out, void* scratch, int num_sms,
+                           cudaStream_t st) {
+  typedef typename Elem<E>::T T;
+  RbinScratch s;
+  rbin_layout<E>(n, static_cast<uint8_t*>(scratch), &s);
+  cudaMemsetAsync(s.head, 0, 1024, st);   // the totals
+  const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
+  const uint64_t cap = static_cast<uint64_t>(num_sms) * 4;   // the count: persistent blocks, one set of global additions each
+  rbin_count_kernel<E><<<static_cast<unsigned>(tiles < cap ? tiles : cap), kWbinThreads, 0, st>>>(v, idx, n, s, static_cast<T*>(out));
+  wbin_scan_kernel<<<1, kWbinMaxBins, 0, st>>>(s.head);
+  rbin_scatter_kernel<E><<<static_cast<unsigned>((tiles + kRbinTilesPerBlock - 1) / kRbinTilesPerBlock), kWbinThreads, 0, st>>>(v, idx, n, s);
+  constexpr uint64_t kTileA = static_cast<uint64_t>(kRbinApplyThreads) * kRbinApplyPer;
+  rbin_apply_kernel<E><<<static_cast<unsigned>((n + kTileA - 1) / kTileA), kRbinApplyThreads, 0, st>>>(v, s);
+  const int smem = static_cast<int>(kRbinTile * (E + 1));
+  cudaFuncSetAttribute(rbin_return_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  rbin_return_kernel<E><<<static_cast<unsigned>((tiles + kRbinTilesPerBlock - 1) / kRbinTilesPerBlock), kWbinThreads, smem, st>>>(s, n, static_cast<T*>(out));
+}
+
+uint64_t rbin_scratch_bytes(uint64_t n, uint32_t E, uint64_t slab_bytes) {
+  if (E > 8 || n < kRbinMin || n > kRbinMax || slab_bytes < kRbinSlabMin || slab_bytes / kRbinBytesPerRead > n)
+    return 0;
+  return E == 4 ? rbin_layout<4>(n, nullptr, nullptr) : rbin_layout<8>(n, nullptr, nullptr);
+}
+
+int launch_read_binned(const ArrayView& v, const uint64_t* idx, uint64_t n, void* out, void* scratch, int num_sms,
+                       cudaStream_t st) {
+  if (v.E == 4) read_binned_as<4>(v, idx, n, out, scratch, num_sms, st);
+  else read_binned_as<8>(v, idx, n, out, scratch, num_sms, st);
+  return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 
 int launch_read(const ArrayView& v, const uint64_t* idx, uint64_t n, void* out, int num_sms, cudaStream_t st) {

@@ -50,6 +50,7 @@ struct gga_array {
   gga::ArrayView* dview;    // device copy of `view`, for kernels that take many arrays
   void* wscratch;           // binned random writes: bins of (address, value), kept between calls
   size_t wscratch_bytes;
+  bool counted;             // among the device's live handles
 };
 
 namespace {
@@ -195,6 +196,65 @@ int pool_read(gga_pool_t* pl, cudaStream_t st, uint64_t* bump, uint64_t* free_by
   return GGA_OK;
 }
 
+// Workspaces of single calls, one stream-ordered memory pool per device.  A
+// call's workspace goes back when the call's kernels are done, so all handles
+// share one set, and concurrent streams and threads each get their own.  The
+// pool keeps up to kWorkspaceKeep bytes between calls (mapping the memory
+// anew would cost more than the kernels save) while any handle lives; with
+// the last one it gives everything back.
+constexpr uint64_t kWorkspaceKeep = 1ull << 30;
+constexpr int kMaxDevices = 64;
+std::mutex g_ws_mu;
+cudaMemPool_t g_ws_pool[kMaxDevices];
+bool g_ws_made[kMaxDevices];
+uint64_t g_ws_handles[kMaxDevices];
+
+void workspace_handle_made(int dev) {
+  if (dev < 0 || dev >= kMaxDevices) return;
+  std::lock_guard<std::mutex> lock(g_ws_mu);
+  ++g_ws_handles[dev];
+}
+
+void workspace_handle_gone(int dev) {   // its device is idle
+  if (dev < 0 || dev >= kMaxDevices) return;
+  std::lock_guard<std::mutex> lock(g_ws_mu);
+  if (--g_ws_handles[dev] == 0 && g_ws_made[dev]) cudaMemPoolTrimTo(g_ws_pool[dev], 0);
+}
+
+// `bytes` of device memory on `st`, or nullptr (a stream being captured, no
+// memory); the runtime's last error is left clear.
+void* workspace_take(int dev, size_t bytes, cudaStream_t st) {
+  if (dev < 0 || dev >= kMaxDevices) return nullptr;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  {
+    std::lock_guard<std::mutex> lock(g_ws_mu);
+    if (!g_ws_made[dev]) {
+      cudaMemPoolProps props;
+      std::memset(&props, 0, sizeof(props));
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      uint64_t keep = kWorkspaceKeep;
+      if (cudaMemPoolCreate(&g_ws_pool[dev], &props) != cudaSuccess ||
+          cudaMemPoolSetAttribute(g_ws_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+      }
+      g_ws_made[dev] = true;
+    }
+  }
+  void* p = nullptr;
+  if (cudaMallocFromPoolAsync(&p, bytes, g_ws_pool[dev], st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  return p;
+}
+
 int sync_status(gga_array* h, cudaStream_t st, bool clear) {
   uint32_t status = 0;
   if (cudaMemcpyAsync(&status, h->view.status, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GGA_ERR_CUDA;
@@ -304,6 +364,8 @@ static int handle_make(const gga_params* p, gga_pool_t* pool, bool own_pool, cud
   // Commit gga_insert_noalloc's fixed scratch on this device now, so that
   // no call of that entry point is the one that places it.
   gga::noalloc_prepare(h->device);
+  workspace_handle_made(h->device);
+  h->counted = true;
   *out = h;
   return GGA_OK;
 }
@@ -386,6 +448,18 @@ int gga_read(gga_handle h, const uint64_t* idx_dev, uint64_t n, void* out_dev, v
   if (!h || (n > 0 && (!idx_dev || !out_dev))) return GGA_ERR_INVALID;
   if ((reinterpret_cast<uintptr_t>(out_dev) % h->p.elem_bytes) != 0) return GGA_ERR_INVALID;
   if ((reinterpret_cast<uintptr_t>(idx_dev) & 7) != 0) return GGA_ERR_INVALID;
+  // Large batches are grouped by ranges of indices in a workspace taken from
+  // the library's stream-ordered pool for the call.  A stream being captured
+  // and a failed allocation take the direct kernel.
+  const size_t need = gga::rbin_scratch_bytes(n, h->p.elem_bytes, h->pool->bytes);
+  if (need) {
+    cudaStream_t st = S(stream);
+    void* ws = workspace_take(h->device, need, st);
+    if (ws) {
+      const int rc = gga::launch_read_binned(h->view, idx_dev, n, out_dev, ws, h->num_sms, st);
+      return cudaFreeAsync(ws, st) == cudaSuccess ? rc : GGA_ERR_CUDA;
+    }
+  }
   return gga::launch_read(h->view, idx_dev, n, out_dev, h->num_sms, S(stream));
 }
 
@@ -503,6 +577,7 @@ int gga_destroy(gga_handle h) {
   if (h->wscratch && cudaFree(h->wscratch) != cudaSuccess) rc = GGA_ERR_CUDA;
   if (h->meta && cudaFree(h->meta) != cudaSuccess) rc = GGA_ERR_CUDA;
   if (h->own_pool && h->pool && pool_free(h->pool) != GGA_OK) rc = GGA_ERR_CUDA;
+  if (h->counted) workspace_handle_gone(h->device);
   delete h;
   return rc;
 }

@@ -208,6 +208,11 @@ int launch_insert_generated(const ArrayView& v, const gga_gen_spec& spec, uint32
                             uint32_t* done_counter, int num_sms, cudaStream_t st);
 int launch_finalize(const ArrayView& v, cudaStream_t st);
 int launch_read(const ArrayView& v, const uint64_t* idx, uint64_t n, void* out, int num_sms, cudaStream_t st);
+// A batch large enough to be grouped by ranges first: rbin_scratch_bytes > 0
+// (slab_bytes: of the array's pool); scratch: that many bytes, contents unset.
+uint64_t rbin_scratch_bytes(uint64_t n, uint32_t E, uint64_t slab_bytes);
+int launch_read_binned(const ArrayView& v, const uint64_t* idx, uint64_t n, void* out, void* scratch, int num_sms,
+                       cudaStream_t st);
 // scratch: nullptr, or wbin_scratch_bytes(n, E) bytes whose first 1 KB is
 // zero before the first call (the binned path for n >= 2^20 keeps it so).
 int launch_write(const ArrayView& v, const uint64_t* idx, uint64_t n, const void* in, int num_sms, void* scratch,
