@@ -221,6 +221,22 @@ __device__ __forceinline__ uint64_t ring_pop(PoolState* p, uint32_t c) {
   return reinterpret_cast<const uint64_t*>(p->rings)[p->ring_off[c] + pos % rc];
 }
 
+// ring_pop with one round trip before the atomic and one after it: head, tail
+// and slot range do not move while pops run, so they are loaded together,
+// and an empty queue costs no atomic (its head stays where the fix-up would
+// leave it).  For kernels whose time is this chain; inlined into the pass
+// loop of a push kernel its loads changed the loop's code for the worse
+// (gga_push_expand 0.64 -> 0.81 ms on GB300).
+__device__ __forceinline__ uint64_t ring_pop_early(PoolState* p, uint32_t c) {
+  const unsigned long long rc = p->ring_cap[c], head = p->ring_head[c], tail = p->ring_tail[c];
+  const unsigned long long off = p->ring_off[c];
+  const uint64_t* rings = reinterpret_cast<const uint64_t*>(p->rings);
+  if (rc == 0 || head >= tail) return 0;
+  const unsigned long long pos = head + atomicAdd(&p->ring_taken[c], 1ull);
+  if (pos >= tail) return 0;
+  return rings[off + pos % rc];
+}
+
 // Allocate buckets nb..need-1 of LFVector l (Algorithm 2 for every bucket a
 // reservation reaches).  Queued buckets first; the rest with one bump of the
 // slab for all of them.  A bucket index that cannot be served ends the
@@ -261,7 +277,9 @@ __device__ inline uint32_t grow_buckets(const ArrayView& v, uint32_t l, uint32_t
 // LFVector's buckets are in flight together instead of one after another;
 // the misses get one bump of the slab for all of them, in bucket order.
 // Same result as grow_buckets (which queued bucket of a class a bucket gets
-// may differ; contents, sizes and capacities do not).
+// may differ; contents, sizes and capacities do not).  EARLY: pops by
+// ring_pop_early.
+template <bool EARLY = false>
 __device__ inline uint32_t grow_buckets_warp(const ArrayView& v, uint32_t l, uint32_t nb, uint32_t need) {
   const uint32_t lane = threadIdx.x & 31;
   uint64_t* tab = v.buckets + static_cast<uint64_t>(l) * kMaxBuckets;
@@ -274,7 +292,13 @@ __device__ inline uint32_t grow_buckets_warp(const ArrayView& v, uint32_t l, uin
     uint64_t a = in ? tab[b] : 0;
     const bool pop = in && a == 0;
     const uint64_t sz = pop ? alloc_bytes_for(bucket_len(b, v.log2B) * v.E) : 0;
-    if (pop) a = ring_pop(v.pool, class_of(bucket_len(b, v.log2B) * v.E));
+    if (pop) {
+      if constexpr (EARLY) {   // sz is a power of two
+        a = ring_pop_early(v.pool, 63u - static_cast<uint32_t>(__clzll(static_cast<long long>(sz))));
+      } else {
+        a = ring_pop(v.pool, class_of(bucket_len(b, v.log2B) * v.E));
+      }
+    }
     const uint64_t mb = (pop && a == 0) ? sz : 0;
     const uint64_t incl = warp_incl_scan(mb);
     const uint64_t total = __shfl_sync(0xffffffffu, incl, 31);

@@ -1230,21 +1230,25 @@ int launch_write(const ArrayView& v, const uint64_t* idx, uint64_t n, const void
 }
 
 template <int E>
-static void sweep_as(const ArrayView& v, int mode, uint64_t delta, uint32_t repeats, int num_sms,
+static void sweep_as(const ArrayView& v, int mode, uint64_t delta, uint32_t repeats, uint64_t slab_bytes, int num_sms,
                      cudaStream_t st) {
   if (mode == GGA_RW_G) {
     // The size is on the device, so the grid cannot follow it: 32 blocks per
-    // SM (several times what is resident at once) stride over the array.
-    sweep_g_kernel<E><<<static_cast<unsigned>(num_sms) * 32u, 256, 0, st>>>(v, delta, repeats);
+    // SM (several times what is resident at once) stride over the array, or
+    // as many as the slab could give work.
+    const uint64_t most = slab_bytes / (static_cast<uint64_t>(E) * 256 * kSweepGPerLane) + 1;
+    const uint64_t grid = static_cast<uint64_t>(num_sms) * 32u;
+    sweep_g_kernel<E><<<static_cast<unsigned>(most < grid ? most : grid), 256, 0, st>>>(v, delta, repeats);
   } else {
     const unsigned grid = wave_grid(sweep_b_kernel<E>, 256, 0, num_sms, ~0ull);
     sweep_b_kernel<E><<<grid, 256, 0, st>>>(v, delta, repeats);
   }
 }
 
-int launch_sweep(const ArrayView& v, int mode, uint64_t delta, uint32_t repeats, int num_sms, cudaStream_t st) {
-  if (v.E == 4) sweep_as<4>(v, mode, delta, repeats, num_sms, st);
-  else sweep_as<8>(v, mode, delta, repeats, num_sms, st);
+int launch_sweep(const ArrayView& v, int mode, uint64_t delta, uint32_t repeats, uint64_t slab_bytes, int num_sms,
+                 cudaStream_t st) {
+  if (v.E == 4) sweep_as<4>(v, mode, delta, repeats, slab_bytes, num_sms, st);
+  else sweep_as<8>(v, mode, delta, repeats, slab_bytes, num_sms, st);
   return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 

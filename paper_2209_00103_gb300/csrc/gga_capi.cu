@@ -489,7 +489,7 @@ int gga_write(gga_handle h, const uint64_t* idx_dev, uint64_t n, const void* in_
 int gga_sweep(gga_handle h, int mode, uint64_t delta, uint32_t repeats, void* stream) {
   if (!h || (mode != GGA_RW_G && mode != GGA_RW_B)) return GGA_ERR_INVALID;
   if (h->p.elem_bytes == 16) return GGA_ERR_INVALID;
-  return gga::launch_sweep(h->view, mode, delta, repeats, h->num_sms, S(stream));
+  return gga::launch_sweep(h->view, mode, delta, repeats, h->pool->bytes, h->num_sms, S(stream));
 }
 
 int gga_flatten(gga_handle h, void* dst_dev, uint64_t dst_capacity_elems, void* stream) {

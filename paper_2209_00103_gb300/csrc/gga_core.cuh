@@ -199,7 +199,7 @@ struct InsertScratch {
   uint64_t* ins_base;             // [L] LFVector size before the batch
   uint64_t* ins_len;              // [L] committed elements of the batch
   uint64_t* cp_prefix;            // [L+1] prefix of copy chunks
-  uint32_t* counters;             // [1] last-block-done counter of reserve
+  uint32_t* counters;             // last-block-done counters, zero between calls: [0] of count, [1] of reserve
 };
 
 int launch_insert(const ArrayView& v, const InsertScratch& s, const uint32_t* counts, uint32_t rounds,
@@ -218,7 +218,8 @@ int launch_read_binned(const ArrayView& v, const uint64_t* idx, uint64_t n, void
 int launch_write(const ArrayView& v, const uint64_t* idx, uint64_t n, const void* in, int num_sms, void* scratch,
                  cudaStream_t st);
 uint64_t wbin_scratch_bytes(uint64_t n, uint32_t E);
-int launch_sweep(const ArrayView& v, int mode, uint64_t delta, uint32_t repeats, int num_sms, cudaStream_t st);
+int launch_sweep(const ArrayView& v, int mode, uint64_t delta, uint32_t repeats, uint64_t slab_bytes, int num_sms,
+                 cudaStream_t st);
 int launch_flatten(const ArrayView& v, void* dst, uint64_t cap_elems, int num_sms, cudaStream_t st);
 int launch_reserve(const ArrayView& v, const uint64_t* target, cudaStream_t st);
 int launch_clear(const ArrayView& v, cudaStream_t st);

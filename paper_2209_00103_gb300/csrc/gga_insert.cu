@@ -8,7 +8,8 @@
 //      the tile and the tile's total.
 //   2. tile_scan: one block turns the tile totals into tile prefixes, so the
 //      first-value index of run (r, l) is voff(r*L + l) = tile prefix + row
-//      prefix, with no inter-block waiting anywhere.
+//      prefix, with no inter-block waiting anywhere (the last count block to
+//      finish does it when there are few tiles).
 //   3. reserve: one warp per LFVector.  A shuffle scan over the rounds gives
 //      each round's position in the batch (the per-round size reservation of
 //      Algorithm 1, done for all rounds at once), then the warp's leader
@@ -65,14 +66,61 @@ __device__ __forceinline__ uint64_t voff_at(const InsertScratch& s, uint64_t row
   return s.tile_pre[row / rows_per_tile] + s.row_pre[row];
 }
 
+// Exclusive scan of the tile totals in place; entry n_tiles gets the total.
+// One block (any multiple of 32 threads); warp w takes kItems x 32
+// consecutive tiles with coalesced loads (lane i reads tiles 32k + i), scans
+// them with shuffles, one block scan combines the warp totals, then the warp
+// writes its tiles back the same way.  (A run of consecutive tiles per thread
+// made every load and store instruction touch 32 lines: 19 us for 16,384
+// tiles.)
+template <int kItems>
+__device__ __forceinline__ void scan_tiles(uint64_t* tile, uint64_t n_tiles, uint64_t* s_warp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint64_t per_warp = 32ull * kItems;
+  const uint64_t per_pass = per_warp * (blockDim.x >> 5);
+  uint64_t run = 0;
+  for (uint64_t t0 = 0; t0 < n_tiles; t0 += per_pass) {
+    const uint64_t w0 = t0 + static_cast<uint64_t>(warp) * per_warp;
+    uint64_t x[kItems];
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+      const uint64_t i = w0 + 32 * k + lane;
+      x[k] = i < n_tiles ? __ldcg(tile + i) : 0;
+    }
+    uint64_t carry = 0;   // sum of the warp's tiles before chunk k
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+      const uint64_t inc = warp_incl_scan(x[k]);
+      const uint64_t ex = carry + inc - x[k];
+      carry += __shfl_sync(0xffffffffu, inc, 31);
+      x[k] = ex;
+    }
+    uint64_t tot;
+    const uint64_t e = block_excl_scan_u64(lane == 0 ? carry : 0, s_warp, tot);
+    const uint64_t wbase = run + __shfl_sync(0xffffffffu, e, 0);
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+      const uint64_t i = w0 + 32 * k + lane;
+      if (i < n_tiles) tile[i] = wbase + x[k];
+    }
+    run += tot;
+  }
+  if (threadIdx.x == 0) tile[n_tiles] = run;
+}
+
+// Up to this many tiles the last count block to finish scans them; more take
+// a block of 1024 threads of their own.  On GB300: 5 tiles 7.9 + 6.3 us as
+// two kernels, 10.5 as one; 574 tiles 10.7 + 10.6 and 14.2.
+constexpr uint64_t kCountScanMax = 1024;
+
 // T_TPL > 0: T == T_TPL (a multiple of 128) and counts 16-byte aligned, the
 // row is read with 128-bit loads.  T_TPL == 0: any T, 32-bit loads.
 template <int T_TPL>
 __global__ void __launch_bounds__(kCountThreads) count_kernel(const uint32_t* __restrict__ counts, uint64_t n_rows,
                                                               uint32_t T, uint32_t L, uint32_t R,
                                                               uint64_t* __restrict__ row_pre,
-                                                              uint64_t* __restrict__ tile_agg,
-                                                              uint64_t* __restrict__ pre) {
+                                                              uint64_t* tile_agg, uint64_t* __restrict__ pre,
+                                                              uint32_t* done) {
   constexpr int RPW = count_rows_per_warp(T_TPL);
   constexpr int ROWS = count_rows_per_tile(T_TPL);
   __shared__ uint64_t s_tot[ROWS];
@@ -133,49 +181,24 @@ __global__ void __launch_bounds__(kCountThreads) count_kernel(const uint32_t* __
     }
     if (lane == 0) tile_agg[tile] = run;
   }
+  if (!done) return;
+  // The last block to finish turns the tile totals into prefixes.
+  __shared__ uint64_t s_warp[33];
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  scan_tiles<4>(tile_agg, gridDim.x, s_warp);
+  if (threadIdx.x == 0) *done = 0;
 }
-
-// Exclusive scan of the tile totals in place; entry n_tiles gets the total.
-// One block; warp w takes kTileScanItems x 32 consecutive tiles with
-// coalesced loads (lane i reads tiles 32k + i), scans them with shuffles,
-// one block scan combines the warp totals, then the warp writes its tiles
-// back the same way.  (A run of consecutive tiles per thread made every
-// load and store instruction touch 32 lines: 19 us for 16,384 tiles.)
-constexpr int kTileScanItems = 16;
 
 __global__ void __launch_bounds__(1024) tile_scan_kernel(uint64_t* tile, uint64_t n_tiles) {
   __shared__ uint64_t s_warp[33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint64_t per_warp = 32ull * kTileScanItems;
-  const uint64_t per_pass = per_warp * (blockDim.x >> 5);
-  uint64_t run = 0;
-  for (uint64_t t0 = 0; t0 < n_tiles; t0 += per_pass) {
-    const uint64_t w0 = t0 + static_cast<uint64_t>(warp) * per_warp;
-    uint64_t x[kTileScanItems];
-#pragma unroll
-    for (int k = 0; k < kTileScanItems; ++k) {
-      const uint64_t i = w0 + 32 * k + lane;
-      x[k] = i < n_tiles ? tile[i] : 0;
-    }
-    uint64_t carry = 0;   // sum of the warp's tiles before chunk k
-#pragma unroll
-    for (int k = 0; k < kTileScanItems; ++k) {
-      const uint64_t inc = warp_incl_scan(x[k]);
-      const uint64_t ex = carry + inc - x[k];
-      carry += __shfl_sync(0xffffffffu, inc, 31);
-      x[k] = ex;
-    }
-    uint64_t tot;
-    const uint64_t e = block_excl_scan_u64(lane == 0 ? carry : 0, s_warp, tot);
-    const uint64_t wbase = run + __shfl_sync(0xffffffffu, e, 0);
-#pragma unroll
-    for (int k = 0; k < kTileScanItems; ++k) {
-      const uint64_t i = w0 + 32 * k + lane;
-      if (i < n_tiles) tile[i] = wbase + x[k];
-    }
-    run += tot;
-  }
-  if (threadIdx.x == 0) tile[n_tiles] = run;
+  scan_tiles<16>(tile, n_tiles, s_warp);
 }
 
 // ---------------------------------------------------------------------------
@@ -222,7 +245,7 @@ __global__ void __launch_bounds__(256) reserve_kernel(ArrayView v, InsertScratch
     if (S > 0) {
       nb = v.nbuckets[l];
       need = buckets_for(base + S, v.log2B);
-      if (need > nb) got = grow_buckets_warp(v, static_cast<uint32_t>(l), nb, need);
+      if (need > nb) got = grow_buckets_warp<true>(v, static_cast<uint32_t>(l), nb, need);
     }
     __syncwarp();
     if (lane == 0) {
@@ -691,8 +714,8 @@ template <int T_TPL>
 static void launch_count(const uint32_t* counts, uint64_t n_rows, uint32_t T, uint32_t L, uint32_t R,
                          const InsertScratch& s, cudaStream_t st) {
   const uint64_t n_tiles = (n_rows + count_rows_per_tile(T_TPL) - 1) / count_rows_per_tile(T_TPL);
-  count_kernel<T_TPL><<<static_cast<unsigned>(n_tiles), kCountThreads, 0, st>>>(counts, n_rows, T, L, R, s.row_pre,
-                                                                                 s.tile_pre, s.pre);
+  count_kernel<T_TPL><<<static_cast<unsigned>(n_tiles), kCountThreads, 0, st>>>(
+      counts, n_rows, T, L, R, s.row_pre, s.tile_pre, s.pre, n_tiles <= kCountScanMax ? s.counters : nullptr);
 }
 
 static int count_template(uint32_t T, bool vec_ok) {
@@ -718,7 +741,7 @@ int launch_insert(const ArrayView& v, const InsertScratch& s, const uint32_t* co
     case 1024: launch_count<1024>(counts, n_rows, v.T, v.L, R, s, st); break;
     default: launch_count<0>(counts, n_rows, v.T, v.L, R, s, st); break;
   }
-  tile_scan_kernel<<<1, 1024, 0, st>>>(s.tile_pre, n_tiles);
+  if (n_tiles > kCountScanMax) tile_scan_kernel<<<1, 1024, 0, st>>>(s.tile_pre, n_tiles);
 
   const uint32_t cce = kCopyChunkBytes / v.E;
   const unsigned rblocks = static_cast<unsigned>((static_cast<uint64_t>(v.L) * 32 + 255) / 256);

@@ -39,3 +39,18 @@ def test_sizes_around_bucket_and_chunk_edges(L, B, E):
     assert g.memory()["pool_bump_bytes"] == held
     g.close()
     o.close()
+
+
+@pytest.mark.parametrize("T,R", [(16, 1), (16, 33), (16, 2045), (16, 2047), (16, 2049), (128, 130)])
+def test_count_tiles_around_the_scan_by_the_last_block(T, R):
+    """32 rows a tile (128 for T = 128): one tile, and 1023 to 1025 around the line."""
+    L = 16
+    for rounds in (R, R + 1):
+        counts = (np.arange(rounds * L * T, dtype=np.uint64) * 2654435761 % 3).astype(np.uint32).reshape(rounds, L, T)
+        n = int(counts.sum())
+        g, o = make_pair(L, T, 64, 4, expected_elems=n)
+        for _ in range(2):
+            insert_both(g, o, counts, packed_values(n, 4), 4)
+        assert_same_state(g, o)
+        g.close()
+        o.close()
