@@ -83,31 +83,36 @@ __device__ void append_run(const ArrayView& v, uint32_t l, uint64_t start, uint6
 }
 
 // One block per request: every LFVector's share is reserved (one size
-// update, Algorithm 2 for the buckets it reaches) by its own thread, then
-// the block recomputes the array's offsets from the new sizes.
+// update, Algorithm 2 for the buckets it reaches, taken together) by a warp,
+// then the block recomputes the array's offsets from the new sizes.  The
+// time is the chain of one LFVector's pops: 256 requests on GB300 17.4 us with
+// a thread per LFVector, which takes its buckets one after another, 7.2 now.
 __global__ void __launch_bounds__(kServeThreads) append_reserve_kernel(const __grid_constant__ AppendParams P) {
   __shared__ FinalizeShared sh;
   const uint32_t r = blockIdx.x;
-  const ArrayView& v = *P.view[r];
-  for (uint32_t l = threadIdx.x; l < v.L; l += blockDim.x) {
+  const ArrayView v = *P.view[r];
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t l = threadIdx.x >> 5; l < v.L; l += kServeThreads / 32) {   // warp-uniform
     const uint64_t c = P.n[r] / v.L + (l < P.n[r] % v.L ? 1 : 0);
     const uint64_t base = v.sizes[l];
+    const uint32_t nb = v.nbuckets[l];
     uint64_t len = c;
     if (c) {
-      const uint32_t nb = v.nbuckets[l];
       const uint32_t need = buckets_for(base + c, v.log2B);
       if (need > nb) {
-        const uint32_t got = grow_buckets(v, l, nb, need);
-        v.nbuckets[l] = got;
-        if (got < need) {
-          len = 0;   // the append does not fit: this LFVector takes none of it
-          latch_error(v.status, GGA_ERR_POOL_EXHAUSTED);
+        const uint32_t got = grow_buckets_warp<true>(v, l, nb, need);
+        if (lane == 0) {
+          v.nbuckets[l] = got;
+          if (got < need) latch_error(v.status, GGA_ERR_POOL_EXHAUSTED);
         }
+        if (got < need) len = 0;   // the append does not fit: this LFVector takes none of it
       }
     }
-    v.sizes[l] = base + len;
-    P.res_base[P.slot0[r] + l] = base;
-    P.res_len[P.slot0[r] + l] = len;
+    if (lane == 0) {
+      v.sizes[l] = base + len;
+      P.res_base[P.slot0[r] + l] = base;
+      P.res_len[P.slot0[r] + l] = len;
+    }
   }
   __syncthreads();
   finalize_block(v, nullptr, nullptr, nullptr, 1, sh);
@@ -140,31 +145,54 @@ __global__ void __launch_bounds__(kServeThreads) append_write_kernel(const __gri
   }
 }
 
+// Reads are chains of dependent loads (offsets, bucket table, element), so a
+// block keeps kReadU of them in flight per thread and takes kReadSpan
+// consecutive reads of its request; blockIdx.y walks the request (further
+// than gridDim.y spans by striding).  256 requests of 4096 reads on GB300:
+// 21.5 us with one block per request and one read at a time, 13.3 now; 480
+// requests on 1.9 GB of arrays 31 and 33 (random DRAM accesses bound those).
+constexpr int kReadU = 4;
+constexpr uint64_t kReadSpan = static_cast<uint64_t>(kServeThreads) * kReadU;
+
 template <int E>
-__device__ void read_run(const ArrayView& v, uint64_t n, uint64_t seed, void* out) {
+__device__ __forceinline__ void read_run(const ArrayView& v, uint64_t n, uint64_t seed, void* out) {
   typedef typename Elem<E>::T T;
   T* o = static_cast<T*>(out);
-  const uint64_t N = v.offsets[v.L];
-  for (uint64_t k = threadIdx.x; k < n; k += blockDim.x) {
-    T x = T();
-    if (N) {
-      const uint64_t g = ((splitmix(seed, k) >> 32) * N) >> 32;   // uniform over [0, N)
-      const uint32_t l = find_lfv(v.offsets, v.L, N, g);
-      uint32_t b;
-      uint64_t off;
-      bucket_of(g - v.offsets[l], v.log2B, b, off);
-      x = *reinterpret_cast<const T*>(v.buckets[static_cast<uint64_t>(l) * kMaxBuckets + b] + off * E);
+  const uint64_t N = __ldg(v.offsets + v.L);
+  for (uint64_t k0 = blockIdx.y * kReadSpan + threadIdx.x; k0 < n; k0 += gridDim.y * kReadSpan) {
+    uint64_t a[kReadU];
+#pragma unroll
+    for (int u = 0; u < kReadU; ++u) {
+      const uint64_t k = k0 + static_cast<uint64_t>(u) * kServeThreads;
+      a[u] = 0;
+      if (N && k < n) {
+        const uint64_t g = ((splitmix(seed, k) >> 32) * N) >> 32;   // uniform over [0, N)
+        const uint32_t l = find_lfv(v.offsets, v.L, N, g);
+        uint32_t b;
+        uint64_t off;
+        bucket_of(g - __ldg(v.offsets + l), v.log2B, b, off);
+        a[u] = __ldg(v.buckets + static_cast<uint64_t>(l) * kMaxBuckets + b) + off * E;
+      }
     }
-    o[k] = x;
+    T x[kReadU];
+#pragma unroll
+    for (int u = 0; u < kReadU; ++u) x[u] = a[u] ? *reinterpret_cast<const T*>(a[u]) : T();
+#pragma unroll
+    for (int u = 0; u < kReadU; ++u) {
+      const uint64_t k = k0 + static_cast<uint64_t>(u) * kServeThreads;
+      if (k < n) o[k] = x[u];
+    }
   }
 }
 
 __global__ void __launch_bounds__(kServeThreads) read_batch_kernel(const __grid_constant__ ReadParams P) {
-  const ArrayView& v = *P.view[blockIdx.x];
+  const uint64_t n = P.n[blockIdx.x];
+  if (blockIdx.y * kReadSpan >= n) return;
+  const ArrayView v = *P.view[blockIdx.x];
   switch (v.E) {
-    case 4: read_run<4>(v, P.n[blockIdx.x], P.seed[blockIdx.x], P.out[blockIdx.x]); break;
-    case 8: read_run<8>(v, P.n[blockIdx.x], P.seed[blockIdx.x], P.out[blockIdx.x]); break;
-    default: read_run<16>(v, P.n[blockIdx.x], P.seed[blockIdx.x], P.out[blockIdx.x]); break;
+    case 4: read_run<4>(v, n, P.seed[blockIdx.x], P.out[blockIdx.x]); break;
+    case 8: read_run<8>(v, n, P.seed[blockIdx.x], P.out[blockIdx.x]); break;
+    default: read_run<16>(v, n, P.seed[blockIdx.x], P.out[blockIdx.x]); break;
   }
 }
 
@@ -240,6 +268,7 @@ int gga_read_batch(const gga_read_req* reqs, uint32_t n, void* stream) {
     gga::ReadParams P;
     P.n_req = m;
     P.pad = 0;
+    uint64_t most = 1;
     for (uint32_t j = 0; j < m; ++j) {
       const gga_read_req& q = reqs[i0 + j];
       if (!q.array || (q.n && !q.out)) return GGA_ERR_INVALID;
@@ -247,8 +276,11 @@ int gga_read_batch(const gga_read_req* reqs, uint32_t n, void* stream) {
       P.n[j] = q.n;
       P.seed[j] = q.seed;
       P.out[j] = q.out;
+      most = std::max<uint64_t>(most, q.n);
     }
-    gga::read_batch_kernel<<<m, gga::kServeThreads, 0, st>>>(P);
+    // The largest request's spans, up to 64 blocks a request.
+    const uint64_t spans = std::min<uint64_t>(64, (most + gga::kReadSpan - 1) / gga::kReadSpan);
+    gga::read_batch_kernel<<<dim3(m, static_cast<unsigned>(spans)), gga::kServeThreads, 0, st>>>(P);
   }
   return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
