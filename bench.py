@@ -40,9 +40,28 @@ sys.path.insert(0, ROOT)
 METRIC = "GGArray insert Gelem/s & % HBM roofline; mem/needed; served p99 latency"
 PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # Kernels per phase: a write batch of 2^20 or more goes through bins (count,
-# scan, scatter into bins, apply), a smaller one is one kernel.
-LAUNCHES_PER_STEP = {"clear": 1, "insert": 4, "read": 1, "write": 4, "rw_b": 1, "rw_g": 1, "flatten": 1}
+# scan, scatter into bins, apply), a smaller one is one kernel; a read batch of
+# 2^25 or more from a slab of at most 48 bytes per read goes through bins too
+# (count, scan, scatter, apply, return).  An insertion of up to 1024 count
+# tiles (32 rows each at T = 512) scans them in its count kernel.
+LAUNCHES_PER_STEP = {"clear": 1, "insert": 4, "read": 5, "write": 4, "rw_b": 1, "rw_g": 1, "flatten": 1}
 BINNED_WRITE_MIN = 1 << 20
+BINNED_READ_MIN = 1 << 25
+BINNED_READ_SLAB = (512 << 20, 48)   # bytes at least, bytes per read at most
+
+
+def launches_per_step(n_rand: int, slab_bytes: int, rows: int) -> int:
+    n = sum(LAUNCHES_PER_STEP.values())
+    if n_rand < BINNED_WRITE_MIN:
+        n -= 3
+    if not read_is_binned(n_rand, slab_bytes):
+        n -= 4
+    return n - (1 if rows <= 32 * 1024 else 0)
+
+
+def read_is_binned(n_rand: int, slab_bytes: int) -> bool:
+    least, per_read = BINNED_READ_SLAB
+    return n_rand >= BINNED_READ_MIN and slab_bytes >= least and slab_bytes // per_read <= n_rand
 
 
 def parse_args():
@@ -357,17 +376,19 @@ def run_ours(args, world, rank, local):
         phase_info[name] = d
 
     # The dominant kernel carries the roofline record: the longest phase that
-    # is one kernel (insert and a binned write are several; the launch list
-    # in profiles/ confirms which single kernel takes the most time).
+    # is one kernel (insert and binned reads and writes are several; the launch
+    # list in profiles/ confirms which single kernel takes the most time).
     binned = n_rand >= BINNED_WRITE_MIN
-    single = ["flatten", "rw_b", "rw_g", "read"] + ([] if binned else ["write"])
+    binned_read = read_is_binned(n_rand, pool_bytes)
+    single = ["flatten", "rw_b", "rw_g"] + ([] if binned_read else ["read"]) + ([] if binned else ["write"])
     dom = max(single, key=lambda n: ph_ms[n])
     kernels = {"insert": "count_kernel + tile_scan_kernel + reserve_kernel + copy_bulk_kernel",
                "flatten": "flatten_kernel", "rw_b": "sweep_b_kernel", "rw_g": "sweep_g_kernel",
-               "read": "read_kernel",
+               "read": ("rbin_count_kernel + wbin_scan_kernel + rbin_scatter_kernel + rbin_apply_kernel + "
+                        "rbin_return_kernel" if binned_read else "read_kernel"),
                "write": ("wbin_count_kernel + wbin_scan_kernel + wbin_scatter_kernel + wbin_apply_kernel"
                          if binned else "write_kernel")}
-    for name in ("insert", "write"):
+    for name in ("insert", "read", "write"):
         phase_info[name]["kernels"] = kernels[name]
     ach = ab[dom] / (ph_ms[dom] / 1e3) / 1e9
     units = {"read": n_rand, "write": n_rand, "flatten": N, "rw_b": N, "rw_g": N}
@@ -385,12 +406,12 @@ def run_ours(args, world, rank, local):
     baselines = None
     if not args.no_baselines and rank == 0 and w.E == 4:
         baselines = run_flat_baselines(counts, values, idx_r, idx_w, vals_w, N, R, w.L, w.T, dev, stream)
-        if dom == "read":
+        if dom == "read" or binned_read:
             # A random gather is bound by the DRAM access rate, not by its
             # bytes: the same indices gathered from a flat int32 array by
-            # PyTorch give the ceiling the translated read is held against.
+            # PyTorch (grouped by ranges first, the read phase passes it).
             flat_ms = baselines["static"]["phases_ms"]["read"]
-            roofline["vs_flat_gather"] = {
+            (roofline if dom == "read" else phase_info["read"])["vs_flat_gather"] = {
                 "flat_ms": flat_ms, "ms": round(ph_ms["read"], 4), "frac": round(flat_ms / ph_ms["read"], 3),
                 "accesses_per_s": round(n_rand / (ph_ms["read"] / 1e3) / 1e9, 2), "unit": "G accesses/s",
                 "flat": "torch.index_select on a flat int32 array of the same size, same indices"}
@@ -426,7 +447,7 @@ def run_ours(args, world, rank, local):
         "insert_generated": gen,
         "push_generated": push_gen,
         "push_expand": push_exp,
-        "gpu_launches": K * (sum(LAUNCHES_PER_STEP.values()) - (0 if binned else 3)),
+        "gpu_launches": K * launches_per_step(n_rand, pool_bytes, R * w.L),
         "clocks": clocks,
         "e2e": e2e,
         "baselines": baselines,
@@ -817,15 +838,16 @@ def run_batched(args, world, rank, local):
            "dtype": "u32/u64/record", "data": "synthetic",
            "config": {"workload": f"batched_{len(sizes)}_lognormal_median64K_sigma1.5_cap16M", "arrays": len(sizes),
                       "elements": total, "bytes": bytes_written, "rule": rule.to_json() if hasattr(rule, "to_json") else rule.__dict__,
-                      "step": "captured graph: clear every array + one persistent grow launch + finalize"},
+                      "step": "captured graph: clear every array + persistent grow kernels side by side + finalize"},
            "roofline": {"bound": "hbm", "achieved": round(gbs, 1), "peak": peak, "unit": "GB/s",
-                        "frac": round(gbs / peak, 3), "traffic": None, "kernel": "batch_grow_kernel",
+                        "frac": round(gbs / peak, 3), "traffic": None, "kernel": "batch_cluster_kernel + batch_grow_kernel (three payload sizes)",
                         "algorithmic_bytes_per_launch": bytes_written},
            "mem_over_needed": round(ratio, 4),
            "plain_one_launch_per_array": {"ms": round(plain_ms, 3),
                                           "gelem_s": round(total / (plain_ms / 1e3) / 1e9, 3),
                                           "speedup_of_batched": round(plain_ms / ms, 2)},
-           "gpu_launches": K * 4, "clocks": clocks}
+           # clear 2, a cluster and a block kernel per payload size, finalize
+           "gpu_launches": K * 9, "clocks": clocks}
     batching.teardown(pool, arrays, batch)
     return res
 

@@ -400,9 +400,11 @@ typedef struct {
  * host array read during the call; the arrays must outlive the batch). */
 int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, gga_batch* out);
 
-/* gga_batch_grow -- grow every job's array to its target: one persistent
- * kernel over all (array, LFVector) items, one kernel for the pools, one to
- * finalize the arrays.  Allocates nothing, does not synchronize.  Device
+/* gga_batch_grow -- grow every job's array to its target: persistent kernels
+ * over the (array, LFVector) items of each payload size and count
+ * distribution, side by side (forked from `stream` and joined to it), then one
+ * kernel to finalize the arrays and their pools.  Allocates nothing, does not
+ * synchronize.  Device
  * errors are latched in each array (pool exhausted: the LFVector keeps the
  * rounds that fit). */
 int gga_batch_grow(gga_batch b, void* stream);

@@ -209,10 +209,29 @@ cudaMemPool_t g_ws_pool[kMaxDevices];
 bool g_ws_made[kMaxDevices];
 uint64_t g_ws_handles[kMaxDevices];
 
+// The pool is made with the first handle, like the handle's own memory, so a
+// call allocates only in stream order.
 void workspace_handle_made(int dev) {
   if (dev < 0 || dev >= kMaxDevices) return;
   std::lock_guard<std::mutex> lock(g_ws_mu);
   ++g_ws_handles[dev];
+  if (g_ws_made[dev]) return;
+  cudaMemPoolProps props;
+  std::memset(&props, 0, sizeof(props));
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  uint64_t keep = kWorkspaceKeep;
+  if (cudaMemPoolCreate(&g_ws_pool[dev], &props) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return;
+  }
+  if (cudaMemPoolSetAttribute(g_ws_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    (void)cudaGetLastError();
+    cudaMemPoolDestroy(g_ws_pool[dev]);
+    return;
+  }
+  g_ws_made[dev] = true;
 }
 
 void workspace_handle_gone(int dev) {   // its device is idle
@@ -230,25 +249,14 @@ void* workspace_take(int dev, size_t bytes, cudaStream_t st) {
     (void)cudaGetLastError();
     return nullptr;
   }
+  cudaMemPool_t pool;
   {
     std::lock_guard<std::mutex> lock(g_ws_mu);
-    if (!g_ws_made[dev]) {
-      cudaMemPoolProps props;
-      std::memset(&props, 0, sizeof(props));
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
-      uint64_t keep = kWorkspaceKeep;
-      if (cudaMemPoolCreate(&g_ws_pool[dev], &props) != cudaSuccess ||
-          cudaMemPoolSetAttribute(g_ws_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
-      }
-      g_ws_made[dev] = true;
-    }
+    if (!g_ws_made[dev]) return nullptr;
+    pool = g_ws_pool[dev];
   }
   void* p = nullptr;
-  if (cudaMallocFromPoolAsync(&p, bytes, g_ws_pool[dev], st) != cudaSuccess) {
+  if (cudaMallocFromPoolAsync(&p, bytes, pool, st) != cudaSuccess) {
     (void)cudaGetLastError();
     return nullptr;
   }
