@@ -723,9 +723,9 @@ def time_push_expand(spec, B, counts, pool_bytes, dev, stream):
     return {"elements": n, "ms": round(ms, 4), "gelem_s": round(n / (ms / 1e3) / 1e9, 2),
             "algorithmic_bytes": int(alg), "achieved_gbs": round(gbs, 1), "frac_of_measured_peak": round(gbs / peak, 3),
             "frac_of_8tbs": round(gbs / 8000.0, 3), "device_error": rc,
-            "kernels": "push_expand_kernel + finalize_kernel",
+            "kernels": "push_expand_s_kernel + finalize_kernel",
             "note": "counts [R][L][T] and one input per (round, block, thread) read from HBM; "
-                    "block_push_rounds of 4 rounds, 4 slots per thread, staged 128-bit stores"}
+                    "RoundsPusher pushes of 4 rounds, 4 slots per thread, loads a push ahead, staged 128-bit stores"}
 
 
 # ---------------------------------------------------------------------------
