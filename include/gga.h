@@ -245,7 +245,7 @@ int gga_insert_generated(gga_handle h, const gga_gen_spec* spec, uint32_t rounds
  *
  * gga_push_generated -- gga_insert_generated written as a user kernel of
  *  the device API: one block per LFVector, each thread playing four of its T
- *  threads, one push per round through a gga::BlockPusher, then
+ *  threads (one for T <= 128), one push per round through a gga::BlockPusher, then
  *  gga_device_commit.  Same draws, same result, same errors as
  *  gga_insert_generated; it is the per-round form of Algorithm 1, which
  *  gga_insert_generated batches over rounds.  Each push is assembled in
@@ -253,8 +253,9 @@ int gga_insert_generated(gga_handle h, const gga_gen_spec* spec, uint32_t rounds
  *
  * gga_push_expand -- pushes of values read from device memory, written as a
  *  user kernel of the device API (one block per LFVector of T <= 512 slots,
- *  each thread playing 4 consecutive slots -- 2 for 16-byte elements --;
- *  gga::block_push_rounds, 4 rounds per call for 4-byte elements, 2 for
+ *  each thread playing 4 consecutive slots -- 2 for 16-byte elements, 1 while
+ *  there is no more than one LFVector per SM --;
+ *  gga::RoundsPusher, 4 rounds per push for 4-byte elements, 2 for
  *  8- and 16-byte), then gga_device_commit.  In
  *  round r, thread t of block l appends counts_dev[r][l][t] copies of
  *  inputs_dev[r][l][t].  counts_dev: device, uint32 [rounds][L][T], 4-byte

@@ -840,6 +840,8 @@ template <int E, int DIST>
 struct GenRounds {
   static constexpr bool kMarks = max_count<DIST>() == 0;
   static constexpr int value = E == 4 ? 8 : (kMarks ? (E == 8 ? 8 : 4) : (E == 8 ? 4 : 2));
+  static constexpr int small = E == 16 ? 4 : 8;   // T <= 256: the stage is small anyway (16 x 128 x 300
+                                                  // records: 124 us, at 2 rounds 175)
 };
 
 // One block per LFVector, R rounds in passes of K (grow_passes in
@@ -856,24 +858,24 @@ __global__ void __launch_bounds__(MAXT, MINB) gen_insert_kernel(const __grid_con
 
 template <int E, int DIST>
 static void launch_gen_as(const ArrayView& v, const GenParams& g, uint32_t R, cudaStream_t st) {
-  constexpr int K = GenRounds<E, DIST>::value;
   const bool vt = v.T > 256;
+  const uint32_t rounds = vt ? GenRounds<E, DIST>::value : GenRounds<E, DIST>::small;
   const uint32_t per = vt ? kGenVT : 1;
   const uint32_t nt = ((v.T + per - 1) / per + 31) / 32 * 32;
   // A pass of one element per thread and round and a quarter more, in
   // whole 16-byte words, and a warp's overhang (41,984 bytes at most; eight
   // blocks of T = 512 fit an SM).
   const uint32_t esize = GenRounds<E, DIST>::kMarks ? 4 : E;
-  const size_t smem = (static_cast<size_t>(K) * v.T * esize * 5 / 4 + 1024 + 15) & ~static_cast<size_t>(15);
-#define GGA_GEN(KV, MT, MB)                                                                                  \
+  const size_t smem = (static_cast<size_t>(rounds) * v.T * esize * 5 / 4 + 1024 + 15) & ~static_cast<size_t>(15);
+#define GGA_GEN(K, KV, MT, MB)                                                                               \
   do {                                                                                                       \
     auto kern = gen_insert_kernel<E, K, KV, MT, MB, DIST>;                                                   \
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));         \
     kern<<<v.L, nt, smem, st>>>(v, g, R, static_cast<uint32_t>(smem));                                       \
   } while (0)
-  if (!vt) GGA_GEN(1, 256, 6);
-  else if (v.T <= 512) GGA_GEN(kGenVT, 128, 8);
-  else GGA_GEN(kGenVT, 256, 4);
+  if (!vt) GGA_GEN((GenRounds<E, DIST>::small), 1, 256, 6);
+  else if (v.T <= 512) GGA_GEN((GenRounds<E, DIST>::value), kGenVT, 128, 8);
+  else GGA_GEN((GenRounds<E, DIST>::value), kGenVT, 256, 4);
 #undef GGA_GEN
 }
 

@@ -26,7 +26,11 @@ namespace gga {
 // Measured on GB300 for 1024 LFVectors x 512 threads x 512 rounds, int32:
 // 0.87 ms against 2.27 ms with one thread per LFVector thread (blocks of
 // 512, two per SM) storing its own elements.
+// Up to T = 128 a thread plays one: a block of a few lanes would otherwise do
+// four threads' work in each (1500 LFVectors x 32 threads x 100 rounds with
+// geometric counts, clear and flatten included: 225 us with four, 139 with one).
 constexpr int kPushSlots = 4;
+constexpr uint32_t kPushSlotsMinT = 129;
 
 // Stage of one push, in elements: T at one per thread and eight standard
 // deviations of a sum of T counts of variance up to 2 (a larger push stores
@@ -38,14 +42,13 @@ uint32_t push_half_elems(uint32_t T, uint32_t E) {
   return (T + 8 * root + 2 * vec - 1) / vec * vec;
 }
 
-template <int E, int DIST>
-__global__ void __launch_bounds__(1024 / kPushSlots, 4) push_generated_kernel(const ArrayView* view,
+template <int E, int DIST, int S>
+__global__ void __launch_bounds__(S == 1 ? 128 : 1024 / S, S == 1 ? 8 : 4) push_generated_kernel(const ArrayView* view,
                                                                               const __grid_constant__ GenParams g,
                                                                               uint32_t R, uint32_t T,
                                                                               uint32_t stage_bytes) {
   typedef typename Elem<E>::T V;
   typedef typename std::conditional<E == 4, uint32_t, uint64_t>::type W;   // a 4-byte element keeps the low 32 bits
-  constexpr int S = kPushSlots;
   extern __shared__ uint4 s_stage[];
   __shared__ PushShared sh;
   __shared__ ThresholdTable s_thr;
@@ -98,11 +101,12 @@ __global__ void __launch_bounds__(1024 / kPushSlots, 4) push_generated_kernel(co
 template <int E>
 void launch_push_generated_as(const ArrayView& v, const ArrayView* dview, const GenParams& g, uint32_t rounds,
                               cudaStream_t st) {
-  const uint32_t nt = ((v.T + kPushSlots - 1) / kPushSlots + 31) / 32 * 32;
+  const uint32_t slots = v.T >= kPushSlotsMinT ? kPushSlots : 1;
+  const uint32_t nt = ((v.T + slots - 1) / slots + 31) / 32 * 32;
   const uint32_t smem = 2 * push_half_elems(v.T, E) * E;   // two halves: at most 44 KB (T = 1024, 16-byte elements)
 #define GGA_PUSH(D)                                                                                         \
   do {                                                                                                      \
-    auto kern = push_generated_kernel<E, D>;                                                                \
+    auto kern = slots == 1 ? push_generated_kernel<E, D, 1> : push_generated_kernel<E, D, kPushSlots>;      \
     if (smem > 32768u)   /* with the count table the block's shared memory may pass 48 KB */                \
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));      \
     kern<<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);                                               \
@@ -263,7 +267,7 @@ int launch_expand_s(const ArrayView& v, const ArrayView* dview, const uint32_t* 
                     uint32_t rounds, cudaStream_t st) {
   // Every row of T counts and inputs then starts on a 16-byte boundary (8
   // for two counts), and a thread plays all of its slots or none.
-  const bool wide = v.T % S == 0 &&
+  const bool wide = S > 1 && v.T % S == 0 &&
                     ((reinterpret_cast<uintptr_t>(counts) | reinterpret_cast<uintptr_t>(inputs)) & 15) == 0;
   return wide ? launch_expand_as<E, K, S, MINB, true>(v, dview, counts, inputs, rounds, st)
               : launch_expand_as<E, K, S, MINB, false>(v, dview, counts, inputs, rounds, st);
@@ -272,6 +276,18 @@ int launch_expand_s(const ArrayView& v, const ArrayView* dview, const uint32_t* 
 int launch_push_expand(const ArrayView& v, const ArrayView* dview, const uint32_t* counts, const void* inputs,
                        uint32_t rounds, cudaStream_t st) {
   if (v.T > 512) return GGA_ERR_INVALID;
+  // Few LFVectors: the time is a block's chain of pushes, which more threads
+  // with one slot each shorten (20 LFVectors x 512 x 200 rounds, int32: 249 us
+  // with four slots, 160 with one, clear and flatten included).
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return GGA_ERR_CUDA;
+  if (v.L <= static_cast<uint32_t>(sms)) {
+    if (v.E == 4) return launch_expand_as<4, 4, 1, 2, false>(v, dview, counts, inputs, rounds, st);
+    if (v.E == 8) return launch_expand_as<8, 2, 1, 2, false>(v, dview, counts, inputs, rounds, st);
+    return launch_expand_as<16, 2, 1, 2, false>(v, dview, counts, inputs, rounds, st);
+  }
   if (v.E == 4) return launch_expand_s<4, 4, 4, 7>(v, dview, counts, inputs, rounds, st);
   if (v.E == 8) return launch_expand_s<8, 2, 4, 7>(v, dview, counts, inputs, rounds, st);
   return launch_expand_s<16, 2, 2, 4>(v, dview, counts, inputs, rounds, st);

@@ -1,4 +1,5 @@
-"""gga_push_expand loads a thread's slots as 128-bit words when T is a
+"""gga_push_expand gives a thread one slot or several by the number of
+LFVectors, and loads several as 128-bit words when T is a
 multiple of them and both buffers are 16-byte aligned, element by element
 otherwise, and each round's inputs ahead of the push that uses them: thread
 counts around the slots, rounds around the rounds of a push, buffers off
@@ -19,8 +20,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("E", [4, 8, 16])
 @pytest.mark.parametrize("T,R", [(1, 1), (2, 5), (3, 4), (4, 3), (30, 9), (128, 2), (132, 7), (509, 5), (512, 9)])
 @pytest.mark.parametrize("off", [0, 1])
-def test_slots_rounds_and_alignment(E, T, R, off):
-    L, B = 3, 8
+@pytest.mark.parametrize("L", [3, 200])               # one slot per thread up to one block per SM, then several
+def test_slots_rounds_and_alignment(E, T, R, off, L):
+    B = 8
     rng = np.random.default_rng(E * 1000 + T)
     counts = rng.integers(0, 3, size=(R, L, T)).astype(np.uint32)
     counts[0] = rng.integers(0, 9, size=(L, T))        # past two copies; a push past its stage for large T
