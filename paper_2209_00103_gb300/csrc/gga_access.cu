@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) write_kernel(ArrayView v, const uint64_t*
 
 constexpr uint32_t kWbinMaxBins = 256;
 constexpr uint64_t kWbinMin = 1ull << 20;        // smaller batches write directly
-constexpr uint64_t kWbinHeader = 4096;           // totals[256] u32 | cursors[256] u64 | valid u64
+constexpr uint64_t kWbinHeader = 4096;           // totals[256] u32 | cursors[256] u64 | valid u64 | any u32
 constexpr int kWbinThreads = 256;
 
 // The bins hold, per write, the element's offset inside its bin (32 bits:
@@ -152,6 +152,8 @@ __device__ __forceinline__ unsigned long long* wbin_cursors(uint8_t* scr) {
 __device__ __forceinline__ unsigned long long* wbin_valid(uint8_t* scr) {
   return reinterpret_cast<unsigned long long*>(scr + 3072);
 }
+// Binned reads: whether any tile was left to the scatter and the return.
+__device__ __forceinline__ uint32_t* rbin_any(uint8_t* scr) { return reinterpret_cast<uint32_t*>(scr + 3080); }
 
 template <int E>
 __global__ void __launch_bounds__(kWbinThreads) wbin_count_kernel(ArrayView v, const uint64_t* __restrict__ idx,
@@ -515,7 +517,7 @@ __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, c
   // elements and more (the bins hold 32-bit indices).
   const bool never = N * E < kRbinArrayMin || N > 0xFFFFFFFFull;
   for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x) h[b] = 0;
-  bool bad = false;
+  bool bad = false, left = false;   // left: some tile was not read here
   const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
   for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const uint64_t base = tile * kRbinTile;
@@ -548,6 +550,7 @@ __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, c
         if (i < n) __stcs(out + i, x[u]);
       }
     } else {
+      left = true;
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         if (g[u] < N) atomicAdd(&h[static_cast<uint32_t>(g[u] >> shift)], 1u);
@@ -556,6 +559,7 @@ __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, c
     }
   }
   if (bad) latch_error(v.status, GGA_ERR_OUT_OF_RANGE);
+  if (left && threadIdx.x == 0) *rbin_any(s.head) = 1;
   __syncthreads();
   uint32_t* tot = wbin_totals(s.head);
   for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x)
@@ -575,7 +579,8 @@ __global__ void __launch_bounds__(kWbinThreads, 4) rbin_scatter_kernel(ArrayView
   __shared__ alignas(16) uint16_t s_place[kTile];
   const uint64_t N = __ldg(v.offsets + v.L);
   const uint32_t shift = rbin_shift(N, E);
-  const uint64_t tiles = *wbin_valid(s.head) ? (n + kTile - 1) / kTile : 0;   // none when all were read directly
+  // None when every tile was read directly.
+  const uint64_t tiles = *rbin_any(s.head) ? (n + kTile - 1) / kTile : 0;
   for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     if (s.direct[tile]) continue;   // block-uniform
     for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x) h[b] = 0;
@@ -732,7 +737,9 @@ __global__ void __launch_bounds__(kWbinThreads, 6) rbin_return_kernel(RbinScratc
   uint8_t* s_bin = s_dyn + static_cast<size_t>(kTile) * E;                 // [kTile]
   __shared__ uint32_t at[kWbinMaxBins];
   __shared__ uint16_t off[kWbinMaxBins];
-  const uint64_t tiles = *wbin_valid(s.head) ? (n + kTile - 1) / kTile : 0;   // none when all were read directly
+  // None when every tile was read directly.  (The valid indices do not tell:
+  // a tile of indices out of range has none, and its outputs are zeroed here.)
+  const uint64_t tiles = *rbin_any(s.head) ? (n + kTile - 1) / kTile : 0;
   for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     if (s.direct[tile]) continue;   // block-uniform
     const uint64_t base = tile * kTile;
@@ -1180,7 +1187,7 @@ static void read_binned_as(const ArrayView& v, const uint64_t* idx, uint64_t n, 
   typedef typename Elem<E>::T T;
   RbinScratch s;
   rbin_layout<E>(n, static_cast<uint8_t*>(scratch), &s);
-  cudaMemsetAsync(s.head, 0, 1024, st);   // the totals
+  cudaMemsetAsync(s.head, 0, kWbinHeader, st);   // the totals, and no tile left
   const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
   const uint64_t cap = static_cast<uint64_t>(num_sms) * 4;   // the count: persistent blocks, one set of global additions each
   rbin_count_kernel<E><<<static_cast<unsigned>(tiles < cap ? tiles : cap), kWbinThreads, 0, st>>>(v, idx, n, s, static_cast<T*>(out));

@@ -75,6 +75,30 @@ def test_indices_out_of_range_read_zero_and_latch():
     g.close()
 
 
+@pytest.mark.parametrize("E", [4, 8])
+@pytest.mark.parametrize("kind", ["all", "tiles", "all but one"])
+def test_tiles_with_no_index_in_range_read_zero(E, kind):
+    """Scattered indices out of range, with no scattered tile beside them
+    that holds a valid one ("all but one": a single index of the batch)."""
+    g, n = grown(E, (300 << 20) // E, 600 << 20)
+    flat = g.flatten()
+    beyond = batch("uniform", n) + n
+    idx, bad = beyond, torch.ones(N_READS, dtype=torch.bool, device="cuda")
+    if kind == "tiles":
+        idx, bad = batch("ascending", n), ~bad
+        for tile in (0, 777, N_READS // 4096):        # the last one ends with the batch
+            bad[4096 * tile:4096 * (tile + 1)] = True
+        idx = torch.where(bad, beyond, idx)
+    elif kind == "all but one":
+        idx[N_READS // 2], bad[N_READS // 2] = n - 1, False
+    out = gga.elem_tensor(N_READS, E).fill_(-7)
+    g.read(idx, out)
+    assert g.last_error() == gga.GGA_ERR_OUT_OF_RANGE
+    assert int(out[bad].abs().max()) == 0
+    assert torch.equal(out[~bad], flat[idx[~bad]])
+    g.close()
+
+
 def test_small_and_empty_arrays_in_a_large_slab():
     g, n = grown(4, 5 << 20, 600 << 20)                # the L2 holds it
     flat = g.flatten()
