@@ -119,8 +119,10 @@ typedef struct {
  */
 int gga_pool_create(uint64_t pool_bytes, void* slab_dev, uint64_t min_bucket_bytes, void* stream, gga_pool* out);
 
-/* gga_pool_destroy -- free the pool (its arrays must be destroyed first).
- * Synchronizes the device. */
+/* gga_pool_destroy -- give the pool up: no array can be made in it any more
+ * (GGA_ERR_INVALID, also for a second call while arrays live).  Its memory is
+ * freed now, or with the last array in it, which until then work as before;
+ * a lent slab must last as long.  Synchronizes the device when it frees. */
 int gga_pool_destroy(gga_pool pool);
 
 /* gga_pool_info -- out4 (host) = {slab bytes, slab bytes handed out by the

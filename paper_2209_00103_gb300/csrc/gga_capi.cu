@@ -6,6 +6,7 @@
 // one -- the bucket slab.  Everything the operations compute runs in the
 // kernels of gga_insert.cu and gga_access.cu; this file checks arguments,
 // lays out memory and enqueues launches.
+#include <atomic>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -30,6 +31,8 @@ struct gga_pool_t {
   uint64_t* serve_records;  // device, made on first use by a batched append
   uint64_t serve_slots;
   std::mutex serve_mu;
+  std::atomic<uint32_t> users;   // its creator until gga_pool_destroy, and every array in it
+  std::atomic<bool> closed;      // gga_pool_destroy was called
 };
 
 struct gga_array {
@@ -129,6 +132,8 @@ int pool_make(uint64_t bytes, void* slab, uint64_t min_bucket_bytes, uint64_t lf
   pl->state = nullptr;
   pl->serve_records = nullptr;
   pl->serve_slots = 0;
+  pl->users = 1;
+  pl->closed = false;
   if (cudaGetDevice(&pl->device) != cudaSuccess) {
     delete pl;
     return GGA_ERR_CUDA;
@@ -181,6 +186,11 @@ int pool_free(gga_pool_t* pl) {
   delete pl;
   return rc;
 }
+
+// One user less; the last one frees the pool.  (An array's destruction returns
+// its buckets through the pool's state, so the state outlives its arrays
+// whatever the order of the destructions.)
+int pool_drop(gga_pool_t* pl) { return pl->users.fetch_sub(1) == 1 ? pool_free(pl) : GGA_OK; }
 
 // Bytes parked in a pool's queues and its bump high-water mark (synchronizes).
 int pool_read(gga_pool_t* pl, cudaStream_t st, uint64_t* bump, uint64_t* free_bytes) {
@@ -305,7 +315,8 @@ bool handle_parts(gga_handle h, ArrayView* view, InsertScratch* ins, int* device
 }
 }  // namespace gga
 
-// Metadata and scratch of a handle living in `pool`.
+// Metadata and scratch of a handle living in `pool`; a user of it from here
+// until gga_destroy (none on failure).
 static int handle_make(const gga_params* p, gga_pool_t* pool, bool own_pool, cudaStream_t st, gga_handle* out) {
   gga_array* h = new (std::nothrow) gga_array();
   if (!h) return GGA_ERR_CUDA;
@@ -335,6 +346,7 @@ static int handle_make(const gga_params* p, gga_pool_t* pool, bool own_pool, cud
     delete h;
     return GGA_ERR_CUDA;
   }
+  ++pool->users;
   char* m = static_cast<char*>(h->meta);
   gga::ArrayView& v = h->view;
   v.sizes = reinterpret_cast<uint64_t*>(m + o_sizes);
@@ -365,7 +377,7 @@ static int handle_make(const gga_params* p, gga_pool_t* pool, bool own_pool, cud
   // The insertion scratch is made by the first gga_insert that needs it.
   if (rc == GGA_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = GGA_ERR_CUDA;
   if (rc != GGA_OK) {
-    h->own_pool = false;   // the caller disposes of the pool
+    h->own_pool = true;   // it holds no buckets that a shared pool would get back
     gga_destroy(h);
     return rc;
   }
@@ -388,8 +400,8 @@ int gga_pool_create(uint64_t pool_bytes, void* slab_dev, uint64_t min_bucket_byt
 }
 
 int gga_pool_destroy(gga_pool pool) {
-  if (!pool) return GGA_ERR_INVALID;
-  return pool_free(pool);
+  if (!pool || pool->closed.exchange(true)) return GGA_ERR_INVALID;
+  return pool_drop(pool);
 }
 
 int gga_pool_info(gga_pool pool, uint64_t* out4, void* stream) {
@@ -413,12 +425,12 @@ int gga_create(const gga_params* p, void* pool_dev, void* stream, gga_handle* ou
   int rc = pool_make(p->pool_bytes, pool_dev, p->base_bucket * p->elem_bytes, p->n_lfvectors, st, &pool);
   if (rc != GGA_OK) return rc;
   rc = handle_make(p, pool, true, st, out);
-  if (rc != GGA_OK) pool_free(pool);
-  return rc;
+  const int rc_pool = pool_drop(pool);   // the array alone uses it
+  return rc != GGA_OK ? rc : rc_pool;
 }
 
 int gga_create_in_pool(const gga_params* p, gga_pool pool, void* stream, gga_handle* out) {
-  if (!out || !pool || !valid_params(p)) return GGA_ERR_INVALID;
+  if (!out || !pool || pool->closed || !valid_params(p)) return GGA_ERR_INVALID;
   if (gga::alloc_bytes_for(p->base_bucket * p->elem_bytes) < gga::alloc_bytes_for(pool->min_bucket_bytes))
     return GGA_ERR_INVALID;   // the pool does not serve this array's smallest bucket
   *out = nullptr;
@@ -579,12 +591,12 @@ int gga_destroy(gga_handle h) {
   if (!h) return GGA_ERR_INVALID;
   int rc = GGA_OK;
   // In a shared pool the buckets go back to its queues first.
-  if (!h->own_pool && h->pool && h->meta && gga::launch_clear(h->view, nullptr) != GGA_OK) rc = GGA_ERR_CUDA;
+  if (!h->own_pool && gga::launch_clear(h->view, nullptr) != GGA_OK) rc = GGA_ERR_CUDA;
   if (cudaDeviceSynchronize() != cudaSuccess) rc = GGA_ERR_CUDA;
   if (h->scratch && cudaFree(h->scratch) != cudaSuccess) rc = GGA_ERR_CUDA;
   if (h->wscratch && cudaFree(h->wscratch) != cudaSuccess) rc = GGA_ERR_CUDA;
   if (h->meta && cudaFree(h->meta) != cudaSuccess) rc = GGA_ERR_CUDA;
-  if (h->own_pool && h->pool && pool_free(h->pool) != GGA_OK) rc = GGA_ERR_CUDA;
+  if (pool_drop(h->pool) != GGA_OK) rc = GGA_ERR_CUDA;
   if (h->counted) workspace_handle_gone(h->device);
   delete h;
   return rc;

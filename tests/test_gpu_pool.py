@@ -59,6 +59,41 @@ def test_destroyed_buckets_are_reused():
     pool.close()
 
 
+@pytest.mark.parametrize("lent", [False, True])
+def test_arrays_outlive_their_pool(lent):
+    """A pool destroyed first goes with its last array; until then the arrays
+    grow and return buckets as before, and no other joins them."""
+    rng = np.random.default_rng(71)
+    slab = torch.empty(64 << 20, dtype=torch.uint8, device="cuda") if lent else None
+    pool = gga.GGAPool(64 << 20, 1024, slab)
+    h = pool.h
+    arrays = [(gga.GGArray(5, 64, 256, 4, shared_pool=pool), oracle.OracleGGArray(5, 64, 256, 4)) for _ in range(3)]
+    for closed in (False, True):
+        if closed:
+            pool.close()
+            with pytest.raises(gga.GGAError):
+                gga.gga_create_in_pool(5, 64, 256, 4, h)
+            with pytest.raises(gga.GGAError):
+                gga.gga_pool_destroy(h)
+        for g, o in arrays:
+            counts = random_counts(rng, 7, 5, 64)
+            values = packed_values(int(counts.sum()), 4)
+            g.insert(counts_to_dev(counts), values_to_dev(values, 4))
+            o.insert(counts, values)
+    info = gga.gga_pool_info(h)
+    assert info["bump_bytes"] > 0 and info["free_list_bytes"] == 0
+    arrays[1][0].close()
+    assert gga.gga_pool_info(h)["free_list_bytes"] > 0
+    for k in (0, 2):
+        assert_same_state(*arrays[k])
+    arrays[2][0].close()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    arrays[0][0].close()
+    if not lent:
+        assert torch.cuda.mem_get_info()[0] >= free + (64 << 20)   # the slab goes with the last array
+
+
 def test_pool_rejects_smaller_buckets():
     pool = gga.GGAPool(1 << 20, 4096)
     with pytest.raises(gga.GGAError):
