@@ -834,6 +834,7 @@ int launch_finalize(const ArrayView& v, cudaStream_t st) {
 // registers, 48 KB stage): 0.816 ms.  Other T use one virtual thread per
 // thread and a stage sized by T, so that small blocks fill the SM.
 constexpr int kGenVT = 4;
+constexpr int kGenStageMax = 49152;
 
 // Rounds per pass: counts without a small bound stage 4-byte marks.
 template <int E, int DIST>
@@ -867,10 +868,12 @@ static void launch_gen_as(const ArrayView& v, const GenParams& g, uint32_t R, cu
   // blocks of T = 512 fit an SM).
   const uint32_t esize = GenRounds<E, DIST>::kMarks ? 4 : E;
   const size_t smem = (static_cast<size_t>(rounds) * v.T * esize * 5 / 4 + 1024 + 15) & ~static_cast<size_t>(15);
+  // The limit is the kernel's, whatever the shape: host threads with arrays of
+  // other shapes launch it at the same time.
 #define GGA_GEN(K, KV, MT, MB)                                                                               \
   do {                                                                                                       \
     auto kern = gen_insert_kernel<E, K, KV, MT, MB, DIST>;                                                   \
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));         \
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGenStageMax);                   \
     kern<<<v.L, nt, smem, st>>>(v, g, R, static_cast<uint32_t>(smem));                                       \
   } while (0)
   if (!vt) GGA_GEN((GenRounds<E, DIST>::small), 1, 256, 6);

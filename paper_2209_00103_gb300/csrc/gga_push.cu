@@ -31,6 +31,7 @@ namespace gga {
 // geometric counts, clear and flatten included: 225 us with four, 139 with one).
 constexpr int kPushSlots = 4;
 constexpr uint32_t kPushSlotsMinT = 129;
+constexpr int kPushStageMax = 49152;
 
 // Stage of one push, in elements: T at one per thread and eight standard
 // deviations of a sum of T counts of variance up to 2 (a larger push stores
@@ -107,8 +108,9 @@ void launch_push_generated_as(const ArrayView& v, const ArrayView* dview, const 
 #define GGA_PUSH(D)                                                                                         \
   do {                                                                                                      \
     auto kern = slots == 1 ? push_generated_kernel<E, D, 1> : push_generated_kernel<E, D, kPushSlots>;      \
-    if (smem > 32768u)   /* with the count table the block's shared memory may pass 48 KB */                \
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));      \
+    if (smem > 32768u)   /* with the count table the block's shared memory may pass 48 KB; the limit is the \
+                            kernel's: other threads launch it for arrays of other shapes */                 \
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPushStageMax);               \
     kern<<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);                                               \
   } while (0)
   switch (g.dist) {
