@@ -13,6 +13,7 @@ struct GenParams {
   uint64_t seed, va, vb, vc;
   uint32_t dist, nthr, round0;
   uint32_t thr_sorted;   // 1: thr[0..nthr) ascending (set on the host)
+  float mean;            // of a draw's count
   uint32_t thr[GGA_MAX_THRESHOLDS];
 };
 
@@ -147,6 +148,12 @@ inline GenParams make_gen_params(const gga_gen_spec& spec) {
   for (int i = 0; i < GGA_MAX_THRESHOLDS; ++i) g.thr[i] = spec.thresholds[i];
   for (uint32_t i = 1; i < spec.n_thresholds && i < GGA_MAX_THRESHOLDS; ++i)
     if (g.thr[i] < g.thr[i - 1]) g.thr_sorted = 0;
+  g.mean = g.dist == GGA_DIST_BERNOULLI ? 0.5f : 1.0f;
+  if (g.dist == GGA_DIST_POISSON) {
+    double m = 0;
+    for (uint32_t k = 0; k < g.nthr; ++k) m += 1.0 - g.thr[k] / 4294967296.0;
+    g.mean = static_cast<float>(m);
+  }
   return g;
 }
 
@@ -263,8 +270,8 @@ __device__ inline void finalize_block(const ArrayView& v, const uint64_t* ins_ba
 // longest prefix of whole rounds that fits -- and takes the buckets
 // (Algorithm 2); then (synchronize) the values go to a shared-memory stage
 // at their positions and the block streams the stage to the buckets with
-// aligned 128-bit stores (a pass larger than the stage writes straight to
-// the buckets).  Elements past the target are the ones a round-by-round
+// aligned 128-bit stores (marked passes in as many parts as it takes, others SP
+// rounds at a time; where those do not fit, straight to the buckets).  Elements past the target are the ones a round-by-round
 // growth would clip (positions are round-major).  The LFVector's bucket
 // table is kept in shared memory, so the write-out finds a bucket's
 // address without a global load.
@@ -325,11 +332,12 @@ struct ThresholdTable {
 
   // #{k < nthr : u >= thr[k]} for the high word u of any draw.
   __device__ __forceinline__ uint32_t count(uint32_t nthr, uint32_t u) const {
-    uint32_t c = first_count(u);
-    if (u >= second) {
-      c = 0;
-      while (c < nthr && u >= thr[c]) ++c;
-    }
+    return u >= second ? slow_count(nthr, u) : first_count(u);
+  }
+
+  __device__ __forceinline__ uint32_t slow_count(uint32_t nthr, uint32_t u) const {
+    uint32_t c = 0;
+    while (c < nthr && u >= thr[c]) ++c;
     return c;
   }
 };
@@ -390,37 +398,44 @@ __device__ __forceinline__ void store_shared_if(typename Elem<E>::T* p, typename
 // Marks.  A thread whose counts have no small bound would store its elements
 // one by one in a loop that runs as often as the largest count of its warp,
 // most lanes idle, and compute every value there.  Such a pass stages one
-// 32-bit mark per non-empty draw instead, at its first element's stage index
-// si: ((si + 1) << 13) | (round of the pass << 10) | (virtual thread).  Marks
-// grow with si, so the draw an element belongs to is the largest mark at or
-// before it: a running maximum, which the write-out takes with a warp scan
-// and from which every lane computes its own elements' values.  Indices with
-// no mark hold zero.  Measured on GB300 for 2^25 draws (1024 LFVectors x 512
-// threads), elements stored in loops / by marks: geometric counts 219 / 117
-// us (4 bytes), 378 / 133 (8), 337 / 157 (16); Poisson 216 / 125, 278 / 139,
-// 296 / 161.
+// 32-bit mark per non-empty draw instead, at its first element's place:
+// (word + 1) << 13 | (round of the pass << 10) | (virtual thread), word being
+// the mark's index in the stage.  Marks grow with the place, so the draw an
+// element belongs to is the largest mark at or before it: a running maximum,
+// which the write-out takes with a warp scan and from which every lane computes
+// its own elements' values.  Words with no mark hold zero.  Measured on GB300
+// for 2^25 draws (1024 LFVectors x 512 threads), elements stored in loops / by
+// marks: geometric counts 219 / 117 us (4 bytes), 378 / 133 (8), 337 / 157
+// (16); Poisson 216 / 125, 278 / 139, 296 / 161.
+//
+// A pass of more elements than the stage holds (counts with a mean above the
+// one it is sized for) is written in parts, one stage after another: each has
+// the marks of its own stretch and of the kMarkHalo places before it, as a draw
+// has at most 63 elements.
 constexpr uint32_t kMarkBits = 13;   // 3 of the round, 10 of the virtual thread
-constexpr uint32_t kMarkMaxStage = (1u << (32 - kMarkBits)) - 2u;
+constexpr uint32_t kMarkHalo = 64;   // words before a part's first element
+constexpr uint32_t kMarkMaxStage = (1u << (32 - kMarkBits)) - kMarkHalo - 2u;
 // Consecutive elements of a lane in a step of the write-out: as many as its
 // 128-bit stores still cover whole 32-byte sectors with.  (Four records a
 // lane: 197 us against 161 for 2^25 draws on GB300.)
 constexpr uint32_t mark_group(int E) { return E == 16 ? 2 : 4; }
 
-// Writes the n elements of a marked pass (stage indices shv .. shv + n - 1,
-// position base at shv, shv = base mod mark_group(E)) to
-// their buckets; all threads of the block, after a barrier that follows the
-// marks.  Element m of draw (k, vt) is v0 + va * vt + vb * k + vc * m.  A warp
+// Writes n marked elements (places shv .. shv + n - 1, position base at shv, shv
+// = base mod mark_group(E); place i's mark is word kMarkHalo + i) to their
+// buckets; all threads of the block, after a barrier that follows the marks.
+// Element m of draw (k, vt) is v0 + va * vt + vb * k + vc * m.  A warp
 // takes a contiguous span of each bucket's part, a lane mark_group(E)
 // consecutive elements at a time.
 template <int E, typename V>
 __device__ __forceinline__ void marks_to_buckets(const uint64_t* tab, uint32_t log2B, uint64_t base, uint32_t n,
-                                                 uint32_t shv, const uint32_t* marks, V v0, V va, V vb, V vc,
+                                                 uint32_t shv, const uint32_t* words, V v0, V va, V vb, V vc,
                                                  uint32_t t, uint32_t nt) {
   typedef typename Elem<E>::T T;
   constexpr uint32_t G = mark_group(E);
   const uint32_t lane = t & 31, warp = t >> 5, nw = nt >> 5;
   const uint64_t gbeg = base - shv;
   const uint32_t end = n + shv;
+  const uint32_t* const marks = words + kMarkHalo;
   for (uint32_t s0 = 0; s0 < end;) {       // block-uniform: the part in one bucket
     uint32_t bb;
     uint64_t off;
@@ -432,13 +447,12 @@ __device__ __forceinline__ void marks_to_buckets(const uint64_t* tab, uint32_t l
     uint32_t c = s0 + warp * per * (32 * G);
     const uint32_t cend = min(s1, c + per * (32 * G));
     // The last mark before the span: a draw has at most 63 elements, so it
-    // lies within the 64 indices before (or there is none: the run's start).
+    // lies within the 64 places before (or there is none: the run's start).
     uint32_t carry = 0;
     if (c < cend) {
 #pragma unroll
-      for (uint32_t back = 0; back < 64; back += 32) {
-        const uint32_t d = back + 1 + lane;
-        const uint32_t w = d <= c ? marks[c - d] : 0u;
+      for (uint32_t back = 0; back < kMarkHalo; back += 32) {
+        const uint32_t w = words[c + (kMarkHalo - 1) - back - lane];
         if (carry == 0) carry = __reduce_max_sync(0xffffffffu, w);
       }
     }
@@ -470,7 +484,7 @@ __device__ __forceinline__ void marks_to_buckets(const uint64_t* tab, uint32_t l
       for (uint32_t e = 0; e < G; ++e) {
         const uint32_t m = max(w[e], ex);
         x.e[e] = gen_value<E>(v0 + va * static_cast<V>(m & 1023u) + vb * static_cast<V>((m >> 10) & 7u) +
-                              vc * static_cast<V>(si + e + 1 - (m >> kMarkBits)));
+                              vc * static_cast<V>(si + e + (kMarkHalo + 1) - (m >> kMarkBits)));
       }
       T* const p = dst + (si - s0);
       if (si >= shv && si + G <= s1) {
@@ -504,7 +518,7 @@ __device__ __forceinline__ void clear_marks(uint4* marks4, uint32_t n, uint32_t 
 // buckets; only when it does not, block 0 allocates behind a second cluster
 // barrier.  Draws, positions, clipping and the rounds kept when the pool
 // runs out are those of one block drawing the same rounds one after another.
-template <int E, int K, int KV, bool SEARCH = false, int DIST = -1, int C = 1>
+template <int E, int K, int KV, bool SEARCH = false, int DIST = -1, int C = 1, int SP = K>
 __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t l, uint32_t R, uint64_t target,
                                 GenShared& sh, uint4* stage4, uint32_t cap, bool* done) {
   typedef typename Elem<E>::T T;
@@ -542,9 +556,11 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
   // lane's group); `dirty` marks of the last pass are still set.
   constexpr bool kMarks = !(DIST >= 0 && max_count<DIST>() > 0 && max_count<DIST>() <= 2);
   constexpr uint32_t kGroup = mark_group(E);
-  uint32_t* const marks = reinterpret_cast<uint32_t*>(stage4);
-  const uint32_t mark_cap = v.B < kGroup ? 0u : min(cap * static_cast<uint32_t>(E / 4) - 32 * kGroup, kMarkMaxStage);
-  // (a warp's last step of the write-out reads up to 32 groups past the end)
+  uint32_t* const words = reinterpret_cast<uint32_t*>(stage4);
+  // Elements a part holds: whole groups, beside the halo and the 32 groups that a
+  // warp's last step of the write-out reads past the end.
+  const uint32_t part =
+      v.B < kGroup ? 0u : min(cap * static_cast<uint32_t>(E / 4) - kMarkHalo - 32 * kGroup, kMarkMaxStage) & ~(kGroup - 1u);
   uint32_t dirty = 0;
   if (kMarks) clear_marks(stage4, cap * (E / 4), t0, NT);   // (the pass's barriers come before the first mark)
   uint32_t r0 = 0;   // the pass's first round
@@ -589,9 +605,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
           const uint32_t h = q / KV, i = q % KV;
           const uint64_t r = static_cast<uint64_t>(g.round0) + rb0 + 2 * j + h;
           const uint32_t u = splitmix_mix_hi(RoundDraws(g.seed, gfirst + i).state(r));
-          uint32_t c = 0;
-          while (c < g.nthr && u >= sh.thr.thr[c]) ++c;
-          both |= static_cast<uint64_t>(c) << (32 * h + 8 * i);
+          both |= static_cast<uint64_t>(sh.thr.slow_count(g.nthr, u)) << (32 * h + 8 * i);
         }
         w[0] = static_cast<uint32_t>(both);
         w[1] = static_cast<uint32_t>(both >> 32);
@@ -712,30 +726,73 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
       commit = sh.commit;
       next = base + commit;
     }
-    // Stage index = pass position + shv.
-    const bool marked = kMarks && sh.rb[K] + static_cast<uint32_t>(base & (kGroup - 1)) <= mark_cap;
-    const uint32_t shv = static_cast<uint32_t>(base & ((marked ? kGroup : VEC) - 1));
-    const bool staged = !marked && commit + shv <= cap;
-    // Fast path (block-uniform): the whole pass is kept and staged, so no
-    // element needs the clipping test or the bucket math.
-    const bool whole = !kMarks && staged && commit == sh.rb[K];
+    const bool marked = kMarks && part > 0;
+    // Fast path (block-uniform): the whole pass is kept and staged, SP rounds at
+    // a time, so no element needs the clipping test or the bucket math.
+    bool whole = !kMarks && commit == sh.rb[K];
+#pragma unroll
+    for (int k = 0; k < K; k += SP) whole = whole && sh.rb[k + SP] - sh.rb[k] + VEC - 1 <= cap;
     typedef typename std::conditional<E == 4, uint32_t, uint64_t>::type V;
     if (marked) {
+      // Place (stage index) = pass position + shv.
+      const uint32_t shv = static_cast<uint32_t>(base & (kGroup - 1));
+      const uint32_t end = commit + shv, most = sh.rb[K] + shv;
+      // More than one part: the thread's offsets and counts in local memory, so
+      // that no register holds them over the write-out of a part.
+      uint32_t lex[KP], lcw[KC];
+      if (most <= part) {
 #pragma unroll
-      for (int j = 0; j < KP; ++j) {
-        const uint32_t ex = sh.wt[j][warp] + exw[j];
+        for (int j = 0; j < KP; ++j) {
+          const uint32_t ex = sh.wt[j][warp] + exw[j];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t k = 2 * j + h;
-          uint32_t si = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu) + shv;
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t k = 2 * j + h;
+            uint32_t at = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu) + shv + kMarkHalo;
 #pragma unroll
-          for (int i = 0; i < KV; ++i) {
-            const uint32_t c = count_of(k, i);
-            if (c) marks[si] = ((si + 1) << kMarkBits) + ((k << 10) + static_cast<uint32_t>(tfirst) + i);
-            si += c;
+            for (int i = 0; i < KV; ++i) {
+              if (i > 0 && static_cast<uint32_t>(i) >= kv) break;
+              const uint32_t c = count_of(k, i);
+              if (c) words[at] = ((at + 1) << kMarkBits) + ((k << 10) + static_cast<uint32_t>(tfirst) + i);
+              at += c;
+            }
           }
         }
+      } else {
+#pragma unroll
+        for (int j = 0; j < KP; ++j) lex[j] = sh.wt[j][warp] + exw[j];
+#pragma unroll
+        for (int q = 0; q < KC; ++q) lcw[q] = cw[q];
       }
+      for (uint32_t lo = 0;;) {   // one part after another, mostly one
+        if (most > part) {
+#pragma unroll 1
+          for (uint32_t k = 0; k < K && sh.rb[k] + shv < lo + part; ++k) {
+            if (sh.rb[k + 1] + shv + kMarkHalo <= lo) continue;   // block-uniform, as the loop's end: rounds of this part
+            const uint32_t w = lcw[k * KV / 4] >> (8 * (k * KV % 4));
+            uint32_t at = sh.rb[k] + ((lex[k / 2] >> (16 * (k % 2))) & 0xFFFFu) + shv + kMarkHalo - lo;
+#pragma unroll
+            for (int i = 0; i < KV; ++i) {
+              const uint32_t c = (w >> (8 * i)) & 0xFFu;
+              if (c && at < part + kMarkHalo)
+                words[at] = ((at + 1) << kMarkBits) + ((k << 10) + static_cast<uint32_t>(tfirst) + i);
+              at += c;
+            }
+          }
+        }
+        __syncthreads();
+        const uint32_t at0 = lo ? 0u : shv;
+        if (commit)
+          marks_to_buckets<E, V>(sh.tab, v.log2B, base - shv + lo + at0, min(part, end - lo) - at0, at0, words,
+                                 static_cast<V>(g.va * (static_cast<uint64_t>(l) * v.T) +
+                                                g.vb * (static_cast<uint64_t>(g.round0) + rb0)),
+                                 static_cast<V>(g.va), static_cast<V>(g.vb), static_cast<V>(g.vc), t0, NT);
+        lo += part;
+        if (lo >= end) break;
+        __syncthreads();   // the part is written out
+        clear_marks(stage4, kMarkHalo + part, t0, NT);
+        __syncthreads();
+      }
+      dirty = kMarkHalo + min(most, part);
     } else {
       // Element m of virtual thread i in round k: va * gid + vb * round + vc * m
       // (a 4-byte element keeps the low 32 bits, which 32-bit arithmetic gives
@@ -745,14 +802,15 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
       const V va = static_cast<V>(g.va), vb = static_cast<V>(g.vb), vc = static_cast<V>(g.vc);
       const V vr = va * static_cast<V>(gfirst) + vb * static_cast<V>(static_cast<uint64_t>(g.round0) + rb0);
       if (whole) {
-        T* const st0 = stage + shv;
 #pragma unroll
-        for (int j = 0; j < KP; ++j) {
-          const uint32_t ex = sh.wt[j][warp] + exw[j];
+        for (int k0 = 0; k0 < K; k0 += SP) {
+          const uint32_t first = sh.rb[k0], n = sh.rb[k0 + SP] - first;
+          const uint32_t at = static_cast<uint32_t>(base + first) & (VEC - 1);
+          if (k0 > 0) __syncthreads();   // the part before is written out
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t k = 2 * j + h;
-            T* st = st0 + sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
+          for (int k = k0; k < k0 + SP; ++k) {
+            const uint32_t ex = sh.wt[k / 2][warp] + exw[k / 2];
+            T* st = stage + (sh.rb[k] - first + at + ((ex >> (16 * (k % 2))) & 0xFFFFu));
             const V v0 = vr + vb * static_cast<V>(k);
 #pragma unroll
             for (int i = 0; i < KV; ++i) {
@@ -764,47 +822,52 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
               st += c;
             }
           }
+          __syncthreads();
+          if (n) stage_to_buckets<T>(sh.tab, v.log2B, v.B, base + first, n, at, stage4, t0, NT);
         }
       } else {
-        // A clipped or unstaged pass: element by element.
+        // A clipped pass, or one that does not fit: SP rounds after SP rounds,
+        // element by element, straight to the buckets where they do not fit.
+        uint32_t lex[KP], lcw[KC];
 #pragma unroll
-        for (int j = 0; j < KP; ++j) {
-          const uint32_t ex = sh.wt[j][warp] + exw[j];
+        for (int j = 0; j < KP; ++j) lex[j] = sh.wt[j][warp] + exw[j];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t k = 2 * j + h;
-            uint32_t q = sh.rb[k] + ((ex >> (16 * h)) & 0xFFFFu);
-#pragma unroll
-            for (int i = 0; i < KV; ++i) {
-              const uint32_t c = count_of(k, i);
+        for (int q = 0; q < KC; ++q) lcw[q] = cw[q];
+        dirty = 0;
+        uint32_t k = 0;
+#pragma unroll 1
+        do {
+          const uint32_t first = sh.rb[k], n = first < commit ? min(sh.rb[k + SP], commit) - first : 0u;
+          const uint32_t at = static_cast<uint32_t>(base + first) & (VEC - 1);
+          const bool staged = n + at <= cap;
+          if (k > 0) __syncthreads();   // the part before is written out
+#pragma unroll 1
+          for (const uint32_t kend = k + SP; k < kend; ++k) {
+            uint32_t q = sh.rb[k] - first + ((lex[k / 2] >> (16 * (k % 2))) & 0xFFFFu);
+#pragma unroll 1
+            for (uint32_t i = 0; i < kv; ++i) {
+              const uint32_t c = (lcw[(k * KV + i) / 4] >> (8 * ((k * KV + i) % 4))) & 0xFFu;
               V val = vr + va * static_cast<V>(i) + vb * static_cast<V>(k);
               for (uint32_t m = 0; m < c; ++m, ++q, val += vc) {
-                if (q >= commit) continue;
+                if (q >= n) continue;
                 if (staged) {
-                  stage[q + shv] = gen_value<E>(val);
+                  stage[q + at] = gen_value<E>(val);
                 } else {
                   uint32_t bb;
                   uint64_t off;
-                  bucket_of(base + q, v.log2B, bb, off);
+                  bucket_of(base + first + q, v.log2B, bb, off);
                   reinterpret_cast<T*>(sh.tab[bb])[off] = gen_value<E>(val);
                 }
               }
             }
           }
-        }
+          __syncthreads();
+          if (staged && n) {
+            stage_to_buckets<T>(sh.tab, v.log2B, v.B, base + first, n, at, stage4, t0, NT);
+            dirty = max(dirty, (n + at) * static_cast<uint32_t>(E / 4));
+          }
+        } while (k < K && sh.rb[k] < commit);
       }
-    }
-    __syncthreads();
-    if (marked) {
-      dirty = sh.rb[K] + shv;
-      if (commit)
-        marks_to_buckets<E, V>(sh.tab, v.log2B, base, commit, shv, marks,
-                               static_cast<V>(g.va * (static_cast<uint64_t>(l) * v.T) +
-                                              g.vb * (static_cast<uint64_t>(g.round0) + rb0)),
-                               static_cast<V>(g.va), static_cast<V>(g.vb), static_cast<V>(g.vc), t0, NT);
-    } else {
-      dirty = staged ? (commit + shv) * (E / 4) : 0u;
-      if (staged && commit) stage_to_buckets<T>(sh.tab, v.log2B, v.B, base, commit, shv, stage4, t0, NT);
     }
     // No barrier here: the next pass writes the stage, sh.wt, sh.rb and
     // sh.commit only after its first two barriers, which every thread reaches

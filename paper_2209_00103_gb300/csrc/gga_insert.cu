@@ -28,6 +28,8 @@
 // leader thread reserves and allocates (Algorithms 1-2), __syncthreads is the
 // synchronize() of Algorithm 1, and the block writes the run.  K rounds share
 // one scan pass to amortise the barriers.
+#include <algorithm>
+
 #include "gga_core.cuh"
 #include "gga_gen.cuh"
 
@@ -822,19 +824,25 @@ int launch_finalize(const ArrayView& v, cudaStream_t st) {
 
 // A pass's elements (or marks) are staged in shared memory, its rounds
 // chosen so that at one element per thread and round a pass fills about
-// two thirds of the stage; a pass that does not fit writes directly, element
-// by element, which costs twice the instructions (8-byte uniform counts at 8
-// rounds in a 24 KB stage: 126 per draw and 250 us for 2^25 draws, at 4
-// rounds 87 us).  T > 256 is played by blocks of T / 4 threads, four
+// two thirds of the stage (8-byte uniform counts at 8 rounds, which do not fit
+// a stage of 24 KB and go out element by element: 126 instructions per draw and
+// 250 us for 2^25 draws, at 4 rounds 87 us).  Marks have no such limit: counts
+// with a mean above 1.25 leave in several parts a pass (grow_passes).
+// T > 256 is played by blocks of T / 4 threads, four
 // virtual threads each: one scan word and one share of every barrier serve
 // them, and eight blocks (four for T > 512) are resident per SM.  Measured
 // on GB300 for the paper-shaped workload (1024 LFVectors x 512 threads x 512
 // rounds, int32) when this was chosen: 128 threads x 4, 8 per SM: 0.737 ms
 // (0.47 ms now); 256 x 2, 4 per SM: 0.753 ms; 512 x 1, 3 per SM (40
 // registers, 48 KB stage): 0.816 ms.  Other T use one virtual thread per
-// thread and a stage sized by T, so that small blocks fill the SM.
+// thread and a stage sized by T and the counts' mean, so that small blocks fill
+// the SM (five of 256 threads with 48 registers: 2^24 Poisson draws at T = 256,
+// int64, 128 us; six with 40: 134).  Measured for 2^24 Poisson draws of mean 3,
+// int32, a stage for mean 1 and the rest element by element / now: T = 256
+// 307 / 153 us, T = 512 405 / 143, T = 1024 353 / 149.
 constexpr int kGenVT = 4;
 constexpr int kGenStageMax = 49152;
+constexpr size_t kGenStageSmall = 38 << 10;   // with five blocks of 256 threads per SM
 
 // Rounds per pass: counts without a small bound stage 4-byte marks.
 template <int E, int DIST>
@@ -863,11 +871,16 @@ static void launch_gen_as(const ArrayView& v, const GenParams& g, uint32_t R, cu
   const uint32_t rounds = vt ? GenRounds<E, DIST>::value : GenRounds<E, DIST>::small;
   const uint32_t per = vt ? kGenVT : 1;
   const uint32_t nt = ((v.T + per - 1) / per + 31) / 32 * 32;
-  // A pass of one element per thread and round and a quarter more, in
-  // whole 16-byte words, and a warp's overhang (41,984 bytes at most; eight
-  // blocks of T = 512 fit an SM).
+  // A pass of one element per thread and round and a quarter more, in whole
+  // 16-byte words, and a warp's overhang (41,984 bytes at most; eight blocks of
+  // T = 512 fit an SM).  Counts with a larger mean get room for their own pass
+  // while as many blocks fit the SM; beyond that a pass goes out in parts.
   const uint32_t esize = GenRounds<E, DIST>::kMarks ? 4 : E;
-  const size_t smem = (static_cast<size_t>(rounds) * v.T * esize * 5 / 4 + 1024 + 15) & ~static_cast<size_t>(15);
+  const size_t one = static_cast<size_t>(rounds) * v.T * esize * 5 / 4 + 1024;
+  size_t smem = one;
+  if (!vt && g.mean > 1.0f)
+    smem = std::max(one, std::min(static_cast<size_t>(g.mean * static_cast<float>(one)), kGenStageSmall * nt / 256));
+  smem = (smem + 15) & ~static_cast<size_t>(15);
   // The limit is the kernel's, whatever the shape: host threads with arrays of
   // other shapes launch it at the same time.
 #define GGA_GEN(K, KV, MT, MB)                                                                               \
@@ -876,7 +889,7 @@ static void launch_gen_as(const ArrayView& v, const GenParams& g, uint32_t R, cu
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGenStageMax);                   \
     kern<<<v.L, nt, smem, st>>>(v, g, R, static_cast<uint32_t>(smem));                                       \
   } while (0)
-  if (!vt) GGA_GEN((GenRounds<E, DIST>::small), 1, 256, 6);
+  if (!vt) GGA_GEN((GenRounds<E, DIST>::small), 1, 256, 5);
   else if (v.T <= 512) GGA_GEN((GenRounds<E, DIST>::value), kGenVT, 128, 8);
   else GGA_GEN((GenRounds<E, DIST>::value), kGenVT, 256, 4);
 #undef GGA_GEN
