@@ -78,17 +78,22 @@ struct gga_batch_t {
 
 namespace {
 
-// Passes one block takes to draw an LFVector of `target` elements: rounds
-// at the distribution's mean count, batch_rounds a pass.
-uint64_t expected_passes(const gga::BatchJob& J, uint64_t target) {
-  double mean = J.g.dist == GGA_DIST_BERNOULLI ? 0.5 : 1.0;
-  if (J.g.dist == GGA_DIST_POISSON) {
-    mean = 0;
-    for (uint32_t k = 0; k < J.g.nthr; ++k) mean += 1.0 - J.g.thr[k] / 4294967296.0;
-  }
-  const double per_pass = mean * J.v.T * gga::batch_rounds(static_cast<int>(J.v.E), J.g.dist);
-  const double p = per_pass > 0 ? static_cast<double>(target) / per_pass : 1e12;
-  return p < 1e12 ? static_cast<uint64_t>(p) + 1 : static_cast<uint64_t>(1e12);
+// Rounds that draw an LFVector of `target` elements.
+double expected_rounds(const gga::BatchJob& J, uint64_t target) {
+  const double per_round = static_cast<double>(J.g.mean) * J.v.T;
+  return per_round > 0 ? std::min(static_cast<double>(target) / per_round + 1, 1e12) : 1e12;
+}
+
+// Its cost in microseconds of a whole GB300 per 2^24 draws and elements, from
+// generated insertions of means 0.5 and 1 at T = 1024 (idle threads draw too).
+// The forms' shares of the chip follow it: by passes, which hold two to eight
+// rounds, 300 arrays of the three payloads took 492 us (T = 1024, uniform
+// counts, 131K elements per LFVector), by cost 262.
+double expected_cost(const gga::BatchJob& J, uint64_t target, double rounds) {
+  const uint32_t kv = (J.v.T + gga::kBatchThreads - 1) / gga::kBatchThreads;
+  const double draw = J.g.dist > GGA_DIST_UNIFORM3 ? 70 : 40;
+  const double elem = J.v.E == 4 ? 15 : (J.v.E == 8 ? 22 : 35);
+  return rounds * gga::kBatchThreads * kv * draw + static_cast<double>(target) * elem;
 }
 
 void launch_form(const gga::BatchLaunch& a, cudaStream_t st) {
@@ -135,7 +140,7 @@ int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, g
   *out = nullptr;
   struct Item {
     uint32_t form;
-    uint64_t passes;
+    double rounds, cost;
     gga::BatchItem it;
   };
   std::vector<gga::BatchJob> hj(n_jobs);
@@ -156,20 +161,22 @@ int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, g
     const uint32_t form = (E == 4 ? 0u : (E == 8 ? 4u : 8u)) + sp.dist;
     for (uint32_t l = 0; l < L; ++l) {
       const uint64_t tl = jobs[j].target / L + (l < jobs[j].target % L ? 1 : 0);
-      if (tl) hi.push_back({form, expected_passes(hj[j], tl), gga::BatchItem{j, l}});
+      if (!tl) continue;
+      const double rounds = expected_rounds(hj[j], tl);
+      hi.push_back({form, rounds, expected_cost(hj[j], tl, rounds), gga::BatchItem{j, l}});
     }
     if (std::find(hp.begin(), hp.end(), hj[j].v.pool) == hp.end()) hp.push_back(hj[j].v.pool);
   }
   // Form by form, longest chains first: the tickets then balance
   // the tail.
   std::stable_sort(hi.begin(), hi.end(), [](const Item& a, const Item& b) {
-    return a.form != b.form ? a.form < b.form : a.passes > b.passes;
+    return a.form != b.form ? a.form < b.form : a.rounds > b.rounds;
   });
   std::vector<gga::BatchItem> items(hi.size());
-  uint64_t sum = 0;
+  double sum = 0;
   for (size_t i = 0; i < hi.size(); ++i) {
     items[i] = hi[i].it;
-    sum += hi[i].passes;
+    sum += hi[i].cost;
   }
 
   gga_batch_t* b = new (std::nothrow) gga_batch_t();   // zeroed
@@ -177,30 +184,34 @@ int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, g
   b->n_jobs = n_jobs;
   b->n_items = static_cast<uint32_t>(items.size());
   b->n_pools = static_cast<uint32_t>(hp.size());
-  // A form's items grown by clusters: those whose chain is long enough for
-  // the cluster's larger passes (of which the target clips the last), and
-  // longer than a quarter of a block's average load over the whole batch.
-  // (The rest then ends within a quarter of that load.)
+  // A form's items grown by clusters (`big`, the first ones): those whose
+  // chain is long enough for the cluster's larger passes -- four of them, or
+  // one while the items leave three quarters of the blocks idle -- and that
+  // cost more than a quarter of a block's average load over the whole batch.
+  // (The rest then ends within a quarter of that load.)  Measured on GB300, four
+  // / one: 30 arrays of 32 to 131K elements per LFVector at T = 1024, uniform
+  // counts, 117 / 63 us; 300 arrays at T = 256 462 / 629.
   struct Form {
     uint32_t id, first, n, big;
-    uint64_t passes, big_passes;
+    double cost, big_cost;
   };
   std::vector<Form> forms;
-  uint64_t big_sum = 0;
+  double big_sum = 0;
   const uint64_t blocks = static_cast<uint64_t>(std::max(num_sms, 1)) * gga::kBatchMinBlocks;
+  const double least = (hi.size() * 4 <= blocks ? 1 : 4) * gga::kBatchCluster * gga::kBatchRounds;
   for (uint32_t i = 0; i < b->n_items; ++i) {
     if (forms.empty() || forms.back().id != hi[i].form) forms.push_back({hi[i].form, i, 0, 0, 0, 0});
     Form& f = forms.back();
-    if (f.big == f.n && hi[i].passes >= 4 * gga::kBatchCluster && hi[i].passes * 4 > sum / blocks) {
+    if (f.big == f.n && hi[i].rounds >= least && hi[i].cost * 4 > sum / static_cast<double>(blocks)) {
       ++f.big;
-      f.big_passes += hi[i].passes;
-      big_sum += hi[i].passes;
+      f.big_cost += hi[i].cost;
+      big_sum += hi[i].cost;
     }
     ++f.n;
-    f.passes += hi[i].passes;
+    f.cost += hi[i].cost;
   }
   // The form with most work first.
-  std::stable_sort(forms.begin(), forms.end(), [](const Form& x, const Form& y) { return x.passes > y.passes; });
+  std::stable_sort(forms.begin(), forms.end(), [](const Form& x, const Form& y) { return x.cost > y.cost; });
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = GGA_OK;
   if (cudaMalloc(&b->jobs, sizeof(gga::BatchJob) * (n_jobs ? n_jobs : 1)) != cudaSuccess ||
@@ -225,10 +236,10 @@ int gga_batch_create(const gga_batch_job* jobs, uint32_t n_jobs, void* stream, g
       const uint32_t n = clusters ? f.big : f.n - f.big, unit = clusters ? gga::kBatchCluster : 1;
       if (n == 0) continue;
       // As many units as are resident at once -- for the cluster kernels the
-      // form's share of them by its passes, so that every form's longest
+      // form's share of them by its cost, so that every form's longest
       // chains start at once -- or as there are items.
       uint64_t fit = static_cast<uint64_t>(num_sms) * blocks_per_sm(f.id, clusters != 0) / unit;
-      if (clusters) fit = fit * f.big_passes / big_sum;
+      if (clusters) fit = static_cast<uint64_t>(static_cast<double>(fit) * (f.big_cost / big_sum) + 0.5);
       const uint32_t i = b->n_launches++;
       b->launch[i] = gga::BatchLaunch{f.id, clusters != 0, b->jobs, b->items + f.first + (clusters ? 0 : f.big),
                                       n, b->tickets + i, static_cast<uint32_t>(std::max<uint64_t>(1, std::min<uint64_t>(fit, n))) * unit};

@@ -10,31 +10,27 @@
 namespace gga {
 
 // Threads per block, virtual threads per thread (T <= kBatchThreads *
-// kBatchKV = 1024) and resident blocks per SM.
-#ifndef GGA_BATCH_THREADS
-#define GGA_BATCH_THREADS 256
-#endif
-#ifndef GGA_BATCH_CLUSTER
-#define GGA_BATCH_CLUSTER 4
-#endif
-constexpr int kBatchThreads = GGA_BATCH_THREADS;
-constexpr int kBatchKV = 1024 / kBatchThreads;
-constexpr int kBatchMinBlocks = 1024 / kBatchThreads;
-constexpr uint32_t kBatchStageBytes = 160 * kBatchThreads;
+// kBatchKV = 1024; a block draws for ceil(T / kBatchThreads) of them) and
+// resident blocks per SM.  Drawing for all four whatever T was, arrays of T = 256
+// took 1300 us where it now takes 550 (300 arrays of lognormal sizes).
+constexpr int kBatchThreads = 256;
+constexpr int kBatchKV = 4;
+constexpr int kBatchMinBlocks = 4;
+constexpr uint32_t kBatchStageBytes = 40960;
 constexpr uint32_t kBatchMaxRounds = 1u << 20;
 constexpr int kBatchLaunches = 24;   // a cluster and a block kernel per (payload size, distribution)
 // Blocks of a cluster.  An LFVector's rounds follow one another, so one block
 // grows a large one in one long chain of passes: for 1024 arrays of lognormal
 // sizes (2.1e8 elements) the longest chains, 256 passes, took 1.9 ms while the
-// blocks' average load is a third of that.  The largest items (n_big of them,
-// chosen in gga_batch_create) are therefore grown by whole clusters, one pass
+// blocks' average load is a third of that.  The largest items (chosen in
+// gga_batch_create) are therefore grown by whole clusters, one pass
 // of kBatchCluster times the rounds at a time; the others by single blocks,
 // which take the SMs as the clusters finish.  Measured on GB300 for that
 // batch, growth with its reads and flattens: 2.19 ms by single blocks, 1.36
-// with clusters of 4, 1.37 of 8 (a larger part of the last pass is clipped),
-// 1.96 of 2; blocks of 512 threads with two virtual threads per thread and
-// clusters of 4: 1.54.  (Of the 1.36 ms 0.23 are the reads and flattens.)
-constexpr int kBatchCluster = GGA_BATCH_CLUSTER;
+// with clusters of 4 (1.25 now), 1.37 of 8 (a larger part of the last pass is
+// clipped), 1.96 of 2; blocks of 512 threads with two virtual threads per thread
+// and clusters of 4: 1.54.  (Of the 1.25 ms 0.2 are the reads and flattens.)
+constexpr int kBatchCluster = 4;
 
 struct BatchJob {
   ArrayView v;
@@ -47,12 +43,11 @@ struct BatchItem {
   uint32_t l;
 };
 
-// Rounds per pass: a pass of T <= 1024 threads at one element per thread
-// and round then averages 32 KB of the 40 KB stage.  Bernoulli and uniform
-// counts stage their elements, the others 4-byte marks.
-__host__ __device__ constexpr int batch_rounds(int E, uint32_t dist) {
-  return E == 4 ? 8 : (dist > GGA_DIST_UNIFORM3 ? (E == 8 ? 8 : 4) : (E == 8 ? 4 : 2));
-}
+// Rounds per pass.  Bernoulli and uniform counts stage their elements,
+// batch_staged rounds at a time (at T = 1024 threads and one element per thread
+// and round 32 KB of the 40 KB stage), the others 4-byte marks.
+constexpr int kBatchRounds = 8;
+constexpr int batch_staged(int E, uint32_t dist) { return dist > GGA_DIST_UNIFORM3 ? kBatchRounds : 32 / E; }
 
 // Grow LFVector l of job J to its share of the target: rounds of in-thread
 // insertions in passes of K (grow_passes in gga_gen.cuh), clipped at the
@@ -68,7 +63,7 @@ __device__ __forceinline__ void grow_item(const BatchJob* __restrict__ jobs, con
   const ArrayView& v = s_job.v;
   const uint64_t target = s_job.target / v.L + (item.l < s_job.target % v.L ? 1 : 0);
   bool done;
-  const uint32_t drawn = grow_passes<E, batch_rounds(E, DIST), kBatchKV, true, DIST, C>(
+  const uint32_t drawn = grow_passes<E, kBatchRounds, kBatchKV, true, DIST, C, batch_staged(E, DIST)>(
       v, s_job.g, item.l, kBatchMaxRounds, target, sh, stage, kBatchStageBytes / E, &done);
   if (threadIdx.x == 0 && !done && drawn >= kBatchMaxRounds) latch_error(v.status, GGA_ERR_TIMEOUT);
   __syncthreads();

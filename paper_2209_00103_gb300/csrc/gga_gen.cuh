@@ -356,7 +356,19 @@ struct GenShared {
   // parity) and the allocated buckets after a growth.
   uint32_t peer_total[2][kMaxCluster];
   uint32_t peer_nb;
+  uint32_t rounds;            // rounds the cluster's next pass takes
 };
+
+// Rounds a cluster's pass takes: its C K, or as many as the `rem` elements up
+// to the target should need (a draw's mean and four deviations of their sum;
+// if they do not suffice, another pass follows).  Blocks with none of them
+// draw nothing.  (Without it the last pass draws half its rounds for nothing,
+// an eighth of what a chain of 16 single passes draws.)
+__device__ __forceinline__ uint32_t pass_rounds(uint64_t rem, float per_round, uint32_t most) {
+  const float r = static_cast<float>(rem);
+  const float n = (r + 4.0f * sqrtf(r)) / per_round + 1.0f;   // (a mean of zero: inf)
+  return n < static_cast<float>(most) ? static_cast<uint32_t>(n) : most;
+}
 
 // Thread-block cluster operations (the blocks of a cluster are co-resident,
 // so their barrier always completes).
@@ -511,7 +523,8 @@ __device__ __forceinline__ void clear_marks(uint4* marks4, uint32_t n, uint32_t 
 // gen_count_state (-1: g.dist at run time).
 //
 // C > 1: the C blocks of a cluster grow the LFVector together, block q of a
-// pass drawing its rounds q K .. q K + K - 1 of the pass's C K.  The blocks
+// pass drawing its rounds q K .. q K + K - 1 of the pass's C K (the last pass
+// takes fewer: pass_rounds).  The blocks
 // store their totals into one another's shared memory, one cluster barrier
 // takes the place of the pass's second block barrier, and every block then
 // knows where its run starts and whether the pass stays inside the allocated
@@ -542,6 +555,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
     sh.base = v.sizes[l];
     sh.nb = v.nbuckets[l];
     sh.stop = sh.base >= target ? 2 : 0;
+    if constexpr (C > 1) sh.rounds = pass_rounds(target - sh.base, g.mean * static_cast<float>(v.T), C * K);
   }
   {
     const uint32_t nb0 = v.nbuckets[l];
@@ -566,7 +580,8 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
   uint32_t r0 = 0;   // the pass's first round
   while (r0 < R && sh.stop == 0) {
     const uint32_t rb0 = r0 + rank * K;   // this block's first round of the pass
-    const uint32_t kk = rb0 < R ? min(static_cast<uint32_t>(K), R - rb0) : 0u;
+    const uint32_t rend = C > 1 ? r0 + min(R - r0, sh.rounds) : R;   // rounds before this one are drawn
+    const uint32_t kk = rb0 < rend ? min(static_cast<uint32_t>(K), rend - rb0) : 0u;
     // exw: the thread's offsets in its warp, two rounds per word; cw: its
     // counts, one byte each (round k, virtual thread i at byte k * KV + i).
     constexpr int KC = (K * KV + 3) / 4;
@@ -574,53 +589,58 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
 #pragma unroll
     for (int q = 0; q < KC; ++q) cw[q] = 0;
     auto count_of = [&](uint32_t k, uint32_t i) { return (cw[(k * KV + i) / 4] >> (8 * ((k * KV + i) % 4))) & 0xFFu; };
+    // G rounds at a time, virtual thread by virtual thread (the block plays kv
+    // of them); all its draws of the G rounds are made, and masked a round at a
+    // time (a branch or a test around every draw costs more than the draws of
+    // the threads and rounds past the end).
+    constexpr int G = KV == 1 ? 2 : K;
 #pragma unroll
-    for (int j = 0; j < KP; ++j) {
-      // The counts of rounds 2 j and 2 j + 1, drawn for every virtual thread
-      // and masked a round at a time (a branch or a test around every draw
-      // costs more than the draws of the threads and rounds past the end).
-      uint32_t w[2] = {0, 0}, top = 0;
+    for (int k0 = 0; k0 < K; k0 += G) {
+      uint32_t w[G];   // a round's counts, one byte per virtual thread
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint64_t r = static_cast<uint64_t>(g.round0) + rb0 + 2 * j + h;
+      for (int h = 0; h < G; ++h) w[h] = 0;
+      const uint64_t r1 = static_cast<uint64_t>(g.round0) + rb0 + k0;
 #pragma unroll
-        for (int i = 0; i < KV; ++i) {
+      for (int i = 0; i < KV; ++i) {
+        if ((i > 0 && static_cast<uint32_t>(i) >= kv) || (C > 1 && kk == 0)) break;   // block-uniform
+        uint32_t top = 0;
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
           uint32_t ci;
           if (DIST == GGA_DIST_POISSON && tabled) {
-            const uint32_t u = splitmix_mix_hi(dv[i].state(r));
+            const uint32_t u = splitmix_mix_hi(dv[i].state(r1 + h));
             top = max(top, u);
             ci = sh.thr.first_count(u);
           } else {
-            ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r));
+            ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r1 + h));
           }
           w[h] |= ci << (8 * i);
         }
-      }
-      if (DIST == GGA_DIST_POISSON && tabled && top >= sh.thr.second) {
-        // A draw among the thresholds the table does not tell apart: all of
-        // this thread's draws of the two rounds again, threshold by threshold.
-        uint64_t both = 0;
+        if (DIST == GGA_DIST_POISSON && tabled && top >= sh.thr.second) {
+          // A draw among the thresholds the table does not tell apart: the
+          // virtual thread's draws again, threshold by threshold.
+          uint64_t all = 0;
 #pragma unroll 1
-        for (uint32_t q = 0; q < 2 * KV; ++q) {
-          const uint32_t h = q / KV, i = q % KV;
-          const uint64_t r = static_cast<uint64_t>(g.round0) + rb0 + 2 * j + h;
-          const uint32_t u = splitmix_mix_hi(RoundDraws(g.seed, gfirst + i).state(r));
-          both |= static_cast<uint64_t>(sh.thr.slow_count(g.nthr, u)) << (32 * h + 8 * i);
-        }
-        w[0] = static_cast<uint32_t>(both);
-        w[1] = static_cast<uint32_t>(both >> 32);
-      }
-      uint32_t pk = 0;
+          for (uint32_t h = 0; h < G; ++h)
+            all |= static_cast<uint64_t>(sh.thr.slow_count(g.nthr, splitmix_mix_hi(dv[i].state(r1 + h)))) << (8 * h);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t k = 2 * j + h;
-        w[h] &= k < kk ? played : 0u;
-        cw[k * KV / 4] |= w[h] << (8 * (k * KV % 4));
-        pk |= (KV == 1 ? w[h] : __dp4a(w[h], 0x01010101u, 0u)) << (16 * h);
+          for (int h = 0; h < G; ++h)
+            w[h] = (w[h] & ~(0xFFu << (8 * i))) | (static_cast<uint32_t>(all >> (8 * h)) & 0xFFu) << (8 * i);
+        }
       }
-      const uint32_t inc = warp_incl_scan_u32(pk);
-      exw[j] = inc - pk;
-      if (lane == 31) sh.wt[j][warp] = inc;
+#pragma unroll
+      for (int j2 = 0; j2 < G / 2; ++j2) {
+        uint32_t pk = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t k = k0 + 2 * j2 + h, x = w[2 * j2 + h] & (k < kk ? played : 0u);
+          cw[k * KV / 4] |= x << (8 * (k * KV % 4));
+          pk |= (KV == 1 ? x : __dp4a(x, 0x01010101u, 0u)) << (16 * h);
+        }
+        const uint32_t inc = warp_incl_scan_u32(pk);
+        exw[k0 / 2 + j2] = inc - pk;
+        if (lane == 31) sh.wt[k0 / 2 + j2][warp] = inc;
+      }
     }
     __syncthreads();
     if (kMarks) clear_marks(stage4, dirty, t0, NT);   // the last pass's write-out is over
@@ -719,6 +739,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
       if (t0 == 0) {         // read by the others after the stage's barrier
         if (rank == 0 && !full) v.sizes[l] = next;
         sh.stop = full ? 1 : (next >= target ? 2 : 0);
+        sh.rounds = pass_rounds(target - next, g.mean * static_cast<float>(v.T), C * K);
       }
     } else {
       __syncthreads();   // synchronize(): the buckets exist before any write
@@ -876,7 +897,8 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
     // others after it; sh.stop was set before this pass's second barrier;
     // sh.tab only gains entries past those this pass reads.
     if (t0 == 0) sh.base = next;
-    r0 = R - r0 > static_cast<uint32_t>(C * K) ? r0 + C * K : R;
+    if constexpr (C > 1) r0 = rend;
+    else r0 = R - r0 > static_cast<uint32_t>(K) ? r0 + K : R;
   }
   *done = sh.stop != 0;
   __syncthreads();   // the caller may reuse the stage and sh

@@ -125,3 +125,26 @@ def test_three_elements_a_draw_cost_no_more_than_as_many_draws(T, most):
     assert g.last_error() == gga.GGA_OK
     g.close()
 
+
+def test_blocks_of_256_threads_draw_for_themselves_alone():
+    """A batch of 600 LFVectors by 256 threads each against 1024: as many draws
+    (drawing for 1024 threads whatever T is took three times as long)."""
+    def grow(T):
+        pool = gga.GGAPool(1 << 30, 1024)
+        arrays = [gga.GGArray(1, T, 8192, 4, shared_pool=pool) for _ in range(600)]
+        batch = gga.GGABatch([(g, gga.make_gen_spec(a, "poisson", COEFFS, thresholds=poisson(1)), 100_000)
+                              for a, g in enumerate(arrays)])
+
+        def call():
+            batch.clear()
+            batch.grow()
+
+        t = microseconds(call)
+        batch.close()
+        for g in arrays:
+            assert g.size() == (100_000, gga.GGA_OK)
+            g.close()
+        pool.close()
+        return t
+
+    assert grow(256) < 2.3 * grow(1024)
