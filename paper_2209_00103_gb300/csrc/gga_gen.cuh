@@ -332,7 +332,9 @@ struct ThresholdTable {
 
   // #{k < nthr : u >= thr[k]} for the high word u of any draw.
   __device__ __forceinline__ uint32_t count(uint32_t nthr, uint32_t u) const {
-    return u >= second ? slow_count(nthr, u) : first_count(u);
+    uint32_t c = first_count(u);   // (loaded whatever u is: no branch before it)
+    if (u >= second) c = slow_count(nthr, u);
+    return c;
   }
 
   __device__ __forceinline__ uint32_t slow_count(uint32_t nthr, uint32_t u) const {

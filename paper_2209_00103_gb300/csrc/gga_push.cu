@@ -4,6 +4,9 @@
 // paper states it: one block per LFVector, one push per round, through the
 // device API's BlockPusher), and pushes of values read from device memory
 // (block_push_rounds, several rounds per call).
+#include <algorithm>
+#include <cmath>
+
 #include "gga_core.cuh"
 #include "gga_device.cuh"
 #include "gga_gen.cuh"
@@ -31,16 +34,30 @@ namespace gga {
 // geometric counts, clear and flatten included: 225 us with four, 139 with one).
 constexpr int kPushSlots = 4;
 constexpr uint32_t kPushSlotsMinT = 129;
-constexpr int kPushStageMax = 49152;
 
-// Stage of one push, in elements: T at one per thread and eight standard
-// deviations of a sum of T counts of variance up to 2 (a larger push stores
-// straight to the buckets), in whole 16-byte groups.
-uint32_t push_half_elems(uint32_t T, uint32_t E) {
-  uint32_t root = 1;
-  while (root * root < 2 * T) ++root;
-  const uint32_t vec = 16 / E;
-  return (T + 8 * root + 2 * vec - 1) / vec * vec;
+// Shared memory for the stage's two halves.  Wanted: a push at the counts' mean
+// and eight standard deviations of its sum (a larger push stores straight to
+// the buckets), for mean 1 and variance 2 at least.  Where that would keep
+// blocks off the SM, as many blocks as hold 2.5 deviations stay resident and
+// share its memory: 2^24 Poisson draws of mean 6 into 16-byte elements at T =
+// 512: 569 us with two blocks per SM, 845 with one that has room for all.
+// (Stage for mean one, larger pushes by the threads' own stores, int32 at T =
+// 512, mean 3 and 6: 280 and 646 us; now 155 and 258.)
+constexpr uint32_t kSmBytes = 233472, kPushOwnBytes = 6144;   // an SM's shared memory; a block's beside the stage
+
+uint32_t push_stage_bytes(uint32_t T, uint32_t E, uint32_t nt, const GenParams& g) {
+  double mean = 1, var = 2;
+  if (g.dist == GGA_DIST_POISSON) {
+    double sq = 0;   // of c^2 = sum over k < c of 2 k + 1 (ascending thresholds; a bound of the kind for others)
+    for (uint32_t k = 0; k < g.nthr; ++k) sq += (2.0 * k + 1.0) * (1.0 - g.thr[k] / 4294967296.0);
+    mean = std::max(mean, static_cast<double>(g.mean));
+    var = std::max(var, sq - static_cast<double>(g.mean) * g.mean);
+  }
+  const double sd = std::sqrt(T * var), vec = 16.0 / E;
+  const double want = 2 * E * (T * mean + 8 * sd + 2 * vec), least = 2 * E * (T * mean + 2.5 * sd + 2 * vec);
+  const uint32_t blocks = std::min(1024 / nt, static_cast<uint32_t>(kSmBytes / (least + kPushOwnBytes)));   // by registers
+  if (blocks == 0) return 0;
+  return static_cast<uint32_t>(std::min(want, static_cast<double>(kSmBytes / blocks - kPushOwnBytes))) / 32 * 32;
 }
 
 template <int E, int DIST, int S>
@@ -104,13 +121,13 @@ void launch_push_generated_as(const ArrayView& v, const ArrayView* dview, const 
                               cudaStream_t st) {
   const uint32_t slots = v.T >= kPushSlotsMinT ? kPushSlots : 1;
   const uint32_t nt = ((v.T + slots - 1) / slots + 31) / 32 * 32;
-  const uint32_t smem = 2 * push_half_elems(v.T, E) * E;   // two halves: at most 44 KB (T = 1024, 16-byte elements)
+  const uint32_t smem = push_stage_bytes(v.T, E, nt, g);
 #define GGA_PUSH(D)                                                                                         \
   do {                                                                                                      \
     auto kern = slots == 1 ? push_generated_kernel<E, D, 1> : push_generated_kernel<E, D, kPushSlots>;      \
     if (smem > 32768u)   /* with the count table the block's shared memory may pass 48 KB; the limit is the \
                             kernel's: other threads launch it for arrays of other shapes */                 \
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPushStageMax);               \
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmBytes - kPushOwnBytes);    \
     kern<<<v.L, nt, smem, st>>>(dview, g, rounds, v.T, smem);                                               \
   } while (0)
   switch (g.dist) {
