@@ -575,7 +575,7 @@ int gga_twophase_spawn(gga_handle h, uint32_t gen, uint64_t seed, int only_newbo
                        void* stream) {
   if (!h || h->p.elem_bytes != 16 || (only_newborn && !born_dev)) return GGA_ERR_INVALID;
   if (born_dev && (reinterpret_cast<uintptr_t>(born_dev) & 7) != 0) return GGA_ERR_INVALID;
-  return gga::launch_twophase_spawn(h->view, gen, seed, only_newborn ? 1 : 0, born_dev, S(stream));
+  return gga::launch_twophase_spawn(h->view, gen, seed, only_newborn ? 1 : 0, born_dev, h->ins.counters + 2, S(stream));
 }
 
 int gga_twophase_work(void* records_dev, uint64_t n, uint32_t passes, void* stream) {

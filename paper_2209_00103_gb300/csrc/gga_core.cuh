@@ -199,7 +199,7 @@ struct InsertScratch {
   uint64_t* ins_base;             // [L] LFVector size before the batch
   uint64_t* ins_len;              // [L] committed elements of the batch
   uint64_t* cp_prefix;            // [L+1] prefix of copy chunks
-  uint32_t* counters;             // last-block-done counters, zero between calls: [0] of count, [1] of reserve
+  uint32_t* counters;             // last-block-done counters, zero between calls: [0] of count, [1] of reserve, [2] of spawn
 };
 
 int launch_insert(const ArrayView& v, const InsertScratch& s, const uint32_t* counts, uint32_t rounds,
@@ -227,7 +227,7 @@ int launch_caps(const ArrayView& v, uint64_t* caps, cudaStream_t st);
 int launch_memory(const ArrayView& v, uint64_t* out2, cudaStream_t st);
 
 int launch_twophase_spawn(const ArrayView& v, uint32_t gen, uint64_t seed, int only_newborn, uint64_t* born,
-                          cudaStream_t st);
+                          uint32_t* done, cudaStream_t st);
 int launch_twophase_work(void* records, uint64_t n, uint32_t passes, int num_sms, cudaStream_t st);
 
 // Handle internals for entry points defined outside gga_capi.cu (null

@@ -13,6 +13,7 @@
 // children consecutively, and child k of a parent is the parent with
 // id = ((gen + 1) << 56) | (l << 40) | (the child's LFVector-local index).
 #include "gga_core.cuh"
+#include "gga_gen.cuh"
 
 namespace gga {
 
@@ -50,7 +51,7 @@ __device__ __forceinline__ uint32_t warp_scan_packed(uint32_t v) {
 constexpr int kSpawnP = 8;             // parents per thread per pass (coarsening)
 constexpr uint32_t kSpawnGroup = 1024; // parents whose children are kept or dropped together
 
-// One block per LFVector.  A warp takes 32 * kSpawnP consecutive parents of a
+// An LFVector of the growth, by one block.  A warp takes 32 * kSpawnP consecutive parents of a
 // pass, 32 at a time, so its children are one run of the LFVector, round
 // after round, and the block needs one total per warp: one block barrier per
 // pass, after which every thread knows where its warp's run starts and
@@ -70,9 +71,9 @@ constexpr uint32_t kSpawnGroup = 1024; // parents whose children are kept or dro
 // generations from 2^20 records (2^27 parents, as many children, 1024
 // LFVectors; 4.3 GB): 1.04 ms before, 0.80 now (0.63 at the copy rate); with the
 // children's loop unrolled over the rounds 1.07 (instruction-cache misses).
-template <int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) spawn_kernel(const __grid_constant__ ArrayView v, uint32_t gen,
-                                                         uint64_t seed, int only_newborn, uint64_t* born) {
+template <int NT>
+__device__ __forceinline__ void spawn_lfv(const ArrayView& v, uint32_t l, uint32_t gen, uint64_t seed, int only_newborn,
+                                          uint64_t* born) {
   constexpr int P = kSpawnP, KP = P / 2, NW = NT / 32;
   constexpr uint32_t kPass = NT * P;
   static_assert(kPass % kSpawnGroup == 0, "whole groups of parents per pass");
@@ -82,8 +83,7 @@ __global__ void __launch_bounds__(NT, MINB) spawn_kernel(const __grid_constant__
   __shared__ uint64_t s_tab[kMaxBuckets];    // the LFVector's bucket table (copy)
   __shared__ uint32_t s_nb;
 
-  const uint32_t l = blockIdx.x, t = threadIdx.x;
-  const uint32_t lane = t & 31, w = t >> 5;
+  const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5;
   const uint32_t upto = 0xffffffffu >> (31 - lane);          // lanes 0 .. lane
   uint2* const my_pv = s_pv + w * (32 * P);
   uint32_t* const my_ce = reinterpret_cast<uint32_t*>(s_pv + NT * P) + w * (32 * P);
@@ -250,6 +250,60 @@ __global__ void __launch_bounds__(NT, MINB) spawn_kernel(const __grid_constant__
   }
 }
 
+// An LFVector that a small block would be too long with: its rounds follow one another, and the others' blocks leave the SMs
+// idle meanwhile.  (Half of 2^20 records in one of 1024 LFVectors, 4
+// generations: 23.0 ms by its block of 128 threads, 7.9 by one of 1024.)
+// From the offsets, which stay those of the generation's start.
+constexpr uint64_t kSpawnLarge = 16384;
+__device__ __forceinline__ bool spawn_large(const ArrayView& v, uint64_t l) {
+  const uint64_t size = v.offsets[l + 1] - v.offsets[l];
+  return size > kSpawnLarge && size / 4 > v.offsets[v.L] / v.L;
+}
+
+// One block per LFVector; with small blocks, those that are not large.
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) spawn_kernel(const __grid_constant__ ArrayView v, uint32_t gen,
+                                                         uint64_t seed, int only_newborn, uint64_t* born) {
+  if (NT < 512 && spawn_large(v, blockIdx.x)) return;   // spawn_finish_kernel's
+  spawn_lfv<NT>(v, blockIdx.x, gen, seed, only_newborn, born);
+}
+
+// After spawn_kernel: the large ones -- every block looks through its share of
+// the LFVectors (at most a quarter are large, usually none) -- and, by the last
+// block to finish, what ends every insertion (finalize_kernel).  A kernel of
+// its own for the large ones was 5 us more per generation.
+__global__ void __launch_bounds__(1024, 1) spawn_finish_kernel(const __grid_constant__ ArrayView v, uint32_t gen,
+                                                               uint64_t seed, int only_newborn, uint64_t* born,
+                                                               uint32_t* done) {
+  __shared__ uint32_t s_large[1024];
+  __shared__ uint32_t s_n;
+  for (uint64_t l0 = blockIdx.x; l0 < v.L; l0 += static_cast<uint64_t>(gridDim.x) * 1024) {   // block-uniform
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const uint64_t l = l0 + static_cast<uint64_t>(gridDim.x) * threadIdx.x;
+    if (l < v.L && spawn_large(v, l)) s_large[atomicAdd(&s_n, 1u)] = static_cast<uint32_t>(l);
+    __syncthreads();
+    const uint32_t n = s_n;
+    for (uint32_t i = 0; i < n; ++i) {
+      spawn_lfv<1024>(v, s_large[i], gen, seed, only_newborn, born);
+      __syncthreads();
+    }
+    __syncthreads();   // s_n and s_large are read
+  }
+  __shared__ FinalizeShared s_fin;
+  __shared__ int s_last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  ring_fixup_class(v.pool, threadIdx.x);
+  finalize_block(v, nullptr, nullptr, nullptr, 1, s_fin);
+  if (threadIdx.x == 0) *done = 0;
+}
+
 // One streaming pass over flattened records: pos += vel.
 __global__ void __launch_bounds__(256) work_pass_kernel(uint4* __restrict__ rec, uint64_t n) {
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
@@ -271,33 +325,38 @@ __global__ void __launch_bounds__(256) work_pass_kernel(uint4* __restrict__ rec,
 
 }  // namespace
 
+template <int NT>
+constexpr int spawn_smem() { return NT * kSpawnP * static_cast<int>(sizeof(uint2) + sizeof(uint32_t)); }
+
 template <int NT, int MINB>
-static void launch_spawn(const ArrayView& v, uint32_t gen, uint64_t seed, int only_newborn, uint64_t* born,
-                         cudaStream_t st) {
-  const int smem = NT * kSpawnP * static_cast<int>(sizeof(uint2) + sizeof(uint32_t));
+static int launch_spawn(const ArrayView& v, uint32_t gen, uint64_t seed, int only_newborn, uint64_t* born,
+                        uint32_t* done, int sms, cudaStream_t st) {
   auto kern = spawn_kernel<NT, MINB>;
-  if (smem > 32768) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  kern<<<v.L, NT, smem, st>>>(v, gen, seed, only_newborn, born);
+  if (spawn_smem<NT>() > 32768) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, spawn_smem<NT>());
+  kern<<<v.L, NT, spawn_smem<NT>(), st>>>(v, gen, seed, only_newborn, born);
+  if (NT >= 512) return cudaGetLastError() == cudaSuccess ? launch_finalize(v, st) : GGA_ERR_CUDA;
+  cudaFuncSetAttribute(spawn_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, spawn_smem<1024>());
+  spawn_finish_kernel<<<sms, 1024, spawn_smem<1024>(), st>>>(v, gen, seed, only_newborn, born, done);
+  return cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
 }
 
 int launch_twophase_spawn(const ArrayView& v, uint32_t gen, uint64_t seed, int only_newborn, uint64_t* born,
-                          cudaStream_t st) {
+                          uint32_t* done, cudaStream_t st) {
   // The children's order and values depend on parent indices only, so the
   // block size is free, whatever T is: the smallest whose blocks still fill
   // the SMs (about 1024 threads each).  Small blocks wait less at their
   // barriers and leave no wave half empty: 1024 LFVectors are 1024 resident
   // blocks of 128 threads, but seven waves of one 1024-thread block per SM.
+  // They leave LFVectors far above the average to blocks of 1024.
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return GGA_ERR_CUDA;
   const uint32_t per_sm = v.L / static_cast<uint32_t>(sms);
-  if (per_sm >= 4) launch_spawn<128, 8>(v, gen, seed, only_newborn, born, st);
-  else if (per_sm >= 2) launch_spawn<256, 4>(v, gen, seed, only_newborn, born, st);
-  else if (per_sm >= 1) launch_spawn<512, 2>(v, gen, seed, only_newborn, born, st);
-  else launch_spawn<1024, 1>(v, gen, seed, only_newborn, born, st);
-  if (cudaGetLastError() != cudaSuccess) return GGA_ERR_CUDA;
-  return launch_finalize(v, st);
+  if (per_sm >= 4) return launch_spawn<128, 8>(v, gen, seed, only_newborn, born, done, sms, st);
+  if (per_sm >= 2) return launch_spawn<256, 4>(v, gen, seed, only_newborn, born, done, sms, st);
+  if (per_sm >= 1) return launch_spawn<512, 2>(v, gen, seed, only_newborn, born, done, sms, st);
+  return launch_spawn<1024, 1>(v, gen, seed, only_newborn, born, done, sms, st);
 }
 
 int launch_twophase_work(void* records, uint64_t n, uint32_t passes, int num_sms, cudaStream_t st) {
