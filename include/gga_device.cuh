@@ -190,15 +190,38 @@ __host__ __device__ __forceinline__ uint64_t prefix_capacity(uint32_t nb, uint32
 }
 
 // What the pushers' push_run hands to its writer (for one round): put(m, x)
-// stores the thread's element m.  kOneStore: it is a single shared-memory
-// store to put.at[m] (the usual case: the whole push is staged), so a writer
-// may unroll around it; otherwise it tests and looks buckets up.
+// stores the thread's element m, put.fill(count, f) its elements f(0), ...,
+// f(count - 1) (f is called for those that are kept, in order, and a bucket
+// looked up once).  kOneStore: an element is a single shared-memory store to
+// put.at[m] (the usual case: the whole push is staged), so a writer may unroll
+// around it; otherwise put tests and looks buckets up.
 template <class T>
 struct StagePut {
   static constexpr bool kOneStore = true;
   T* at;
   __device__ __forceinline__ void operator()(uint32_t m, T x) const { at[m] = x; }
+  template <class F>
+  __device__ __forceinline__ void fill(uint32_t count, F f) const {
+    for (uint32_t m = 0; m < count; ++m) at[m] = static_cast<T>(f(m));
+  }
 };
+
+// Elements f(0), ..., f(n - 1) to positions j, j + 1, ... of an LFVector.
+template <class T, class F>
+__device__ __forceinline__ void fill_buckets(const uint64_t* tab, uint32_t log2B, uint64_t j, uint32_t n, F f) {
+  T* p = nullptr;         // where element m would be: p[m]
+  uint64_t end = 0;       // first element past the bucket
+  for (uint32_t m = 0; m < n; ++m) {
+    if (m == end) {
+      uint32_t b;
+      uint64_t off;
+      bucket_of(j + m, log2B, b, off);
+      p = reinterpret_cast<T*>(tab[b]) + off - m;
+      end = m + bucket_len(b, log2B) - off;
+    }
+    p[m] = static_cast<T>(f(m));
+  }
+}
 
 template <class T>
 struct BucketPut {
@@ -217,6 +240,10 @@ struct BucketPut {
       bucket_of(j0 + m, log2B, b, off);
       reinterpret_cast<T*>(tab[b])[off] = x;
     }
+  }
+  template <class F>
+  __device__ __forceinline__ void fill(uint32_t count, F f) const {
+    fill_buckets<T>(tab, log2B, j0, count, f);
   }
 };
 
@@ -290,13 +317,14 @@ struct BlockPusher {
   // (in every thread) when the block's elements were appended.
   template <class F>
   __device__ bool push(uint32_t count, F value_of_k, uint64_t* first = nullptr) {
-    return push_run(count, [&](auto put) {
-      for (uint32_t k = 0; k < count; ++k) put(k, value_of_k(k));
-    }, first);
+    return push_run(count, [&](auto put) { put.fill(count, value_of_k); }, first);
   }
 
-  // push with the thread's elements in any order: write(put) is called once
-  // and calls put(k, element k) for every k < count.  A thread that stands
+  // push with the thread's elements in any order: write(put) is called at most
+  // once and calls put(k, element k) for every k < count.  It is not called
+  // in a push that fails or appends nothing, and in a push without a stage or
+  // larger than it not in threads with count 0: what every thread has to do in
+  // every push does not belong there.  A thread that stands
   // for several consecutive threads of the LFVector (its elements are the
   // first one's, then the next one's) then writes each one's elements at
   // their known places, without a search per element.  CMAX > 0 promises
@@ -548,6 +576,15 @@ struct CheckedPut {
       reinterpret_cast<T*>(tab[b])[off] = x;
     }
   }
+  template <class F>
+  __device__ __forceinline__ void fill(uint32_t count, F f) const {
+    const uint32_t keep = q < n ? (n - q < count ? n - q : count) : 0u;
+    if (stage) {
+      for (uint32_t m = 0; m < keep; ++m) stage[q + m] = static_cast<T>(f(m));
+    } else {
+      fill_buckets<T>(tab, log2B, base + q, keep, f);
+    }
+  }
 };
 
 // Shared memory of one RoundsPusher<T, K> (declare it __shared__, one per
@@ -630,12 +667,12 @@ struct RoundsPusher {
   __device__ uint32_t push(const uint32_t (&count)[K], F value_of, uint32_t* kept = nullptr,
                            uint64_t* first = nullptr) {
     return push_run(count, [&](uint32_t kr, auto put) {
-      if (CMAX > 0) {
+      if constexpr (CMAX > 0 && decltype(put)::kOneStore) {
 #pragma unroll
         for (uint32_t m = 0; m + 1 <= CMAX; ++m)
-          if (m < count[kr]) put(m, value_of(kr, m));
+          if (m < count[kr]) put(m, static_cast<T>(value_of(kr, m)));
       } else {
-        for (uint32_t m = 0; m < count[kr]; ++m) put(m, value_of(kr, m));
+        put.fill(count[kr], [&](uint32_t m) { return value_of(kr, m); });
       }
     }, kept, first);
   }
