@@ -268,7 +268,10 @@ int gga_insert_generated(gga_handle h, const gga_gen_spec* spec, uint32_t rounds
  *  positions of Sec. III-B).  GGA_ERR_INVALID on the host for a null
  *  pointer, misalignment or T > 512; GGA_ERR_POOL_EXHAUSTED latched when a
  *  call's buckets do not fit (the LFVector keeps the longest prefix of
- *  whole rounds of that call that fits and stops).
+ *  whole rounds of that call that fits and stops).  Four neighbouring slots'
+ *  counts (two for 16-byte elements) that sum to 2^32 or more in a round are
+ *  taken as zero and GGA_ERR_INVALID is latched; a push's elements must stay
+ *  below 2^32 per LFVector.
  */
 int gga_device_view(gga_handle h, const void** view_dev);
 int gga_device_commit(gga_handle h, void* stream);
