@@ -112,17 +112,29 @@ int blocks_per_sm(uint32_t form, bool clusters) {
 
 int batch_grow(gga_batch_t* b, cudaStream_t st) {
   bool ok = true;
+  uint32_t started = 0;
   if (b->n_launches > 1) ok = cudaEventRecord(b->fork, st) == cudaSuccess;
   for (uint32_t i = 0; i < b->n_launches && ok; ++i) {
     cudaStream_t s = i == 0 ? st : b->side[i];
     if (i) ok = cudaStreamWaitEvent(s, b->fork, 0) == cudaSuccess;
+    if (!ok) break;   // the launch would not wait for what comes before
     launch_form(b->launch[i], s);
-    if (i) ok = cudaEventRecord(b->join[i], s) == cudaSuccess && ok;
+    started = i + 1;
+    if (i) ok = cudaEventRecord(b->join[i], s) == cudaSuccess;
   }
-  for (uint32_t i = 1; i < b->n_launches && ok; ++i) ok = cudaStreamWaitEvent(st, b->join[i], 0) == cudaSuccess;
+  for (uint32_t i = 1; i < started && ok; ++i) ok = cudaStreamWaitEvent(st, b->join[i], 0) == cudaSuccess;
+  if (!ok) {
+    // Growth kernels may be running that `st` does not wait for: what follows a
+    // growth is launched when they are done (a stream that is captured runs
+    // none, and its capture fails).
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return GGA_ERR_CUDA;
+    for (uint32_t i = 1; i < started; ++i)
+      if (cudaStreamSynchronize(b->side[i]) != cudaSuccess) return GGA_ERR_CUDA;
+  }
   if (b->n_jobs)
     gga::batch_finalize_kernel<<<b->n_jobs, 256, 0, st>>>(b->jobs, b->pools, b->n_pools, b->tickets);
-  return ok && cudaGetLastError() == cudaSuccess ? GGA_OK : GGA_ERR_CUDA;
+  return cudaGetLastError() == cudaSuccess && ok ? GGA_OK : GGA_ERR_CUDA;
 }
 
 int batch_clear(gga_batch_t* b, cudaStream_t st) {
