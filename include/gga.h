@@ -288,7 +288,8 @@ int gga_push_expand(gga_handle h, const uint32_t* counts_dev, const void* inputs
  * its output element is zeroed.  A batch of 2^25 reads or more of 4- or
  * 8-byte elements, from a slab of 512 MB or more and at most 48 bytes per
  * read, is grouped by ranges of global indices first (the values come back in
- * the order of idx_dev).  That takes 6.4 bytes (E = 8: 14.4) of
+ * the order of idx_dev), unless the array has less than 192 MB or a sample of
+ * the batch, taken on the device, meets in little of it.  The grouping takes 6.4 bytes (E = 8: 14.4) of
  * device memory per read during the call, stream-ordered, from a pool of the
  * library that keeps up to 1 GB between calls while any handle of the device
  * lives; without that memory, and while `stream` is captured, the batch is

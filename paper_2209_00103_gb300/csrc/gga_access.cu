@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) write_kernel(ArrayView v, const uint64_t*
 
 constexpr uint32_t kWbinMaxBins = 256;
 constexpr uint64_t kWbinMin = 1ull << 20;        // smaller batches write directly
-constexpr uint64_t kWbinHeader = 4096;           // totals[256] u32 | cursors[256] u64 | valid u64 | any u32
+constexpr uint64_t kWbinHeader = 4096;           // totals[256] u32 | cursors[256] u64 | valid u64 | of binned reads: rbin_word
 constexpr int kWbinThreads = 256;
 
 // The bins hold, per write, the element's offset inside its bin (32 bits:
@@ -152,8 +152,9 @@ __device__ __forceinline__ unsigned long long* wbin_cursors(uint8_t* scr) {
 __device__ __forceinline__ unsigned long long* wbin_valid(uint8_t* scr) {
   return reinterpret_cast<unsigned long long*>(scr + 3072);
 }
-// Binned reads: whether any tile was left to the scatter and the return.
-__device__ __forceinline__ uint32_t* rbin_any(uint8_t* scr) { return reinterpret_cast<uint32_t*>(scr + 3080); }
+// Binned reads: single words behind it.
+enum RbinWord { kRbinAny, kRbinDirect, kRbinDone, kRbinTicket };
+__device__ __forceinline__ uint32_t* rbin_word(uint8_t* scr, int w) { return reinterpret_cast<uint32_t*>(scr + 3080) + w; }
 
 template <int E>
 __global__ void __launch_bounds__(kWbinThreads) wbin_count_kernel(ArrayView v, const uint64_t* __restrict__ idx,
@@ -190,10 +191,9 @@ __global__ void __launch_bounds__(kWbinThreads) wbin_count_kernel(ArrayView v, c
 }
 
 // One block of kWbinMaxBins threads, one bin each.
-__global__ void __launch_bounds__(kWbinMaxBins) wbin_scan_kernel(uint8_t* scr) {
-  __shared__ uint64_t wsum[kWbinMaxBins / 32];
+__device__ __forceinline__ void wbin_scan(uint8_t* scr, uint64_t* wsum) {
   uint32_t* tot = wbin_totals(scr);
-  const uint64_t c = tot[threadIdx.x];
+  const uint64_t c = __ldcg(tot + threadIdx.x);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint64_t sc = c;
 #pragma unroll
@@ -208,6 +208,11 @@ __global__ void __launch_bounds__(kWbinMaxBins) wbin_scan_kernel(uint8_t* scr) {
   wbin_cursors(scr)[threadIdx.x] = sc - c + add;
   tot[threadIdx.x] = 0;   // ready for the next batch
   if (threadIdx.x == kWbinMaxBins - 1) *wbin_valid(scr) = sc + add;
+}
+
+__global__ void __launch_bounds__(kWbinMaxBins) wbin_scan_kernel(uint8_t* scr) {
+  __shared__ uint64_t wsum[kWbinMaxBins / 32];
+  wbin_scan(scr, wsum);
 }
 
 template <int E>
@@ -422,9 +427,11 @@ __global__ void __launch_bounds__(kWbinThreads) wbin_apply_kernel(ArrayView v, c
 // the writes, a large batch is therefore grouped by ranges of global indices
 // and read range by range, each range streamed into L2 ahead of its reads;
 // the values then go back to their places through the tiles they came from:
-//   count:   per-bin totals; a tile whose indices are local (a sorted batch,
-//            a window) is read here, directly, and takes no further part
-//   scan:    bin cursors (wbin_scan_kernel)
+//   decide:  by a sample, whether the batch reaches over more than the L2 holds;
+//            if not the count reads it and the others have nothing to do
+//   count:   per-bin totals, and by the last block the bin cursors; a tile whose
+//            indices are local (a sorted batch, a window) is read here, directly,
+//            and takes no further part
 //   scatter: a tile's indices, 32 bits each, sorted by bin in shared memory
 //            go to the bins, and the tile keeps where its runs lie and each
 //            sorted index's place in the tile
@@ -450,10 +457,30 @@ constexpr uint64_t kRbinMin = 1ull << 25;
 constexpr uint64_t kRbinMax = 1ull << 30;         // (run places are 32 bits)
 constexpr uint64_t kRbinSlabMin = 512ull << 20;
 constexpr uint64_t kRbinBytesPerRead = 48;
-constexpr uint64_t kRbinArrayMin = 192ull << 20;  // arrays the L2 (129 MB) mostly holds: direct, decided on the device
 
-constexpr uint64_t kRbinTilesPerBlock = 2;        // scatter and return (1: 2% faster, but a sorted batch, with no tile left
-                                                  // to do, pays 22 us for empty blocks instead of 12)
+// Which of them do better directly: those that mostly meet in L2 (129 MB),
+// because the array is small, its hot part is, or a few elements take most of
+// the reads.  The latter two show in the pieces of 64 KB that a sample of 4096
+// of the batch's indices touches, which is known on the device only.  Uniform
+// indices over 256 MB touch 2600.  Measured on GB300 for 2^26 int32 reads of 0.97
+// GB, pieces: direct / binned (us): uniform 3650: 1390 / 905; uniform over 400 MB
+// of it 3000: 1210 / 885; over 200 MB 2340: 1015 / 860; over 64 MB in parts of 64
+// KB 1000: 608 / 898; normal around one place with sd 5% 2270: 950 / 1095 (many
+// reads in few bins); Zipf with exponent 1.05 at scattered places 2490: 873 / 803,
+// 1.3 950: 355 / 820, next to each other 95: 227 / 2916.  Where the LFVectors'
+// sizes differ so much that the proportional guess mostly misses, the search
+// costs a direct read more than L2 saves it (256 hot pieces of an array with
+// every seventh LFVector empty: 1220 / 980): only batches that crowd into a bin or
+// two are read directly then.
+constexpr uint64_t kRbinArrayMin = 192ull << 20;   // smaller arrays: directly
+constexpr uint32_t kRbinSample = 4096;
+constexpr uint32_t kRbinPieces = 2300;             // batches that touch fewer: directly
+constexpr uint32_t kRbinPiecesSearched = 128;      // ... where the guess misses for most
+constexpr int kRbinPieceLog2 = 16;
+constexpr uint32_t kRbinPieceBits = 1u << 16;      // (arrays above 4 GB share them)
+
+constexpr uint64_t kRbinTilesPerBlock = 2;        // scatter and return (1: 2% faster, but a batch with no tile left
+                                                  // to do pays 22 us for empty blocks instead of 12)
 constexpr int kRbinApplyThreads = 512;
 constexpr int kRbinApplyPer = 8;                   // reads per thread of the apply
 constexpr int kRbinPer = 16;                      // indices per thread of a tile
@@ -504,6 +531,74 @@ __device__ __forceinline__ uint32_t rbin_shift(uint64_t N, uint32_t E) {
   return s;
 }
 
+// One block: the header cleared, and whether the whole batch is read directly
+// (also arrays of 2^32 elements and more: the bins hold 32-bit indices).
+template <int E>
+__global__ void __launch_bounds__(1024) rbin_decide_kernel(ArrayView v, const uint64_t* __restrict__ idx, uint64_t n,
+                                                           uint8_t* head) {
+  __shared__ uint32_t seen[kRbinPieceBits / 32];
+  __shared__ uint32_t pieces, missed;
+  constexpr int kPer = kRbinSample / 1024;
+  const uint64_t N = __ldg(v.offsets + v.L);
+  const uint64_t step = n / kRbinSample;   // >= 1: n >= kRbinMin
+  uint64_t g[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    // One index of every kRbinSample-th part of the batch, at no fixed place of it.
+    const uint64_t i = static_cast<uint64_t>(u) * 1024 + threadIdx.x;
+    g[u] = __ldg(idx + i * step + ((i * 0x9E3779B97F4A7C15ull) >> 32) % step);
+  }
+  for (uint32_t w = threadIdx.x; w < kRbinPieceBits / 32; w += 1024) seen[w] = 0;
+  reinterpret_cast<uint32_t*>(head)[threadIdx.x] = 0;
+  static_assert(kWbinHeader == 4 * 1024, "a word of the header per thread");
+  if (threadIdx.x == 0) pieces = missed = 0;
+  __syncthreads();
+  uint32_t fresh = 0, miss = 0;
+  const float scale = static_cast<float>(v.L) / __ull2float_rz(N);
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    if (g[u] >= N) continue;
+    const uint32_t l = min(__float2uint_rz(__ull2float_rz(g[u]) * scale), v.L - 1);
+    if (g[u] < __ldg(v.offsets + l) || g[u] >= __ldg(v.offsets + l + 1)) ++miss;
+    const uint32_t p = static_cast<uint32_t>((g[u] * E) >> kRbinPieceLog2) % kRbinPieceBits;
+    const uint32_t bit = 1u << (p % 32);
+    if (!(atomicOr(&seen[p / 32], bit) & bit)) ++fresh;
+  }
+  fresh = __reduce_add_sync(0xffffffffu, fresh);
+  miss = __reduce_add_sync(0xffffffffu, miss);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&pieces, fresh);
+    atomicAdd(&missed, miss);
+  }
+  __syncthreads();
+  if (threadIdx.x) return;
+  const uint32_t least = missed * 2 > kRbinSample ? kRbinPiecesSearched : kRbinPieces;
+  if (N * E < kRbinArrayMin || N > 0xFFFFFFFFull || pieces < least) *rbin_word(head, kRbinDirect) = 1;
+}
+
+// A block's tiles of the count, in order: a tile's ticket is taken while the one
+// before is worked on.  Blocks that take every gridDim.x-th tile drift apart
+// where the reads go to memory (normal indices around one place, 2^26 int32 read
+// directly: 1031 us, by tickets 882).
+struct RbinTiles {
+  uint32_t* ticket;
+  uint32_t* at;         // shared
+  uint32_t next;
+  __device__ __forceinline__ RbinTiles(uint32_t* t, uint32_t* shared) : ticket(t), at(shared), next(0) {
+    if (threadIdx.x == 0) *at = atomicAdd(ticket, 1u);
+    __syncthreads();
+  }
+  __device__ __forceinline__ uint32_t tile() {
+    if (threadIdx.x == 0) next = atomicAdd(ticket, 1u);
+    return *at;
+  }
+  __device__ __forceinline__ void advance() {
+    __syncthreads();   // the tile is done, and its number read
+    if (threadIdx.x == 0) *at = next;
+    __syncthreads();
+  }
+};
+
 template <int E>
 __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, const uint64_t* __restrict__ idx,
                                                                   uint64_t n, RbinScratch s,
@@ -513,14 +608,14 @@ __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, c
   __shared__ uint32_t h[kWbinMaxBins];
   const uint64_t N = __ldg(v.offsets + v.L);
   const uint32_t shift = rbin_shift(N, E);
-  // Arrays that the L2 mostly holds are read directly, and those of 2^32
-  // elements and more (the bins hold 32-bit indices).
-  const bool never = N * E < kRbinArrayMin || N > 0xFFFFFFFFull;
+  const bool never = *rbin_word(s.head, kRbinDirect) != 0;
   for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x) h[b] = 0;
   bool bad = false, left = false;   // left: some tile was not read here
-  const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
-  for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const uint64_t base = tile * kRbinTile;
+  __shared__ uint32_t s_tile;
+  const uint32_t tiles = static_cast<uint32_t>((n + kRbinTile - 1) / kRbinTile);
+  RbinTiles todo(rbin_word(s.head, kRbinTicket), &s_tile);
+  for (uint32_t tile; (tile = todo.tile()) < tiles; todo.advance()) {
+    const uint64_t base = static_cast<uint64_t>(tile) * kRbinTile;
     uint64_t g[kPer];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
@@ -533,7 +628,7 @@ __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, c
     const uint64_t d = g[kPer / 2] - __shfl_up_sync(0xffffffffu, g[kPer / 2], 1) + 128 / E;
     const uint64_t db = (g[kPer / 2] >> shift) - (__ldg(idx + base) >> shift) + 1;
     const bool near = ((threadIdx.x & 31) != 0 && d <= 2 * (128 / E)) || db <= 2;
-    const bool direct = __syncthreads_count(near) * 2 > kWbinThreads || never;
+    const bool direct = never || __syncthreads_count(near) * 2 > kWbinThreads;
     if (threadIdx.x == 0) s.direct[tile] = direct ? 1 : 0;
     if (direct) {
       T x[kPer];
@@ -559,11 +654,22 @@ __global__ void __launch_bounds__(kWbinThreads) rbin_count_kernel(ArrayView v, c
     }
   }
   if (bad) latch_error(v.status, GGA_ERR_OUT_OF_RANGE);
-  if (left && threadIdx.x == 0) *rbin_any(s.head) = 1;
+  if (never) return;
+  if (left && threadIdx.x == 0) *rbin_word(s.head, kRbinAny) = 1;
   __syncthreads();
   uint32_t* tot = wbin_totals(s.head);
   for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x)
     if (h[b]) atomicAdd(tot + b, h[b]);
+  // The last block to finish turns the totals into cursors.
+  __shared__ uint64_t wsum[kWbinMaxBins / 32];
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(rbin_word(s.head, kRbinDone), 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  wbin_scan(s.head, wsum);
 }
 
 template <int E>
@@ -579,8 +685,8 @@ __global__ void __launch_bounds__(kWbinThreads, 4) rbin_scatter_kernel(ArrayView
   __shared__ alignas(16) uint16_t s_place[kTile];
   const uint64_t N = __ldg(v.offsets + v.L);
   const uint32_t shift = rbin_shift(N, E);
-  // None when every tile was read directly.
-  const uint64_t tiles = *rbin_any(s.head) ? (n + kTile - 1) / kTile : 0;
+  if (!*rbin_word(s.head, kRbinAny)) return;   // every tile was read directly
+  const uint64_t tiles = (n + kTile - 1) / kTile;
   for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     if (s.direct[tile]) continue;   // block-uniform
     for (uint32_t b = threadIdx.x; b < kWbinMaxBins; b += blockDim.x) h[b] = 0;
@@ -737,9 +843,10 @@ __global__ void __launch_bounds__(kWbinThreads, 6) rbin_return_kernel(RbinScratc
   uint8_t* s_bin = s_dyn + static_cast<size_t>(kTile) * E;                 // [kTile]
   __shared__ uint32_t at[kWbinMaxBins];
   __shared__ uint16_t off[kWbinMaxBins];
-  // None when every tile was read directly.  (The valid indices do not tell:
-  // a tile of indices out of range has none, and its outputs are zeroed here.)
-  const uint64_t tiles = *rbin_any(s.head) ? (n + kTile - 1) / kTile : 0;
+  // (The valid indices do not tell: a tile of indices out of range has none,
+  // and its outputs are zeroed here.)
+  if (!*rbin_word(s.head, kRbinAny)) return;   // every tile was read directly
+  const uint64_t tiles = (n + kTile - 1) / kTile;
   for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     if (s.direct[tile]) continue;   // block-uniform
     const uint64_t base = tile * kTile;
@@ -1176,6 +1283,7 @@ static void write_as(const ArrayView& v, const uint64_t* idx, uint64_t n, const 
   wbin_scatter_kernel<E><<<grid, kWbinThreads, smem, st>>>(v, idx, static_cast<const T*>(in), n, scr, out_off,
                                                            out_val);
   constexpr int kTileA = kWbinThreads * WbinApplyPer<E>::kPer;
+  const uint64_t halves = (tiles + kRbinTilesPerBlock - 1) / kRbinTilesPerBlock;
   const uint64_t tiles_a = (n + kTileA - 1) / kTileA;
   const unsigned grid_a = static_cast<unsigned>(tiles_a > 0x7FFFFFFFull ? 0x7FFFFFFFull : tiles_a);
   wbin_apply_kernel<E><<<grid_a, kWbinThreads, 0, st>>>(v, out_off, out_val, scr);
@@ -1187,17 +1295,17 @@ static void read_binned_as(const ArrayView& v, const uint64_t* idx, uint64_t n, 
   typedef typename Elem<E>::T T;
   RbinScratch s;
   rbin_layout<E>(n, static_cast<uint8_t*>(scratch), &s);
-  cudaMemsetAsync(s.head, 0, kWbinHeader, st);   // the totals, and no tile left
   const uint64_t tiles = (n + kRbinTile - 1) / kRbinTile;
-  const uint64_t cap = static_cast<uint64_t>(num_sms) * 4;   // the count: persistent blocks, one set of global additions each
-  rbin_count_kernel<E><<<static_cast<unsigned>(tiles < cap ? tiles : cap), kWbinThreads, 0, st>>>(v, idx, n, s, static_cast<T*>(out));
-  wbin_scan_kernel<<<1, kWbinMaxBins, 0, st>>>(s.head);
-  rbin_scatter_kernel<E><<<static_cast<unsigned>((tiles + kRbinTilesPerBlock - 1) / kRbinTilesPerBlock), kWbinThreads, 0, st>>>(v, idx, n, s);
-  constexpr uint64_t kTileA = static_cast<uint64_t>(kRbinApplyThreads) * kRbinApplyPer;
-  rbin_apply_kernel<E><<<static_cast<unsigned>((n + kTileA - 1) / kTileA), kRbinApplyThreads, 0, st>>>(v, s);
-  const int smem = static_cast<int>(kRbinTile * (E + 1));
+  const uint64_t halves = (tiles + kRbinTilesPerBlock - 1) / kRbinTilesPerBlock;
+  const uint64_t tiles_a = (n + kRbinApplyThreads * kRbinApplyPer - 1) / (kRbinApplyThreads * kRbinApplyPer);
+  constexpr int smem = static_cast<int>(kRbinTile * (E + 1));
   cudaFuncSetAttribute(rbin_return_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  rbin_return_kernel<E><<<static_cast<unsigned>((tiles + kRbinTilesPerBlock - 1) / kRbinTilesPerBlock), kWbinThreads, smem, st>>>(s, n, static_cast<T*>(out));
+  const uint64_t cap = static_cast<uint64_t>(num_sms) * 4;   // the count: persistent blocks, one set of global additions each
+  rbin_decide_kernel<E><<<1, 1024, 0, st>>>(v, idx, n, s.head);
+  rbin_count_kernel<E><<<static_cast<unsigned>(tiles < cap ? tiles : cap), kWbinThreads, 0, st>>>(v, idx, n, s, static_cast<T*>(out));
+  rbin_scatter_kernel<E><<<static_cast<unsigned>(halves), kWbinThreads, 0, st>>>(v, idx, n, s);
+  rbin_apply_kernel<E><<<static_cast<unsigned>(tiles_a), kRbinApplyThreads, 0, st>>>(v, s);
+  rbin_return_kernel<E><<<static_cast<unsigned>(halves), kWbinThreads, smem, st>>>(s, n, static_cast<T*>(out));
 }
 
 uint64_t rbin_scratch_bytes(uint64_t n, uint32_t E, uint64_t slab_bytes) {
