@@ -63,7 +63,7 @@ __device__ __forceinline__ void grow_item(const BatchJob* __restrict__ jobs, con
   const ArrayView& v = s_job.v;
   const uint64_t target = s_job.target / v.L + (item.l < s_job.target % v.L ? 1 : 0);
   bool done;
-  const uint32_t drawn = grow_passes<E, kBatchRounds, kBatchKV, true, DIST, C, batch_staged(E, DIST)>(
+  const uint32_t drawn = grow_passes<E, kBatchRounds, kBatchKV, DIST, C, batch_staged(E, DIST), true>(
       v, s_job.g, item.l, kBatchMaxRounds, target, sh, stage, kBatchStageBytes / E, &done);
   if (threadIdx.x == 0 && !done && drawn >= kBatchMaxRounds) latch_error(v.status, GGA_ERR_TIMEOUT);
   __syncthreads();

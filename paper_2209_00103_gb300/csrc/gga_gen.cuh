@@ -64,10 +64,11 @@ struct RoundDraws {
 // Count of one draw from the mixed state z.  DIST >= 0 fixes the
 // distribution at compile time (GGA_DIST_*), -1 reads g.dist.  Every
 // distribution but the geometric one uses only the high word of the draw.
-// SEARCH: g lives in shared memory, where a binary search over the
-// thresholds costs a few indexed loads; for kernel parameters (constant
-// bank) the unrolled count reads each threshold as an operand instead, and
-// an indexed read would copy the parameters to local memory.
+// SEARCH: g lives in shared memory, where a binary search over ascending
+// thresholds costs a few indexed loads; for kernel parameters (constant bank)
+// the unrolled count reads each threshold as an operand instead, and an indexed
+// read would copy the parameters to local memory.  (The pass loops take ascending
+// thresholds through a ThresholdTable, and come here with others.)
 template <bool SEARCH = false, int DIST = -1>
 __device__ __forceinline__ uint32_t gen_count_state(const GenParams& g, uint64_t z) {
   const uint32_t dist = DIST >= 0 ? static_cast<uint32_t>(DIST) : g.dist;
@@ -78,9 +79,8 @@ __device__ __forceinline__ uint32_t gen_count_state(const GenParams& g, uint64_t
   const uint32_t u = splitmix_mix_hi(z);
   if (dist == GGA_DIST_BERNOULLI) return u >> 31;
   if (dist == GGA_DIST_UNIFORM3) return __umulhi(u, 3u);
-  // c = #{k < nthr : u >= thr[k]}.  Ascending thresholds (the CDF of the
-  // distribution, the usual case) make that set a prefix, whose length a
-  // binary search finds in five steps; other tables are counted.
+  // c = #{k < nthr : u >= thr[k]}.  Ascending thresholds make that set a prefix,
+  // whose length a binary search finds in five steps; other tables are counted.
   uint32_t c = 0;
   if (SEARCH && g.thr_sorted) {
 #pragma unroll
@@ -91,34 +91,6 @@ __device__ __forceinline__ uint32_t gen_count_state(const GenParams& g, uint64_t
     for (uint32_t k = 0; k < GGA_MAX_THRESHOLDS; ++k) c += (k < g.nthr) & (u >= g.thr[k]);
   }
   return c;
-}
-
-// Count of draw h = splitmix(seed, key) (the whole 64-bit output).
-template <bool SEARCH = false>
-__device__ __forceinline__ uint32_t gen_count(const GenParams& g, uint64_t h) {
-  switch (g.dist) {
-    case GGA_DIST_BERNOULLI:
-      return static_cast<uint32_t>(h >> 63);
-    case GGA_DIST_UNIFORM3:
-      return static_cast<uint32_t>(((h >> 32) * 3ull) >> 32);
-    case GGA_DIST_GEOMETRIC: {
-      const uint64_t inv = ~h;
-      return inv == 0 ? 63u : min(63u, static_cast<uint32_t>(__ffsll(static_cast<long long>(inv)) - 1));
-    }
-    default: {
-      const uint32_t u = static_cast<uint32_t>(h >> 32);
-      uint32_t c = 0;
-      if (SEARCH && g.thr_sorted) {
-#pragma unroll
-        for (uint32_t step = 16; step > 0; step >>= 1)
-          if (c + step <= g.nthr && u >= g.thr[c + step - 1]) c += step;
-      } else {
-#pragma unroll
-        for (uint32_t k = 0; k < GGA_MAX_THRESHOLDS; ++k) c += (k < g.nthr) & (u >= g.thr[k]);
-      }
-      return c;
-    }
-  }
 }
 
 template <int E>
@@ -521,8 +493,7 @@ __device__ __forceinline__ void clear_marks(uint4* marks4, uint32_t n, uint32_t 
 
 // Returns the number of rounds it drew; *done is set when the LFVector
 // reached `target` or the pool ran out.  Every thread of the block calls
-// it.  SEARCH as for gen_count (g in shared memory); DIST as for
-// gen_count_state (-1: g.dist at run time).
+// it.  DIST as for gen_count_state (-1: g.dist at run time).
 //
 // C > 1: the C blocks of a cluster grow the LFVector together, block q of a
 // pass drawing its rounds q K .. q K + K - 1 of the pass's C K (the last pass
@@ -533,7 +504,7 @@ __device__ __forceinline__ void clear_marks(uint4* marks4, uint32_t n, uint32_t 
 // buckets; only when it does not, block 0 allocates behind a second cluster
 // barrier.  Draws, positions, clipping and the rounds kept when the pool
 // runs out are those of one block drawing the same rounds one after another.
-template <int E, int K, int KV, bool SEARCH = false, int DIST = -1, int C = 1, int SP = K>
+template <int E, int K, int KV, int DIST = -1, int C = 1, int SP = K, bool SKIP = false>
 __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t l, uint32_t R, uint64_t target,
                                 GenShared& sh, uint4* stage4, uint32_t cap, bool* done) {
   typedef typename Elem<E>::T T;
@@ -591,11 +562,16 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
 #pragma unroll
     for (int q = 0; q < KC; ++q) cw[q] = 0;
     auto count_of = [&](uint32_t k, uint32_t i) { return (cw[(k * KV + i) / 4] >> (8 * ((k * KV + i) % 4))) & 0xFFu; };
-    // G rounds at a time, virtual thread by virtual thread (the block plays kv
-    // of them); all its draws of the G rounds are made, and masked a round at a
-    // time (a branch or a test around every draw costs more than the draws of
-    // the threads and rounds past the end).
-    constexpr int G = KV == 1 ? 2 : K;
+    // G rounds at a time, virtual thread by virtual thread: all its draws of the
+    // G rounds are made, and masked a round at a time (a branch or a test around
+    // every draw costs more than the draws of the threads and rounds past the
+    // end).  kSkip: virtual threads that no thread of the block plays are left
+    // out, for a test per virtual thread and all rounds together (SKIP: batches,
+    // whose blocks are not sized by T and whose g lives in shared memory).  Elsewhere bounded counts take two
+    // rounds at a time (paper-shaped workload, flatten included: 837 us, with the
+    // test 845, with the test and two rounds 855).
+    constexpr bool kSkip = SKIP || kMarks;
+    constexpr int G = KV == 1 || !kSkip ? 2 : K;
 #pragma unroll
     for (int k0 = 0; k0 < K; k0 += G) {
       uint32_t w[G];   // a round's counts, one byte per virtual thread
@@ -604,7 +580,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
       const uint64_t r1 = static_cast<uint64_t>(g.round0) + rb0 + k0;
 #pragma unroll
       for (int i = 0; i < KV; ++i) {
-        if ((i > 0 && static_cast<uint32_t>(i) >= kv) || (C > 1 && kk == 0)) break;   // block-uniform
+        if (kSkip && ((i > 0 && static_cast<uint32_t>(i) >= kv) || (C > 1 && kk == 0))) break;   // block-uniform
         uint32_t top = 0;
 #pragma unroll
         for (int h = 0; h < G; ++h) {
@@ -614,7 +590,7 @@ __device__ uint32_t grow_passes(const ArrayView& v, const GenParams& g, uint32_t
             top = max(top, u);
             ci = sh.thr.first_count(u);
           } else {
-            ci = gen_count_state<SEARCH, DIST>(g, dv[i].state(r1 + h));
+            ci = gen_count_state<SKIP, DIST>(g, dv[i].state(r1 + h));
           }
           w[h] |= ci << (8 * i);
         }

@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(MAXT, MINB) gen_insert_kernel(const __grid_con
   extern __shared__ uint4 s_stage4[];
   __shared__ GenShared sh;
   bool done;
-  grow_passes<E, K, KV, false, DIST>(v, g, blockIdx.x, R, ~0ull, sh, s_stage4, stage_bytes / E, &done);
+  grow_passes<E, K, KV, DIST>(v, g, blockIdx.x, R, ~0ull, sh, s_stage4, stage_bytes / E, &done);
 }
 
 template <int E, int DIST>

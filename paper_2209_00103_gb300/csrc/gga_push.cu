@@ -3,7 +3,7 @@
 // insertion written as a user kernel would write it (Algorithm 1 as the
 // paper states it: one block per LFVector, one push per round, through the
 // device API's BlockPusher), and pushes of values read from device memory
-// (block_push_rounds, several rounds per call).
+// (RoundsPusher, several rounds per push).
 #include <algorithm>
 #include <cmath>
 
