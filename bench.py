@@ -42,7 +42,7 @@ PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # Kernels per phase: a write batch of 2^20 or more goes through bins (count,
 # scan, scatter into bins, apply), a smaller one is one kernel; a read batch of
 # 2^25 or more from a slab of at most 48 bytes per read goes through bins too
-# (count, scan, scatter, apply, return).  An insertion of up to 1024 count
+# (decide, count, scatter, apply, return).  An insertion of up to 1024 count
 # tiles (32 rows each at T = 512) scans them in its count kernel.
 LAUNCHES_PER_STEP = {"clear": 1, "insert": 4, "read": 5, "write": 4, "rw_b": 1, "rw_g": 1, "flatten": 1}
 BINNED_WRITE_MIN = 1 << 20
@@ -384,7 +384,7 @@ def run_ours(args, world, rank, local):
     dom = max(single, key=lambda n: ph_ms[n])
     kernels = {"insert": "count_kernel + tile_scan_kernel + reserve_kernel + copy_bulk_kernel",
                "flatten": "flatten_kernel", "rw_b": "sweep_b_kernel", "rw_g": "sweep_g_kernel",
-               "read": ("rbin_count_kernel + wbin_scan_kernel + rbin_scatter_kernel + rbin_apply_kernel + "
+               "read": ("rbin_decide_kernel + rbin_count_kernel + rbin_scatter_kernel + rbin_apply_kernel + "
                         "rbin_return_kernel" if binned_read else "read_kernel"),
                "write": ("wbin_count_kernel + wbin_scan_kernel + wbin_scatter_kernel + wbin_apply_kernel"
                          if binned else "write_kernel")}
@@ -660,7 +660,7 @@ def run_e2e(args, g, counts, values, idx_r, idx_w, vals_w, out_r, dst, N, world,
 def time_generated(w, R, pool_bytes, dev, stream, per_round=False):
     """The generated insertion of the workload's rounds: gga_insert_generated
     (rounds batched in passes), or with per_round gga_push_generated (the
-    device API: one gga::block_push_back per round, Algorithm 1 as written)."""
+    device API: one gga::BlockPusher push per round, Algorithm 1 as written)."""
     from paper_2209_00103_gb300 import gga
     g = gga.GGArray(w.L, w.T, w.B, w.E, pool_bytes)
     spec = gga.make_gen_spec(w.spec.seed, w.spec.dist, w.spec.coeffs)
@@ -691,7 +691,7 @@ def time_generated(w, R, pool_bytes, dev, stream, per_round=False):
 
 def time_push_expand(spec, B, counts, pool_bytes, dev, stream):
     """Pushes of values read from device memory through the device API
-    (gga_push_expand: gga::block_push_rounds, 4 rounds per call): the same
+    (gga_push_expand: gga::RoundsPusher, 4 rounds per push): the same
     counts as the step's insertion, and one int32 input per (round, block,
     thread) that the thread appends `count` times.  Algorithmic bytes: the
     counts and inputs read (4 + E per thread and round) and E per element

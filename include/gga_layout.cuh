@@ -33,9 +33,9 @@ constexpr uint64_t kGrain = 256;             // bucket alignment / allocation gr
 // reused first.  Queues are touched with atomicAdd only: insertion kernels
 // (and kernels calling block_push_back) pop (ring_taken), clear kernels push
 // (ring_tail), never both in one kernel, and kernels using one pool are
-// ordered on the device (one stream, or events); a one-thread fix-up after
-// each insertion (gga_device_commit after a user kernel) folds the pops into
-// ring_head.  A class's queue has room for every bucket of that class the
+// ordered on the device (one stream, or events); the step that ends each
+// insertion (gga_device_commit after a user kernel) folds the pops into
+// ring_head, a class per thread.  A class's queue has room for every bucket of that class the
 // slab can hold (or, for a handle's private pool, that its LFVectors can
 // hold), so pushes never overrun it.
 struct PoolState {

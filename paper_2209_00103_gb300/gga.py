@@ -592,11 +592,11 @@ class GGArray:
         gga_device_commit(self.h, stream)
 
     def push_generated(self, spec, rounds, stream=None):
-        """insert_generated through the device API, one block_push_back per round."""
+        """insert_generated through the device API, one BlockPusher push per round."""
         gga_push_generated(self.h, spec, rounds, stream)
 
     def push_expand(self, counts, inputs, stream=None):
-        """Memory-sourced pushes through the device API (block_push_rounds)."""
+        """Memory-sourced pushes through the device API (a RoundsPusher per LFVector)."""
         gga_push_expand(self.h, counts, inputs, stream)
 
     def read(self, idx, out=None, stream=None):
