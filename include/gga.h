@@ -109,7 +109,8 @@ typedef struct {
  * queue per power-of-two bucket size; buckets handed back are reused first).
  *  pool_bytes       : slab size.
  *  slab_dev         : device slab of pool_bytes bytes, 256-byte aligned,
- *                     borrowed (must outlive the pool); NULL = allocate one.
+ *                     borrowed (must outlive the pool and every array in it);
+ *                     NULL = allocate one.
  *  min_bucket_bytes : smallest bucket (B * E) any array in the pool will
  *                     use; the queues take pool_bytes / min_bucket_bytes * 16
  *                     bytes of device memory at most.
@@ -349,7 +350,9 @@ int gga_offsets(gga_handle h, uint64_t* offsets_dev, void* stream);
  */
 int gga_clear(gga_handle h, void* stream);
 
-/* gga_memory -- memory accounting (host pointer out).  Synchronizes. */
+/* gga_memory -- memory accounting (host pointer out) of the array and its
+ * pool; the workspaces of calls (gga_insert's scratch, the bins of gga_write and
+ * gga_read) are not counted.  Synchronizes. */
 int gga_memory(gga_handle h, gga_mem* out, void* stream);
 
 /* gga_last_error -- synchronize, return the latched device error and clear it. */
